@@ -257,7 +257,7 @@ def spectrum_rho(M):
     decay over four orders of magnitude in every sector."""
     blocks = []
     for d in M.dim:
-        q, _ = torch.linalg.qr(M.gauss(d, d))
+        q = torch.linalg.qr(M.gauss(d, d).cpu())[0].cuda()      # small: the host does it as fast
         k = torch.arange(d, device="cuda", dtype=torch.float64)
         lam = d * torch.exp(-9.0 * (k + torch.rand(d, generator=M.gen, device="cuda", dtype=torch.float64)) / d)
         r = (q * lam) @ q.mH
