@@ -63,6 +63,13 @@ __global__ void __launch_bounds__(256) k_seg_weight(const SegNorm* __restrict__ 
     }
 }
 
+// The tiles of the first nfirst tasks, longest first, ahead of the others, longest first: each group's tiles
+// are one contiguous range, so that no tile of the first group's sectors is left to the other stream's launch.
+void first_tiles(TaskList& tl, int nfirst) {
+    const auto mid = std::stable_partition(tl.tiles.begin(), tl.tiles.end(), [=](const Tile& t) { return t.task < nfirst; });
+    tl.ntiles_first = (int)(mid - tl.tiles.begin());
+}
+
 }  // namespace
 
 int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx* const* psi, const double* w, cplx* rho,
@@ -181,7 +188,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
             tl->tasks.push_back(tk);
         }
         make_tiles(*tl, kTileF64, kTileF64, kSplitK);
-        for (const Tile& t : tl->tiles) tl->ntiles_first += t.task < nfirst ? 1 : 0;
+        first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
         if (rc) { release(c, *tl); return rc; }
         it = c->rho_plans.emplace(key, std::move(tl)).first;
@@ -214,7 +221,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
             tl->tasks.push_back(tk);
         }
         make_tiles(*tl, kTileF64, kTileF64, kSplitK);
-        for (const Tile& t : tl->tiles) tl->ntiles_first += t.task < nfirst ? 1 : 0;
+        first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
         if (rc) { release(c, *tl); return rc; }
         it = c->rho_plans.emplace(key, std::move(tl)).first;
