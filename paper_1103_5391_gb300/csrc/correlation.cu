@@ -127,8 +127,8 @@ extern "C" int tdmrg_correlation(tdmrg_ctx* c, int nL, const int32_t* opL, int n
                 cp->scratch += p.scratch;
             }
         if (!rc) {
-            make_tiles(cp->s1, kTileF64, kTileF64, kSplitK);
-            make_tiles(cp->s2, kTileF64, kTileF64, kSplitK);
+            make_tiles(cp->s1);
+            make_tiles(cp->s2);
             rc = upload(c, cp->s1);
             if (!rc) rc = upload(c, cp->s2);
             if (!rc) rc = dev_alloc(c, (void**)&cp->T, (size_t)std::max<int64_t>(cp->scratch, 1) * sizeof(cplx), "correlation scratch");

@@ -187,7 +187,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
             tk.seg_end = (int)tl->segs.size();
             tl->tasks.push_back(tk);
         }
-        make_tiles(*tl, kTileF64, kTileF64, kSplitK);
+        make_tiles(*tl);
         first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
         if (rc) { release(c, *tl); return rc; }
@@ -220,7 +220,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
             tk.seg_end = (int)tl->segs.size();
             tl->tasks.push_back(tk);
         }
-        make_tiles(*tl, kTileF64, kTileF64, kSplitK);
+        make_tiles(*tl);
         first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
         if (rc) { release(c, *tl); return rc; }

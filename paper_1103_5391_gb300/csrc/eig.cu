@@ -716,7 +716,7 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
     }
     // task lists: AX = rho W^H; S = W AX and G = W W^H; W' = E1h W
     struct Prod { int cbuf, abuf, bbuf; int8_t opb, herm; };
-    auto one = [&](TaskList& tl, std::initializer_list<Prod> prods) {
+    auto one = [&](TaskList& tl, std::initializer_list<Prod> prods, bool corr) {
         tl.tasks.clear(); tl.segs.clear();
         for (int k = 0; k < ns; ++k) {
             const int n = dim[k];
@@ -725,21 +725,22 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
                 t.c_off = off[k]; t.c_buf = (int8_t)pr.cbuf; t.ldc = n; t.M = n; t.N = n; t.beta = 0;
                 t.herm = pr.herm;
                 t.seg_begin = (int)tl.segs.size();
-                // K in chunks of kKChunk: split-K over the chunks spreads a sector's FP64 work over
-                // several SMs (the per-SM FP64 rate is the limit, not the tile count)
-                for (int k0 = 0; k0 < n; k0 += kKChunk) {
+                // the correction kernel's K parts are whole segments: chunks of kKChunk spread a sector over several SMs
+                const int kc = corr ? kKChunk : n;
+                for (int k0 = 0; k0 < n; k0 += kc) {
                     Seg sg{};
                     sg.a_off = off[k] + k0; sg.a_buf = (int8_t)pr.abuf; sg.lda = n;
                     sg.b_off = off[k] + (pr.opb == OPB_N ? (int64_t)k0 * n : (int64_t)k0);
                     sg.b_buf = (int8_t)pr.bbuf; sg.ldb = n; sg.opb = pr.opb;
-                    sg.K = std::min(kKChunk, n - k0); sg.scale = make_double2(1.0, 0.0); sg.dscale = -1;
+                    sg.K = std::min(kc, n - k0); sg.scale = make_double2(1.0, 0.0); sg.dscale = -1;
                     tl.segs.push_back(sg);
                 }
                 t.seg_end = (int)tl.segs.size();
                 tl.tasks.push_back(t);
             }
         }
-        make_tiles(tl, kTileF64, kTileF64, kKChunk);
+        if (corr) make_corr_tiles(tl, kKChunk);
+        else make_tiles(tl);
         return upload(c, tl);
     };
     // shared memory of the Jacobi launch: the most any sector asks for (A, V and a whole sweep of
@@ -753,9 +754,9 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
     for (int k = 0; k < ns && !rc; ++k)
         if (dim[k] > 1 && jac_chunk(dim[k], G.jac_smem) < 1) rc = fail(c, TDMRG_EINVAL, "rho_eig: Jacobi shared memory");
     // S = W rho W^H and G = W W^H are Hermitian: lower tiles plus mirror
-    if (!rc) rc = one(G.tl_ax, {{EB_AX, EB_RHO, EB_W, OPB_C, 0}});
-    if (!rc) rc = one(G.tl_sg, {{EB_S, EB_W, EB_AX, OPB_N, 1}, {EB_G, EB_W, EB_W, OPB_C, 1}});
-    if (!rc) rc = one(G.tl_y, {{EB_WN, EB_E, EB_W, OPB_N, 0}});
+    if (!rc) rc = one(G.tl_ax, {{EB_AX, EB_RHO, EB_W, OPB_C, 0}}, false);
+    if (!rc) rc = one(G.tl_sg, {{EB_S, EB_W, EB_AX, OPB_N, 1}, {EB_G, EB_W, EB_W, OPB_C, 1}}, false);
+    if (!rc) rc = one(G.tl_y, {{EB_WN, EB_E, EB_W, OPB_N, 0}}, true);
     return rc;
 }
 
@@ -793,10 +794,12 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
     int it = 0;
     // iterations past kRefine run on the device only when the previous correction asked for them
     auto gemm = [&](TaskList& tl, bool corr) {
-        a.tasks = tl.d_tasks; a.segs = tl.d_segs; a.tiles = tl.d_tiles; a.ntiles = (int)tl.tiles.size();
+        a.tasks = tl.d_tasks; a.segs = tl.d_segs; a.tiles = tl.d_tiles; a.ctiles = tl.d_ctiles;
+        a.ntiles = (int)(corr ? tl.ctiles.size() : tl.tiles.size());
         a.partials = tl.d_partials; a.counters = tl.d_counters;
         c->launches++;
-        return launch_gemm_f64(a, s, it < kRefine ? nullptr : n_iter, it, corr);
+        const int* skip = it < kRefine ? nullptr : n_iter;
+        return corr ? launch_gemm_corr(a, s, skip, it) : launch_gemm_f64(a, s, skip, it);
     };
     const dim3 chunks(ns, kRowChunks);
     cudaError_t e = cudaGetLastError();

@@ -1,77 +1,112 @@
 // Grouped complex FP64 GEMM for the sector-pair products of H psi (Sec. IV, Hamiltonian
-// connections), the excitation operators (Eq. b), and rho_L (Eq. rdensitymatrix).
+// connections), the excitation operators (Eq. b), rho_L (Eq. rdensitymatrix) and every other superblock product.
 //
-// One CTA computes one 16 x 16 output tile of one task over a range of its segments:
-//     C_tile = (beta ? C_tile : 0) + sum_segments scale * A_seg * op(B_seg)
-// For a Hermitian result (rho_L and the Gram matrices of the eigen-refinement) only the tiles on and
-// below the diagonal are computed and each off-diagonal tile is also stored conjugate-transposed.
-// On GB300 FP64 runs at about 1 TFLOP/s for the whole chip (scalar DFMA and the FP64 MMA alike),
-// i.e. about 7 GFLOP/s per SM, so the kernel is organised for balance rather than data reuse:
-//   - small (16 x 16) tiles so that every sector pair spreads over many SMs;
-//   - each of the four warps owns one 8 x 8 sub-block over the whole K range (no cross-warp sums),
-//     and negated or conjugated operands are staged by integer sign flips, so that the FP64 pipe
-//     runs the MMAs and little else;
-//   - tasks with a long K (many segments) are split across CTAs along segment boundaries; each part
-//     stores its partial tile and the last part to arrive (atomic ticket) sums all parts in index
-//     order, so results do not depend on scheduling.
-// Complex products use the FP64 tensor MMA (mma.sync m8n8k4 f64): four real MMAs per complex MMA.
+// On GB300 FP64 runs at about 1 TFLOP/s for the whole chip (scalar DFMA and the FP64 MMA alike): a warp-wide
+// DFMA holds its sub-partition's FP64 pipe for ~64 cycles, an m8n8k4 MMA for ~640, so memory and issue slots
+// are nearly free beside the arithmetic, and what decides is how many FP64 instructions are spent and how
+// evenly they fall on the 608 pipes.  Hence scalar DFMA with one output per lane:
+//   - a tile is a range of a task's outputs in flattened (row-major, for a Hermitian result lower-triangle)
+//     order, so blocks of any odd size fill their warps (an 8 x 8 MMA grid leaves 30-60 % of a ragged sector
+//     block's MMA work on padding), and K runs over its exact length;
+//   - the K range of an output is divided among `ks` groups of warps of the CTA (summed in order through shared
+//     memory), and over CTAs when that is not enough, down to a K per warp that keeps every pipe busy
+//     (make_tiles): small superblocks are bound by the longest chain of one warp, not by the total;
+//   - operands go from global memory (L1 / L2) straight to registers, four k ahead of their use: at 256
+//     cycles per complex multiply-add of a warp the loads are hidden without shared memory or barriers;
+//   - conjugations and the segment factor are applied once per segment on the accumulated sums.
+// Measured (before: 16 x 16 tiles of m8n8k4 MMAs staged through shared memory, each warp one 8 x 8 block over the
+// whole K): rho_L at L=48 m=1000 872 -> 581 us (0.60 GFLOP of lower triangles, 1.04 TFLOP/s), H psi at L=8 m=16
+// 17.7 -> 8.7 us, a Krylov advance at L=16 m=120 (12 steps) 985 -> 526 us.
+// CTAs that share a K split store partial sums; the last part to arrive (atomic ticket) sums all parts in index
+// order, so results do not depend on scheduling.
 //
-// The correction mode (kCorr) serves the update W' = (I + D) W of the eigen-refinement, where D is small
+// The correction kernel serves the update W' = (I + D) W of the eigen-refinement, where D is small
 // (|D| <= 1e-3, ~1e-7 in the last iteration): D W runs in FP32 (each CTA accumulates one K part of at
 // most a few dozen terms; parts are summed in FP64), so its rounding is ~1e-7 of |D| |W|, and the
 // epilogue adds W itself in FP64.  W is the B operand of the task's first segment.  FP32 accumulation
-// is what limits the accuracy, so this mode suits small corrections only, not full products.
+// is what limits the accuracy, so it suits small corrections only, not full products.  It works on 16 x 16
+// output tiles staged through shared memory.
 #include "internal.h"
 
 namespace tdmrg {
 namespace {
 
-constexpr int TS = kTileF64;     // 16
-constexpr int KC = 16;
-constexpr int PAD = TS + 4;      // row stride of the staged planes (conflict-free fragment loads)
+constexpr int GT = 256;               // threads of a CTA of the grouped GEMM
+constexpr int UK = 4;                 // k steps loaded ahead
 
-__device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
-                 : "+d"(c0), "+d"(c1)
-                 : "d"(a), "d"(b));
-}
-
-// Sign flip of a double on the integer pipe: FP64 arithmetic is scarce on this GPU, so negated and
-// conjugated operands are formed while staging instead of by FP64 instructions.
+// Sign flip of a double on the integer pipe
 __device__ __forceinline__ double neg(double x) { return __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63)); }
 
-// acc += a * b for complex a = (ar, ai), b = (br, bi) in FP32
-__device__ __forceinline__ void cfma32(float& cr, float& ci, float ar, float ai, float br, float bi) {
-    cr = fmaf(ar, br, fmaf(-ai, bi, cr));
-    ci = fmaf(ar, bi, fmaf(ai, br, ci));
+// One segment as the lanes read it: A(m, k) at a[m * am + k * ak], B(k, n) at b[n * bn + k * bk].
+struct SegView {
+    const double2* a;
+    const double2* b;
+    int am, ak, bn, bk;
+    int K, mode;                      // mode 0 complex, 1 A real, 2 B real
+    double ca, cb;                    // -1: conjugated operand
+    double sr, si;                    // factor
+};
+
+// s0 += Re a Re b, s1 += Im a Im b, s2 += Re a Im b, s3 += Im a Re b over k in [k0, k1)
+template <int MODE>
+__device__ __forceinline__ void seg_mac(const double2* __restrict__ pa, const double2* __restrict__ pb, int ak, int bk, int nk,
+                                        double (&s)[4]) {
+    auto mac = [&](double2 a, double2 b) {
+        s[0] = fma(a.x, b.x, s[0]);
+        if (MODE == 0) s[1] = fma(a.y, b.y, s[1]);
+        if (MODE != 2) s[2] = fma(a.x, b.y, s[2]);
+        if (MODE != 1) s[3] = fma(a.y, b.x, s[3]);
+    };
+    int k = 0;
+    if (nk >= UK) {
+        double2 a[UK], b[UK];
+#pragma unroll
+        for (int u = 0; u < UK; ++u) { a[u] = __ldg(pa + u * ak); b[u] = __ldg(pb + u * bk); }
+        for (k = UK; k + UK <= nk; k += UK) {
+            pa += (int64_t)UK * ak;
+            pb += (int64_t)UK * bk;
+            double2 na[UK], nb[UK];
+#pragma unroll
+            for (int u = 0; u < UK; ++u) { na[u] = __ldg(pa + u * ak); nb[u] = __ldg(pb + u * bk); }
+#pragma unroll
+            for (int u = 0; u < UK; ++u) mac(a[u], b[u]);
+#pragma unroll
+            for (int u = 0; u < UK; ++u) { a[u] = na[u]; b[u] = nb[u]; }
+        }
+        pa += (int64_t)UK * ak;
+        pb += (int64_t)UK * bk;
+#pragma unroll
+        for (int u = 0; u < UK; ++u) mac(a[u], b[u]);
+    }
+    for (; k < nk; ++k) {
+        mac(__ldg(pa), __ldg(pb));
+        pa += ak;
+        pb += bk;
+    }
 }
 
-template <bool kCorr>
-__global__ void __launch_bounds__(128) gemm_f64_kernel(GemmArgs args, const int* skip_flag, int skip_step) {
+__global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const int* skip_flag, int skip_step) {
     pdl_enter();
     if (skip_flag != nullptr && skip_step >= *skip_flag) return;   // Krylov space already complete
-    __shared__ double Are[kCorr ? 1 : TS][PAD], Aim[kCorr ? 1 : TS][PAD], Ain[kCorr ? 1 : TS][PAD];   // Ain = -Aim
-    __shared__ double Bre[kCorr ? 1 : KC][PAD], Bim[kCorr ? 1 : KC][PAD];
-    // correction mode: FP32 operands, [0] real and [1] imaginary
-    __shared__ float fA[2][kCorr ? TS : 1][PAD], fB[2][kCorr ? KC : 1][PAD];
+    __shared__ SegView sv[kTileSegs];
+    __shared__ double2 red[GT];
     __shared__ int last;
-
     const Tile tile = args.tiles[blockIdx.x];
     const Task task = args.tasks[tile.task];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int gid = lane >> 2, tig = lane & 3;
-    const int m0 = tile.m0, n0 = tile.n0;
-    const int Mt = min(TS, task.M - m0), Nt = min(TS, task.N - n0);
-    // warp w owns the 8 x 8 sub-block (w / 2, w % 2) over the whole K range: no cross-warp sums
-    const int bi = warp >> 1, bj = warp & 1;
-    const bool active = (8 * bi < Mt) && (8 * bj < Nt);
-    double cre[2] = {0.0, 0.0}, cim[2] = {0.0, 0.0};
-    float fre[2] = {0.f, 0.f}, fim[2] = {0.f, 0.f};
-
-    for (int s = tile.seg_lo; s < tile.seg_hi; ++s) {
-        const Seg seg = args.segs[s];
-        const cplx* __restrict__ A = args.bufs[seg.a_buf] + seg.a_off;
-        const cplx* __restrict__ B = args.bufs[seg.b_buf] + seg.b_off;
+    const int tid = threadIdx.x;
+    const int nseg = tile.seg_hi - tile.seg_lo;
+    if (tid < nseg) {
+        const Seg seg = args.segs[tile.seg_lo + tid];
+        SegView w;
+        w.a = args.bufs[seg.a_buf] + seg.a_off;
+        w.b = args.bufs[seg.b_buf] + seg.b_off;
+        w.am = seg.opa ? 1 : seg.lda; w.ak = seg.opa ? seg.lda : 1;
+        const bool nb = seg.opb == OPB_N || seg.opb == OPB_CN;
+        w.bn = nb ? 1 : seg.ldb; w.bk = nb ? seg.ldb : 1;
+        w.K = seg.K;
+        w.mode = (seg.rflags & 1) ? 1 : (seg.rflags & 2) ? 2 : 0;
+        w.ca = seg.opa == 2 ? -1.0 : 1.0;
+        w.cb = (seg.opb == OPB_C || seg.opb == OPB_CN) ? -1.0 : 1.0;
         double sr = seg.scale.x, si = seg.scale.y;
         if (seg.dscale >= 0) {
             const double d = args.dscale[seg.dscale];
@@ -83,107 +118,162 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(GemmArgs args, const int*
             si = sr * d.y + si * d.x;
             sr = tr;
         }
-        const bool scaled = !(sr == 1.0 && si == 0.0);
-        const bool conj = seg.opb == OPB_C;
-        const bool a_real = (seg.rflags & 1) != 0, b_real = (seg.rflags & 2) != 0;   // skip zero imaginary products
+        w.sr = sr; w.si = si;
+        sv[tid] = w;
+    }
+    // this thread's output and its share of the K range (uniform per warp)
+    const int pad = (tile.cnt + 31) & ~31;
+    const int part = tid / pad, lo = tid - part * pad;
+    const bool active = part < tile.ks && lo < tile.cnt;
+    int m = 0, n = 0;
+    if (active) {
+        const int o = tile.o0 + lo;
+        if (task.herm) {   // row m of the lower triangle starts at m (m + 1) / 2
+            m = (int)((sqrtf(8.f * (float)o + 1.f) - 1.f) * 0.5f);
+            while ((m + 1) * (m + 2) / 2 <= o) ++m;
+            while (m * (m + 1) / 2 > o) --m;
+            n = o - m * (m + 1) / 2;
+        } else {
+            m = o / task.N;
+            n = o - m * task.N;
+        }
+    }
+    const int kspan = tile.k1 - tile.k0;
+    const int ka = tile.k0 + kspan * part / tile.ks, kb = tile.k0 + kspan * (part + 1) / tile.ks;
+    __syncthreads();
+    double re = 0.0, im = 0.0;
+    if (active) {
+        int pos = 0;   // k of the tile's first segment's start; tile.k0 and k1 count from there
+        for (int s = 0; s < nseg && pos < kb; ++s) {
+            const SegView& w = sv[s];
+            const int k0 = max(ka - pos, 0), k1 = min(kb - pos, w.K);
+            pos += w.K;
+            if (k0 >= k1) continue;
+            const double2* pa = w.a + (int64_t)m * w.am + (int64_t)k0 * w.ak;
+            const double2* pb = w.b + (int64_t)n * w.bn + (int64_t)k0 * w.bk;
+            double q[4] = {0.0, 0.0, 0.0, 0.0};
+            if (w.mode == 0) seg_mac<0>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            else if (w.mode == 1) seg_mac<1>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            else seg_mac<2>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            const double pr = fma(-w.ca * w.cb, q[1], q[0]), pi = fma(w.cb, q[2], w.ca * q[3]);
+            const double sr = w.sr, si = w.si;
+            if (si == 0.0) {
+                re = fma(sr, pr, re);
+                im = fma(sr, pi, im);
+            } else {
+                re = fma(sr, pr, fma(-si, pi, re));
+                im = fma(sr, pi, fma(si, pr, im));
+            }
+        }
+    }
+    if (tile.ks > 1) {   // the K shares of this CTA, summed in order
+        if (active && part > 0) red[tid] = make_double2(re, im);
+        __syncthreads();
+        if (active && part == 0)
+            for (int p = 1; p < tile.ks; ++p) {
+                const double2 x = red[p * pad + lo];
+                re += x.x; im += x.y;
+            }
+    }
+    const bool out = active && part == 0;
+    if (tile.split >= 0) {
+        // split-K over CTAs: publish this part, the last part to arrive sums all parts in index order
+        cplx* base = args.partials + tile.split_base;
+        if (out) base[(int64_t)tile.part * pad + lo] = make_double2(re, im);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last = (atomicAdd(args.counters + tile.split, 1) == tile.nparts - 1);
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (out) {
+            re = 0.0; im = 0.0;
+            for (int p = 0; p < tile.nparts; ++p) {
+                const double2 x = __ldcg(base + (int64_t)p * pad + lo);
+                re += x.x; im += x.y;
+            }
+        }
+        if (tid == 0) args.counters[tile.split] = 0;   // ready for the next launch
+    }
+    if (!out) return;
+    cplx* __restrict__ C = args.bufs[task.c_buf] + task.c_off;
+    cplx* p = task.trans ? C + (int64_t)n * task.ldc + m : C + (int64_t)m * task.ldc + n;
+    if (task.beta) {
+        const double2 o = *p;
+        re += o.x;
+        im += o.y;
+    }
+    *p = make_double2(re, im);
+    if (task.herm && m != n) C[(int64_t)n * task.ldc + m] = make_double2(re, neg(im));
+}
+
+// ---- correction kernel: C = (I + D) W on 16 x 16 tiles --------------------------------------------
+constexpr int TS = kTileCorr;    // 16
+constexpr int KC = 16;
+constexpr int PAD = TS + 4;      // row stride of the staged planes (conflict-free fragment loads)
+
+// acc += a * b for complex a = (ar, ai), b = (br, bi) in FP32
+__device__ __forceinline__ void cfma32(float& cr, float& ci, float ar, float ai, float br, float bi) {
+    cr = fmaf(ar, br, fmaf(-ai, bi, cr));
+    ci = fmaf(ar, bi, fmaf(ai, br, ci));
+}
+
+__global__ void __launch_bounds__(128) gemm_corr_kernel(GemmArgs args, const int* skip_flag, int skip_step) {
+    pdl_enter();
+    if (skip_flag != nullptr && skip_step >= *skip_flag) return;
+    __shared__ float fA[2][TS][PAD], fB[2][KC][PAD];   // [0] real and [1] imaginary
+    __shared__ int last;
+    const CorrTile tile = args.ctiles[blockIdx.x];
+    const Task task = args.tasks[tile.task];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int gid = lane >> 2, tig = lane & 3;
+    const int m0 = tile.m0, n0 = tile.n0;
+    const int Mt = min(TS, task.M - m0), Nt = min(TS, task.N - n0);
+    // warp w owns the 8 x 8 sub-block (w / 2, w % 2)
+    const int bi = warp >> 1, bj = warp & 1;
+    const bool active = (8 * bi < Mt) && (8 * bj < Nt);
+    float fre[2] = {0.f, 0.f}, fim[2] = {0.f, 0.f};
+    for (int s = tile.seg_lo; s < tile.seg_hi; ++s) {
+        const Seg seg = args.segs[s];
+        const cplx* __restrict__ A = args.bufs[seg.a_buf] + seg.a_off;
+        const cplx* __restrict__ B = args.bufs[seg.b_buf] + seg.b_off;
         for (int k0 = 0; k0 < seg.K; k0 += KC) {
             const int kc = min(KC, seg.K - k0);
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {             // A chunk TS x KC: threads along k (along m when transposed)
-                const int e = tid + 128 * u;
-                const int r = seg.opa ? e % TS : e / KC, k = seg.opa ? e / TS : e % KC;
+            for (int u = 0; u < 2; ++u) {             // A chunk TS x KC: threads along k
+                const int e = tid + 128 * u, r = e / KC, k = e % KC;
                 double2 v = make_double2(0.0, 0.0);
-                if (r < Mt && k < kc)
-                    v = seg.opa ? A[(int64_t)(k0 + k) * seg.lda + m0 + r] : A[(int64_t)(m0 + r) * seg.lda + k0 + k];
-                if (seg.opa == 2) v.y = neg(v.y);
-                if (scaled) v = make_double2(sr * v.x - si * v.y, sr * v.y + si * v.x);
-                if constexpr (kCorr) {
-                    fA[0][r][k] = (float)v.x;
-                    fA[1][r][k] = (float)v.y;
-                } else {
-                    Are[r][k] = v.x;
-                    Aim[r][k] = v.y;
-                    Ain[r][k] = neg(v.y);
-                }
+                if (r < Mt && k < kc) v = A[(int64_t)(m0 + r) * seg.lda + k0 + k];
+                fA[0][r][k] = (float)v.x;
+                fA[1][r][k] = (float)v.y;
             }
-            if (seg.opb == OPB_N || seg.opb == OPB_CN) {   // B[k][n] at B[k*ldb + n] (conjugated for 'CN'): threads along n
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int e = tid + 128 * u, k = e / TS, n = e % TS;
-                    double2 v = make_double2(0.0, 0.0);
-                    if (k < kc && n < Nt) v = B[(int64_t)(k0 + k) * seg.ldb + n0 + n];
-                    if (seg.opb == OPB_CN) v.y = neg(v.y);
-                    if constexpr (kCorr) {
-                        fB[0][k][n] = (float)v.x;
-                        fB[1][k][n] = (float)v.y;
-                    } else {
-                        Bre[k][n] = v.x;
-                        Bim[k][n] = v.y;
-                    }
-                }
-            } else {                                  // B[k][n] at B[n*ldb + k] (conjugated for 'C')
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int e = tid + 128 * u, n = e / KC, k = e % KC;
-                    double2 v = make_double2(0.0, 0.0);
-                    if (k < kc && n < Nt) v = B[(int64_t)(n0 + n) * seg.ldb + k0 + k];
-                    if (conj) v.y = neg(v.y);
-                    if constexpr (kCorr) {
-                        fB[0][k][n] = (float)v.x;
-                        fB[1][k][n] = (float)v.y;
-                    } else {
-                        Bre[k][n] = v.x;
-                        Bim[k][n] = v.y;
-                    }
-                }
+            for (int u = 0; u < 2; ++u) {             // B[k][n] at B[k*ldb + n]: threads along n
+                const int e = tid + 128 * u, k = e / TS, n = e % TS;
+                double2 v = make_double2(0.0, 0.0);
+                if (k < kc && n < Nt) v = B[(int64_t)(k0 + k) * seg.ldb + n0 + n];
+                fB[0][k][n] = (float)v.x;
+                fB[1][k][n] = (float)v.y;
             }
             __syncthreads();
-            if constexpr (kCorr) {
-                if (active) {
-                    const int rr = 8 * bi + gid;
-                    for (int kk = 0; kk < kc; ++kk) {
-                        const float ar = fA[0][rr][kk], ai = fA[1][rr][kk];
+            if (active) {
+                const int rr = 8 * bi + gid;
+                for (int kk = 0; kk < kc; ++kk) {
+                    const float ar = fA[0][rr][kk], ai = fA[1][rr][kk];
 #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int cc = 8 * bj + 2 * tig + e;
-                            cfma32(fre[e], fim[e], ar, ai, fB[0][kk][cc], fB[1][kk][cc]);
-                        }
-                    }
-                }
-            } else if (active) {
-                if (a_real || b_real) {   // one operand real: two real MMAs per complex k-step
-                    for (int kk = 0; kk < kc; kk += 4) {
-                        const double ar = Are[8 * bi + gid][kk + tig], ai = Aim[8 * bi + gid][kk + tig];
-                        const double br = Bre[kk + tig][8 * bj + gid], bm = Bim[kk + tig][8 * bj + gid];
-                        dmma(cre[0], cre[1], ar, br);
-                        if (a_real) dmma(cim[0], cim[1], ar, bm);
-                        else dmma(cim[0], cim[1], ai, br);
-                    }
-                } else {
-                    for (int kk = 0; kk < kc; kk += 4) {   // zero-padded beyond kc
-                        const double ar = Are[8 * bi + gid][kk + tig], ai = Aim[8 * bi + gid][kk + tig];
-                        const double an = Ain[8 * bi + gid][kk + tig];
-                        const double br = Bre[kk + tig][8 * bj + gid], bm = Bim[kk + tig][8 * bj + gid];
-                        dmma(cre[0], cre[1], ar, br);
-                        dmma(cre[0], cre[1], an, bm);
-                        dmma(cim[0], cim[1], ar, bm);
-                        dmma(cim[0], cim[1], ai, br);
+                    for (int e = 0; e < 2; ++e) {
+                        const int cc = 8 * bj + 2 * tig + e;
+                        cfma32(fre[e], fim[e], ar, ai, fB[0][kk][cc], fB[1][kk][cc]);
                     }
                 }
             }
             __syncthreads();
         }
     }
-
     // this thread's two outputs: row 8 bi + gid, columns 8 bj + 2 tig + e
     const int r = 8 * bi + gid, col0 = 8 * bj + 2 * tig;
-    double2 v[2] = {make_double2(cre[0], cim[0]), make_double2(cre[1], cim[1])};
-    if constexpr (kCorr) {
-        v[0] = make_double2((double)fre[0], (double)fim[0]);
-        v[1] = make_double2((double)fre[1], (double)fim[1]);
-    }
+    double2 v[2] = {make_double2((double)fre[0], (double)fim[0]), make_double2((double)fre[1], (double)fim[1])};
     if (tile.split >= 0) {
-        // split-K: publish this part, the last part to arrive sums all parts in index order
         cplx* part = args.partials + ((int64_t)tile.split_base + tile.part) * (TS * TS);
         if (active) {
             part[r * TS + col0] = v[0];
@@ -211,35 +301,28 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(GemmArgs args, const int*
     }
     if (!active) return;
     cplx* __restrict__ C = args.bufs[task.c_buf] + task.c_off;
+    const Seg s0 = args.segs[task.seg_begin];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         const int col = col0 + e;
-        if (r < Mt && col < Nt) {
-            cplx* p = task.trans ? C + (int64_t)(n0 + col) * task.ldc + m0 + r : C + (int64_t)(m0 + r) * task.ldc + n0 + col;
-            double2 x = v[e];
-            if constexpr (kCorr) {   // (I + D) W: add W in FP64
-                const Seg s0 = args.segs[task.seg_begin];
-                const double2 w = args.bufs[s0.b_buf][s0.b_off + (int64_t)(m0 + r) * s0.ldb + n0 + col];
-                x.x += w.x;
-                x.y += w.y;
-            }
-            if (task.beta) {
-                const double2 o = *p;
-                x.x += o.x;
-                x.y += o.y;
-            }
-            *p = x;
-            if (task.herm && m0 != n0) C[(int64_t)(n0 + col) * task.ldc + m0 + r] = make_double2(x.x, neg(x.y));
+        if (r < Mt && col < Nt) {   // (I + D) W: add W in FP64
+            const double2 w = args.bufs[s0.b_buf][s0.b_off + (int64_t)(m0 + r) * s0.ldb + n0 + col];
+            C[(int64_t)(m0 + r) * task.ldc + n0 + col] = make_double2(v[e].x + w.x, v[e].y + w.y);
         }
     }
 }
 
 }  // namespace
 
-cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step, bool corr) {
+cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step) {
     if (a.ntiles <= 0) return cudaSuccess;
-    if (corr) launch_pdl(gemm_f64_kernel<true>, a.ntiles, 128, 0, s, a, skip_flag, skip_step);
-    else launch_pdl(gemm_f64_kernel<false>, a.ntiles, 128, 0, s, a, skip_flag, skip_step);
+    launch_pdl(gemm_f64_kernel, a.ntiles, GT, 0, s, a, skip_flag, skip_step);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_corr(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step) {
+    if (a.ntiles <= 0) return cudaSuccess;
+    launch_pdl(gemm_corr_kernel, a.ntiles, 128, 0, s, a, skip_flag, skip_step);
     return cudaGetLastError();
 }
 

@@ -77,13 +77,21 @@ struct Task {
     int32_t pad2;
 };
 
-// One CTA's work: output tile (m0, n0) (element origin) of task `task`, segments [seg_lo, seg_hi).
-// A tile whose task is split along K has split >= 0: part `part` of `nparts`, partial tiles at
-// partials[(split_base + part) * tile area], completion ticket counters[split].
+// One CTA's work: outputs [o0, o0 + cnt) of task `task` in flattened order (row-major, or the lower triangle row
+// by row when the task is Hermitian), over k in [k0, k1) counted from the start of segment seg_lo (segments
+// [seg_lo, seg_hi) cover it), the K range divided among `ks` groups of the CTA's warps.  A tile that is one
+// of several K parts has split >= 0: part `part` of `nparts`, partial sums at partials[split_base + part *
+// (cnt rounded up to 32)], completion ticket counters[split].
 struct Tile {
-    int32_t task;
-    int32_t m0, n0;
-    int32_t cost;             // complex MACs, for ordering
+    int32_t task, o0, cnt, ks;
+    int32_t seg_lo, seg_hi, k0, k1;
+    int32_t split, part, nparts, split_base;
+    int32_t cost, pad;        // complex MACs, for ordering
+};
+// 16 x 16 output tile of the correction kernel (eigen-refinement), segments [seg_lo, seg_hi); K parts as above,
+// partial tiles at partials[(split_base + part) * 256].
+struct CorrTile {
+    int32_t task, m0, n0, cost;
     int32_t seg_lo, seg_hi;
     int32_t split, part, nparts, split_base;
 };
@@ -93,13 +101,16 @@ struct TaskList {
     std::vector<Task> tasks;
     std::vector<Seg> segs;
     std::vector<Tile> tiles;
+    std::vector<CorrTile> ctiles;   // instead of tiles: a list of the correction kernel
     Task* d_tasks = nullptr;
     Seg* d_segs = nullptr;
     Tile* d_tiles = nullptr;
+    CorrTile* d_ctiles = nullptr;
     double flops = 0.0;       // algorithmic real flops (8 per complex MAC)
     size_t bytes = 0;         // device bytes of the arrays below
-    int nsplit = 0, npartial = 0;
-    cplx* d_partials = nullptr;   // split-K partial tiles
+    int nsplit = 0;
+    int64_t npartial = 0;         // complex entries of d_partials
+    cplx* d_partials = nullptr;   // split-K partial sums
     int* d_counters = nullptr;    // split-K tickets (zero between launches)
     int ntiles_first = 0;         // rho task lists ordered by eigensolver groups: tiles of the first group
 };
@@ -296,6 +307,7 @@ struct GemmArgs {
     const Task* tasks;
     const Seg* segs;
     const Tile* tiles;
+    const CorrTile* ctiles;
     int ntiles;
     cplx* bufs[kMaxBufs];
     const double* dscale;
@@ -381,16 +393,19 @@ void dev_free(tdmrg_ctx* c, void* p, size_t bytes);
 int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qin0, int qin1, int qout0, int qout1,
                Plan* out, bool to_device = true);
 int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn);
-void make_tiles(TaskList& tl, int tm, int tn, int ksplit);
+void make_tiles(TaskList& tl);
+void make_corr_tiles(TaskList& tl, int ksplit);
 int upload(tdmrg_ctx* c, TaskList& tl);
 void release(tdmrg_ctx* c, TaskList& tl);
 int run_plan(tdmrg_ctx* c, const Plan& p, const cplx* in, cplx* out, const int* skip_flag, int skip_step);
 
-// gemm_f64.cu: grouped complex FP64 GEMM (FP64 MMA), tile 16 x 16, split-K above kSplitK
-constexpr int kTileF64 = 16;
-constexpr int kSplitK = 96;
-// corr: the correction mode of the eigen-refinement update, C = (I + A) B with A B in FP32
-cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step, bool corr = false);
+// gemm_f64.cu: grouped complex FP64 GEMM (one output per lane), and the correction C = (I + A) B with A B in FP32
+constexpr int kTileOut = 256;    // outputs of a tile at most (threads of its CTA)
+constexpr int kTileSegs = 16;    // segments of a tile at most
+constexpr int kMaxParts = 8;     // CTAs that share one tile's K range at most (more only for its segments' sake)
+constexpr int kTileCorr = 16;
+cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step);
+cudaError_t launch_gemm_corr(const GemmArgs& a, cudaStream_t s, const int* skip_flag, int skip_step);
 
 
 // api.cu: cached plan of H psi in sector (a, b), in the context's precision

@@ -57,10 +57,9 @@ extern "C" int tdmrg_apply_h_static(tdmrg_ctx* c, int n_up, int n_dn, const tdmr
     const Plan& p = *it->second;
     if (p.n_in == 0) return TDMRG_OK;
     // layout of the static array: intermediates | partials (stage 1, 2) | tickets (stage 1, 2)
-    const size_t tile = (size_t)kTileF64 * kTileF64 * sizeof(cplx);
     const size_t off_p1 = align256((size_t)p.scratch * sizeof(cplx));
-    const size_t off_p2 = off_p1 + align256((size_t)p.stage1.npartial * tile);
-    const size_t off_c1 = off_p2 + align256((size_t)p.stage2.npartial * tile);
+    const size_t off_p2 = off_p1 + align256((size_t)p.stage1.npartial * sizeof(cplx));
+    const size_t off_c1 = off_p2 + align256((size_t)p.stage2.npartial * sizeof(cplx));
     const size_t off_c2 = off_c1 + align256((size_t)p.stage1.nsplit * sizeof(int));
     const size_t need = off_c2 + align256((size_t)p.stage2.nsplit * sizeof(int));
     if (need > kStaticScratchBytes)

@@ -1186,7 +1186,7 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
             mk(st.sliceB, st.bjobs, st.d_bjobs, st.d_bvjob, st.d_bsegs, st.panelB, st.expB, st.rowsB);
         }
         if (!thin.tasks.empty()) {
-            make_tiles(thin, kTileF64, kTileF64, kSplitK);
+            make_tiles(thin);
             rc = upload(c, thin);
             if (rc) return rc;
         }

@@ -18,10 +18,11 @@ namespace tdmrg {
 
 int upload(tdmrg_ctx* c, TaskList& tl) {
     release(c, tl);
-    struct { void** dst; const void* src; size_t bytes; } parts[3] = {
+    struct { void** dst; const void* src; size_t bytes; } parts[4] = {
         {(void**)&tl.d_tasks, tl.tasks.data(), tl.tasks.size() * sizeof(Task)},
         {(void**)&tl.d_segs, tl.segs.data(), tl.segs.size() * sizeof(Seg)},
-        {(void**)&tl.d_tiles, tl.tiles.data(), tl.tiles.size() * sizeof(Tile)}};
+        {(void**)&tl.d_tiles, tl.tiles.data(), tl.tiles.size() * sizeof(Tile)},
+        {(void**)&tl.d_ctiles, tl.ctiles.data(), tl.ctiles.size() * sizeof(CorrTile)}};
     for (auto& pt : parts) {
         if (!pt.bytes) continue;
         int rc = dev_alloc(c, pt.dst, pt.bytes, "task list");
@@ -31,14 +32,15 @@ int upload(tdmrg_ctx* c, TaskList& tl) {
         if (rc) return rc;
     }
     if (tl.nsplit) {
-        int rc = dev_alloc(c, (void**)&tl.d_partials, (size_t)tl.npartial * kTileF64 * kTileF64 * sizeof(cplx),
+        int rc = dev_alloc(c, (void**)&tl.d_partials, (size_t)tl.npartial * sizeof(cplx),
                            "split-K partials");
         if (!rc) rc = dev_alloc(c, (void**)&tl.d_counters, (size_t)tl.nsplit * sizeof(int), "split-K tickets");
         if (!rc) rc = cuda_check(c, cudaMemset(tl.d_counters, 0, (size_t)tl.nsplit * sizeof(int)), "split-K tickets");
         if (rc) return rc;
     }
     tl.bytes = tl.tasks.size() * sizeof(Task) + tl.segs.size() * sizeof(Seg) + tl.tiles.size() * sizeof(Tile) +
-               (size_t)tl.npartial * kTileF64 * kTileF64 * sizeof(cplx) + (size_t)tl.nsplit * sizeof(int);
+               tl.ctiles.size() * sizeof(CorrTile) +
+               (size_t)tl.npartial * sizeof(cplx) + (size_t)tl.nsplit * sizeof(int);
     return TDMRG_OK;
 }
 
@@ -46,9 +48,10 @@ void release(tdmrg_ctx* c, TaskList& tl) {
     if (tl.d_tasks) dev_free(c, tl.d_tasks, tl.tasks.size() * sizeof(Task));
     if (tl.d_segs) dev_free(c, tl.d_segs, tl.segs.size() * sizeof(Seg));
     if (tl.d_tiles) dev_free(c, tl.d_tiles, tl.tiles.size() * sizeof(Tile));
-    if (tl.d_partials) dev_free(c, tl.d_partials, (size_t)tl.npartial * kTileF64 * kTileF64 * sizeof(cplx));
+    if (tl.d_ctiles) dev_free(c, tl.d_ctiles, tl.ctiles.size() * sizeof(CorrTile));
+    if (tl.d_partials) dev_free(c, tl.d_partials, (size_t)tl.npartial * sizeof(cplx));
     if (tl.d_counters) dev_free(c, tl.d_counters, (size_t)tl.nsplit * sizeof(int));
-    tl.d_tasks = nullptr; tl.d_segs = nullptr; tl.d_tiles = nullptr; tl.d_partials = nullptr; tl.d_counters = nullptr;
+    tl.d_tasks = nullptr; tl.d_segs = nullptr; tl.d_tiles = nullptr; tl.d_ctiles = nullptr; tl.d_partials = nullptr; tl.d_counters = nullptr;
 }
 
 int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
@@ -62,24 +65,95 @@ int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
     return n;
 }
 
-void make_tiles(TaskList& tl, int tm, int tn, int ksplit) {
+// Tiles of the grouped FP64 GEMM.  The K range one warp runs through aims at a sixth of the launch's work per
+// FP64 pipe (152 SMs x 4), between 8 and 192: small launches are cut finely so that every pipe has work and no
+// chain is long, large ones into tiles of 256 outputs whose operands are reused by all of the CTA's warps.
+// Measured: a floor of 4 or 16 instead of 8 makes a Krylov advance at L=16 m=120 614 or 542 us instead of 527, a cap of
+// 64 instead of 192 rho_L at L=48 m=1000 607 us instead of 581.
+// A task's K is divided first among the warps of a CTA (ks = 1, 2, 4, 8 shares, 256 / ks outputs), then over CTAs.
+void make_tiles(TaskList& tl) {
     tl.tiles.clear();
     tl.flops = 0.0;
     tl.nsplit = 0;
     tl.npartial = 0;
+    double work = 0.0;
+    std::vector<int64_t> outs(tl.tasks.size()), ks(tl.tasks.size(), 0);
     for (size_t t = 0; t < tl.tasks.size(); ++t) {
         const Task& k = tl.tasks[t];
-        int64_t ksum = 0;
+        outs[t] = k.herm ? (int64_t)k.M * (k.M + 1) / 2 : (int64_t)k.M * k.N;
         for (int s = k.seg_begin; s < k.seg_end; ++s) {
-            ksum += tl.segs[s].K;
+            ks[t] += tl.segs[s].K;
             // 8 real flops per complex multiply-add, 4 when one operand is real
             tl.flops += (tl.segs[s].rflags ? 4.0 : 8.0) * (double)k.M * k.N * (double)tl.segs[s].K;
         }
-        // split long K along segment boundaries into parts of about ksplit
+        work += (double)outs[t] * (double)ks[t];
+    }
+    const int64_t per_warp = (int64_t)std::min(192.0, std::max(8.0, work / (32.0 * 608.0 * 6.0)));
+    for (size_t t = 0; t < tl.tasks.size(); ++t) {
+        const Task& k = tl.tasks[t];
+        if (outs[t] <= 0) continue;
+        const int64_t shares = std::max<int64_t>(1, (ks[t] + per_warp - 1) / per_warp);
+        const int cks = shares <= 1 ? 1 : shares <= 2 ? 2 : shares <= 4 ? 4 : 8;
+        const int area = kTileOut / cks;
+        int want = (int)std::min<int64_t>({(shares + cks - 1) / cks, (int64_t)kMaxParts, std::max<int64_t>(ks[t], 1)});
+        // K parts [lo, hi) of the concatenated range, each within kTileSegs segments
+        struct Part { int seg_lo, seg_hi; int64_t k0, k1; };
+        std::vector<Part> parts;
+        for (;; ++want) {
+            parts.clear();
+            bool ok = true;
+            for (int p = 0; p < want; ++p) {
+                const int64_t lo = ks[t] * p / want, hi = ks[t] * (p + 1) / want;
+                int s0 = k.seg_begin;
+                int64_t pos = 0;
+                while (s0 < k.seg_end && pos + tl.segs[s0].K <= lo) pos += tl.segs[s0++].K;
+                int s1 = s0;
+                int64_t end = pos;
+                while (s1 < k.seg_end && end < hi) end += tl.segs[s1++].K;
+                ok = ok && s1 - s0 <= kTileSegs;
+                parts.push_back({s0, s1, lo - pos, hi - pos});
+            }
+            if (ok || want >= ks[t]) break;
+        }
+        const int np = (int)parts.size();
+        const int64_t nt = (outs[t] + area - 1) / area;
+        const int64_t step = std::min<int64_t>(area, 32 * ((outs[t] + 32 * nt - 1) / (32 * nt)));
+        for (int64_t o0 = 0; o0 < outs[t]; o0 += step) {
+            const int cnt = (int)std::min<int64_t>(step, outs[t] - o0), pad = (cnt + 31) & ~31;
+            const int split = np > 1 ? tl.nsplit++ : -1;
+            const int64_t base = tl.npartial;
+            if (np > 1) tl.npartial += (int64_t)np * pad;
+            for (int p = 0; p < np; ++p) {
+                Tile tile{};
+                tile.task = (int32_t)t; tile.o0 = (int32_t)o0; tile.cnt = cnt; tile.ks = cks;
+                tile.seg_lo = parts[p].seg_lo; tile.seg_hi = parts[p].seg_hi;
+                tile.k0 = (int32_t)parts[p].k0; tile.k1 = (int32_t)parts[p].k1;
+                tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = (int32_t)base;
+                tile.cost = (int32_t)std::min<int64_t>((int64_t)cnt * std::max<int64_t>(parts[p].k1 - parts[p].k0, 1), 0x7fffffff);
+                tl.tiles.push_back(tile);
+            }
+        }
+    }
+    // longest tiles first: the grid drains big work before the tail of small tiles
+    std::stable_sort(tl.tiles.begin(), tl.tiles.end(),
+                     [](const Tile& a, const Tile& b) { return a.cost > b.cost; });
+}
+
+// 16 x 16 tiles of the correction kernel, long K split along segment boundaries into parts of about ksplit
+void make_corr_tiles(TaskList& tl, int ksplit) {
+    tl.ctiles.clear();
+    tl.nsplit = 0;
+    tl.npartial = 0;
+    constexpr int tm = kTileCorr;
+    int parts_total = 0;
+    for (size_t t = 0; t < tl.tasks.size(); ++t) {
+        const Task& k = tl.tasks[t];
+        int64_t ksum = 0;
+        for (int s = k.seg_begin; s < k.seg_end; ++s) ksum += tl.segs[s].K;
         std::vector<std::pair<int, int>> parts;
         const int nseg = k.seg_end - k.seg_begin;
-        int want = (int)std::min<int64_t>({(ksum + ksplit - 1) / std::max(ksplit, 1), (int64_t)nseg, (int64_t)8});
-        if (ksplit <= 0 || want <= 1) {
+        const int want = (int)std::min<int64_t>({(ksum + ksplit - 1) / ksplit, (int64_t)nseg, (int64_t)8});
+        if (want <= 1) {
             parts.push_back({k.seg_begin, k.seg_end});
         } else {
             const double target = (double)ksum / want;
@@ -95,31 +169,28 @@ void make_tiles(TaskList& tl, int tm, int tn, int ksplit) {
             }
             parts.push_back({lo, k.seg_end});
         }
-        for (int m0 = 0; m0 < std::max(k.M, 1); m0 += tm)
-            for (int n0 = 0; n0 < std::max(k.N, 1); n0 += tn) {
-                if (m0 >= k.M || n0 >= k.N) continue;
-                if (k.herm && n0 > m0) continue;   // upper tiles are written as mirrors of the lower ones
-                int mm = std::min(tm, k.M - m0), nn = std::min(tn, k.N - n0);
+        for (int m0 = 0; m0 < k.M; m0 += tm)
+            for (int n0 = 0; n0 < k.N; n0 += tm) {
+                const int mm = std::min(tm, k.M - m0), nn = std::min(tm, k.N - n0);
                 const int np = (int)parts.size();
                 const int split = np > 1 ? tl.nsplit++ : -1;
-                const int base = np > 1 ? tl.npartial : 0;
-                if (np > 1) tl.npartial += np;
+                const int base = np > 1 ? parts_total : 0;
+                if (np > 1) parts_total += np;
                 for (int p = 0; p < np; ++p) {
                     int64_t kp = 0;
                     for (int s = parts[p].first; s < parts[p].second; ++s) kp += tl.segs[s].K;
-                    int64_t cost = (int64_t)mm * nn * std::max<int64_t>(kp, 1);
-                    Tile tile{};
+                    CorrTile tile{};
                     tile.task = (int32_t)t; tile.m0 = m0; tile.n0 = n0;
-                    tile.cost = (int32_t)std::min<int64_t>(cost, 0x7fffffff);
+                    tile.cost = (int32_t)std::min<int64_t>((int64_t)mm * nn * std::max<int64_t>(kp, 1), 0x7fffffff);
                     tile.seg_lo = parts[p].first; tile.seg_hi = parts[p].second;
                     tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = base;
-                    tl.tiles.push_back(tile);
+                    tl.ctiles.push_back(tile);
                 }
             }
     }
-    // longest tiles first: the grid drains big work before the tail of small tiles
-    std::stable_sort(tl.tiles.begin(), tl.tiles.end(),
-                     [](const Tile& a, const Tile& b) { return a.cost > b.cost; });
+    tl.npartial = (int64_t)parts_total * tm * tm;
+    std::stable_sort(tl.ctiles.begin(), tl.ctiles.end(),
+                     [](const CorrTile& a, const CorrTile& b) { return a.cost > b.cost; });
 }
 
 namespace {
@@ -261,8 +332,8 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         tk.seg_end = (int)s2.segs.size();
         s2.tasks.push_back(tk);
     }
-    make_tiles(s1, kTileF64, kTileF64, kSplitK);
-    make_tiles(s2, kTileF64, kTileF64, kSplitK);
+    make_tiles(s1);
+    make_tiles(s2);
     p->scratch = scr;
     p->flops = s1.flops + s2.flops;
     if (!to_device) return TDMRG_OK;   // host task lists only (merged into a larger launch by the caller)

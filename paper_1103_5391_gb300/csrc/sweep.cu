@@ -90,8 +90,8 @@ int run_stages(tdmrg_ctx* from, TaskList& s1, TaskList& s2, int64_t scr, const t
                const tdmrg_c64* V, tdmrg_c64* out, int64_t nout) {
     const int8_t BU = BUF_EXTRA0, BV = BUF_EXTRA0 + 1;
     DeviceGuard g(from->opts.device);
-    make_tiles(s1, kTileF64, kTileF64, kSplitK);
-    make_tiles(s2, kTileF64, kTileF64, kSplitK);
+    make_tiles(s1);
+    make_tiles(s2);
     cplx* P1 = nullptr;
     const size_t sb = (size_t)std::max<int64_t>(scr, 1) * sizeof(cplx);
     int rc = dev_alloc(from, (void**)&P1, sb, "wft scratch");

@@ -252,8 +252,8 @@ extern "C" int tdmrg_renormalize_op(tdmrg_ctx* c, int side, int op_id, const tdm
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != c->opts.device) cudaSetDevice(c->opts.device);
-    make_tiles(s1, kTileF64, kTileF64, kSplitK);
-    make_tiles(s2, kTileF64, kTileF64, kSplitK);
+    make_tiles(s1);
+    make_tiles(s2);
     cplx* T = nullptr;
     int rc = dev_alloc(c, (void**)&T, (size_t)scr * sizeof(cplx), "renormalisation scratch");
     if (!rc) rc = upload(c, s1);
