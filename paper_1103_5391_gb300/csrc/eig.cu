@@ -2,22 +2,22 @@
 //
 // GB300 runs FP64 at about 1 TFLOP/s chip-wide (~7 GFLOP/s per SM), so an FP64 Jacobi on one SM per
 // sector would take milliseconds for the largest sectors.  Instead:
-//   1. seed: a cyclic two-sided Jacobi in FP32 per sector (one CTA per sector, parallel round-robin
-//      ordering of disjoint rotations), giving eigenvectors X0 accurate to about 1e-6;
+//   1. seed: a one-sided Jacobi in FP32 on the Cholesky factor of each sector (one CTA per sector, parallel
+//      round-robin ordering of disjoint rotations), giving eigenvectors X0 accurate to about 1e-6;
 //   2. refine: iterative refinement for Hermitian eigenproblems (Ogita & Aishima, 2018), whose work is
 //      grouped GEMMs spread over every SM (FP64, except the small correction E^H W in FP32):
 //         G = X^H X,  S = X^H (rho X),  lambda_i = Re S_ii / Re G_ii,  R = I - G,
 //         E_ij = (S_ij + lambda_j R_ij) / (lambda_j - lambda_i)   if |lambda_i - lambda_j| > delta,
 //         E_ij = R_ij / 2 otherwise (and on the diagonal),  delta = 2 (||S - diag(lambda)|| + ||rho|| ||R||),
 //         X <- X (I + E);
-//      convergence is quadratic: from the FP32 seed (error ~1e-5) two iterations reach rounding level;
+//      convergence is quadratic: from the FP32 seed two iterations reach rounding level;
 //      up to four more run (decided on the device, launched regardless) while the last correction is
 //      above 1e-7, as for near-degenerate pairs that the first iteration treats as a cluster.  If the
 //      sixth is still above it (density matrices of DMRG blocks whose spectra span the whole FP64 range in
 //      large degenerate multiplets), two last steps only orthonormalise W (E = R / 2 for every pair, a
 //      Newton-Schulz step: orthogonality error eps -> ~eps^2 -> rounding), so that the kept states always
 //      form an orthonormal basis and the renormalised operators are projections.  At
-//      iterations 1 and 3 a sector whose clustered pairs stay coupled is re-seeded instead (FP32 Jacobi
+//      iteration 1 a sector whose clustered pairs stay coupled is re-seeded instead (FP32 two-sided Jacobi
 //      on S with a relative criterion, k_jacobi32).  The iterate is kept as W = X^H, so every product
 //      is a plain or conjugate-transposed GEMM operand;
 //   3. sort each sector's eigenpairs by descending eigenvalue.
@@ -45,8 +45,11 @@ constexpr int kOaIters = 6;      // more, each only when the previous correction
 constexpr int kMaxRefine = 8;    // then, if the last one was still not small, two steps that only orthonormalise W
 constexpr float kReseedTol = 1e-7f;    // re-seed rotates (p, q) while |S_pq| > kReseedTol sqrt|S_pp S_qq| ...
 constexpr float kReseedFloor = 1e-14f; // ... and |S_pq| > kReseedFloor ||rho||_F
-// Refinement iterations that may re-seed a sector instead of updating it.
-__host__ __device__ constexpr bool reseed_iter(int it) { return it == 1 || it == 3; }
+// The refinement iteration that may re-seed a sector instead of updating it (a second one, at iteration 3, left the
+// FP32 rounding of its V to too few iterations: simulated over multiplets and random graded spectra, the worst
+// reconstruction 1e-9 ||rho|| with it, 9e-11 without).
+__host__ __device__ constexpr bool reseed_iter(int it) { return it == 1; }
+constexpr double kNearGap = 1e-11, kNearNum = 2e-15;   // in units of ||rho||_F, see k_oa_update
 constexpr double kTolE = 1e-7;   // |E| above this: the next error (~|E|^2) may exceed ~1e-14
 
 struct EigTables {
@@ -160,16 +163,16 @@ __device__ __forceinline__ void jacobi_apply_v(float2* V, int n, int rs, int cs,
 // group replays the record of the previous chunk of rounds on V meanwhile; record buffers swap at a
 // barrier of all threads every `C` rounds.
 //
-// Criterion: (p, q) is rotated while |A_pq|^2 > lim, lim = thr^2 for the seed, and for the re-seed
-// (`rel`) lim = max(kReseedTol^2 |A_pp A_qq|, floor^2), relative to the pair's own diagonal.
-__device__ __forceinline__ float jac_lim(bool rel, float thr2, float a, float d) {
-    return rel ? fmaxf(kReseedTol * kReseedTol * fabsf(a * d), thr2) : thr2;
+// Criterion: (p, q) is rotated while |A_pq|^2 > max(kReseedTol^2 |A_pp A_qq|, floor^2), relative to the pair's
+// own diagonal.
+__device__ __forceinline__ float jac_lim(float thr2, float a, float d) {
+    return fmaxf(kReseedTol * kReseedTol * fabsf(a * d), thr2);
 }
 //
 // Record mode (grec != nullptr, used when V does not fit in shared memory): every thread rotates A
 // (ja = JT), each rotation is also written to the global record grec (round-major, npair per round) and
 // *nrec receives the number of rounds; V is formed afterwards from the record by k_jacobi_replay.
-__device__ __forceinline__ int jacobi_sweeps(float2* A, float2* V, int n, int ld, int vrs, int vcs, float thr, bool rel,
+__device__ __forceinline__ void jacobi_sweeps(float2* A, float2* V, int n, int ld, int vrs, int vcs, float thr,
                                              float4* rec, int C, int ja, float4* __restrict__ grec, int* nrec) {
     const int tid = threadIdx.x;
     const bool agroup = tid < ja;
@@ -179,8 +182,7 @@ __device__ __forceinline__ int jacobi_sweeps(float2* A, float2* V, int n, int ld
     const int warp = tid >> 5, lane = tid & 31;
     int pend = 0, pend_r0 = 0, buf = 0;
     bool done = n <= 1;
-    int sweep = 0;
-    for (; sweep < 12 && !done; ++sweep) {
+    for (int sweep = 0; sweep < kMaxSweeps && !done; ++sweep) {
         for (int r0 = 0; r0 < R; r0 += C) {
             const int nr = min(C, R - r0);
             const bool last = r0 + nr >= R;
@@ -198,7 +200,7 @@ __device__ __forceinline__ int jacobi_sweeps(float2* A, float2* V, int n, int ld
                         if (q < n) {
                             const float2 b = A[p * ld + q];
                             const float ap = A[p * ld + p].x, aq = A[q * ld + q].x;
-                            if (fmaf(b.x, b.x, b.y * b.y) <= jac_lim(rel, thr2, ap, aq)) {
+                            if (fmaf(b.x, b.x, b.y * b.y) <= jac_lim(thr2, ap, aq)) {
                                 A[p * ld + q] = make_float2(0.f, 0.f);
                                 A[q * ld + p] = make_float2(0.f, 0.f);
                             } else {
@@ -255,7 +257,7 @@ __device__ __forceinline__ int jacobi_sweeps(float2* A, float2* V, int n, int ld
                         const int r = e / n, cc = e % n;
                         if (r > cc) {
                             const float2 b = A[r * ld + cc];
-                            above |= fmaf(b.x, b.x, b.y * b.y) > jac_lim(rel, thr2, A[r * ld + r].x, A[cc * ld + cc].x);
+                            above |= fmaf(b.x, b.x, b.y * b.y) > jac_lim(thr2, A[r * ld + r].x, A[cc * ld + cc].x);
                         }
                     }
                 }
@@ -271,7 +273,6 @@ __device__ __forceinline__ int jacobi_sweeps(float2* A, float2* V, int n, int ld
     if (!agroup && pend) jacobi_apply_v(V, n, vrs, vcs, rec + (size_t)(buf ^ 1) * C * npair, pend, pend_r0);
     if (grec != nullptr && tid == 0) *nrec = total;
     __syncthreads();
-    return sweep;
 }
 
 __device__ __forceinline__ void jacobi_load(const cplx* R, double scale, float2* A, float2* V, int n, int ld) {
@@ -283,100 +284,64 @@ __device__ __forceinline__ void jacobi_load(const cplx* R, double scale, float2*
     }
 }
 
-__device__ __forceinline__ float jacobi_fro2(const float2* A, int n, int ld) {
-    float f = 0.f;
-    for (int e = threadIdx.x; e < n * n; e += JT) { const float2 a = A[(e / n) * ld + e % n]; f += a.x * a.x + a.y * a.y; }
-    return f;
-}
-
-// W = V^H - dsub I: row j is the conjugate of eigenvector j (dsub = 1 stores the re-seed as a correction);
-// element (k, j) of V at V[k * rs + j * cs]
-__device__ __forceinline__ void jacobi_store(const float2* V, cplx* Ws, int n, int rs, int cs, double dsub) {
+// V^H - I: row j is the conjugate of eigenvector j, minus the unit vector (V row-major in shared memory)
+__device__ __forceinline__ void jacobi_store(const float2* V, cplx* Ws, int n, int ld) {
     for (int e = threadIdx.x; e < n * n; e += JT) {
         const int j = e / n, k = e % n;
-        const float2 v = V[k * rs + j * cs];
-        Ws[e] = make_double2((double)v.x - (k == j ? dsub : 0.0), -v.y);
+        const float2 v = V[k * ld + j];
+        Ws[e] = make_double2((double)v.x - (k == j ? 1.0 : 0.0), -v.y);
     }
 }
 
-// FP32 Jacobi per sector.  Dynamic shared memory (`smem` bytes): A and V of sectors with n <= kSmemMaxN
-// (A alone for n <= kSmemMaxA, V then in `gwork`, transposed), then the rotation record; larger sectors
-// keep A and V in `gwork`.
-//  - seed (rel = false): src = rho; writes W0 = X0^H (X0: unsorted eigenvector columns), ||rho||_F, the
-//    initial iteration count, and clears the sector's re-seed flag;
-//  - re-seed (rel = true) in refinement iteration `it`, for sectors whose flag is set: src = S = X^H rho X
-//    scaled by 1 / ||rho||_F, so that eigenvalues far below FP32's resolution of rho are resolved relative
-//    to their own size; writes V^H - I (V: eigenvectors of S) over the correction dst = E1h, so that the
-//    iteration's update is W <- V^H W, and asks for two more refinements.
+// Re-seed of refinement iteration `it`: an FP32 two-sided Jacobi per flagged sector on S = X^H rho X scaled by
+// 1 / ||rho||_F, so that eigenvalues far below FP32's resolution of rho are resolved relative to their own size;
+// writes V^H - I (V: eigenvectors of S) over the correction dst = E1h, so that the iteration's update is
+// W <- V^H W, and asks for two more refinements.  Dynamic shared memory (`smem` bytes): A and V of sectors with
+// n <= kSmemMaxN (A alone for n <= kSmemMaxA, V then formed by k_jacobi_replay), then the rotation record; larger
+// sectors keep A in `gwork`.
 __global__ void __launch_bounds__(JT) k_jacobi32(const cplx* __restrict__ src, cplx* __restrict__ dst,
-                                                 double* __restrict__ rho_fro, int* __restrict__ n_iter,
+                                                 const double* __restrict__ rho_fro, int* __restrict__ n_iter,
                                                  int* __restrict__ flags, EigTables tb, float2* __restrict__ gwork,
-                                                 float4* __restrict__ grec, int* __restrict__ nrec,
-                                                 int smem, bool rel, int it, int2* __restrict__ stats) {
+                                                 float4* __restrict__ grec, int* __restrict__ nrec, int smem, int it) {
     pdl_enter();
-    const long long t_start = clock64();
     extern __shared__ float4 fsm4[];
     float2* fsm = reinterpret_cast<float2*>(fsm4);
     const int sct = blockIdx.x, n = tb.dims[sct], tid = threadIdx.x;
     const int mode = jac_mode(n);
-    if (rel && (it >= *n_iter || flags[sct] == 0)) {   // iteration skipped, or nothing to re-seed
+    if (it >= *n_iter || flags[sct] == 0) {   // iteration skipped, or nothing to re-seed
         if (jac_recorded(n) && tid == 0) nrec[sct] = -1;   // nor is there anything to replay
         return;
     }
     const int64_t off = tb.off[sct];
     const int ld = n | 1;   // odd row stride: column accesses of a warp hit distinct banks
     float2* gA = gwork + 4 * off;
-    float2* gV = gA + (int64_t)n * ld;   // transposed: element (k, p) at gV[p * ld + k]
-    (void)gV;
     float4* rec = fsm4 + jac_base_bytes(n) / 16;
     const int C = jac_chunk(n, smem);
-    __shared__ float red[JT / 32];
-    __shared__ float thr_s;
-    const double scale = rel ? 1.0 / rho_fro[sct] : 1.0;
-    if (!rel && sct == 0 && tid == 0) *n_iter = kRefine;
-    float fro;
+    const double scale = 1.0 / rho_fro[sct];
     // V starts as the identity (record modes form V afterwards, in k_jacobi_replay)
-    if (mode == JAC_SMEM) { jacobi_load(src + off, scale, fsm, fsm + n * ld, n, ld); __syncthreads(); fro = jacobi_fro2(fsm, n, ld); }
-    else if (mode == JAC_SMEM_A) { jacobi_load(src + off, scale, fsm, nullptr, n, ld); __syncthreads(); fro = jacobi_fro2(fsm, n, ld); }
-    else { jacobi_load(src + off, scale, gA, nullptr, n, ld); __syncthreads(); fro = jacobi_fro2(gA, n, ld); }
-    for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
-    if ((tid & 31) == 0) red[tid >> 5] = fro;
+    jacobi_load(src + off, scale, mode == JAC_GLOBAL ? gA : fsm, mode == JAC_SMEM ? fsm + n * ld : nullptr, n, ld);
     __syncthreads();
     if (tid == 0) {
-        float f = 0.f;
-        for (int k = 0; k < JT / 32; ++k) f += red[k];
-        if (rel) {
-            thr_s = kReseedFloor;          // S is in units of ||rho||_F
-            flags[sct] = 0;
-            atomicMax(n_iter, min(kOaIters, it + 3));
-        } else {
-            thr_s = 4.8e-7f * sqrtf(f);    // 4 eps_fp32 ||A||_F: above FP32 rounding noise, so sweeps terminate
-            rho_fro[sct] = sqrtf(f);       // ||rho||_F for the refinement's cluster threshold
-            flags[sct] = 0;
-        }
+        flags[sct] = 0;
+        atomicMax(n_iter, min(kOaIters, it + 3));
     }
-    __syncthreads();
-    const float thr = thr_s;
-    int sweeps;
+    constexpr float thr = kReseedFloor;   // S is in units of ||rho||_F
     if (mode == JAC_SMEM) {
-        sweeps = jacobi_sweeps(fsm, fsm + n * ld, n, ld, ld, 1, thr, rel, rec, C, JA, nullptr, nullptr);
-        jacobi_store(fsm + n * ld, dst + off, n, ld, 1, rel ? 1.0 : 0.0);
+        jacobi_sweeps(fsm, fsm + n * ld, n, ld, ld, 1, thr, rec, C, JA, nullptr, nullptr);
+        jacobi_store(fsm + n * ld, dst + off, n, ld);
     } else if (mode == JAC_SMEM_A) {   // dst is written by k_jacobi_replay
-        sweeps = jacobi_sweeps(fsm, nullptr, n, ld, 1, ld, thr, rel, rec, C, JT, grec + tb.roff[sct], nrec + sct);
+        jacobi_sweeps(fsm, nullptr, n, ld, 1, ld, thr, rec, C, JT, grec + tb.roff[sct], nrec + sct);
     } else {
-        sweeps = jacobi_sweeps(gA, nullptr, n, ld, 1, ld, thr, rel, rec, C, JT, grec + tb.roff[sct], nrec + sct);
+        jacobi_sweeps(gA, nullptr, n, ld, 1, ld, thr, rec, C, JT, grec + tb.roff[sct], nrec + sct);
     }
-    // per sector of the last launch: sweeps and SM cycles (a measurement aid; tdmrg_eig_stats)
-    if (tid == 0 && !rel) stats[sct] = make_int2(sweeps, (int)min(clock64() - t_start, (long long)INT_MAX));
 }
 
 // V of the sectors beyond kSmemMaxN from their rotation record: V starts as the identity and every
 // recorded rotation J_r acts on columns (p, q) of every row, so rows are independent: CTA (b, y) holds
 // rows 8y .. 8y + 7 of V of big sector b in shared memory and replays all rounds on them, the record
-// staged through shared memory a batch of rounds at a time.  Writes W = V^H - dsub I like jacobi_store
-// (dsub = 1 for a re-seed).  Runs after each k_jacobi32 launch; nrec < 0 marks a skipped sector.
+// staged through shared memory a batch of rounds at a time.  Writes V^H - I like jacobi_store.  Runs after each k_jacobi32 launch; nrec < 0 marks a skipped sector.
 __global__ void __launch_bounds__(kReplayThreads) k_jacobi_replay(const float4* __restrict__ grec, const int* __restrict__ nrec,
-                                                                  cplx* __restrict__ dst, EigTables tb, int batch, bool rel) {
+                                                                  cplx* __restrict__ dst, EigTables tb, int batch) {
     pdl_enter();
     const int sct = tb.big[blockIdx.x], n = tb.dims[sct];
     const int nr = nrec[sct];
@@ -412,13 +377,273 @@ __global__ void __launch_bounds__(kReplayThreads) k_jacobi_replay(const float4* 
         }
     }
     __syncthreads();
-    const double dsub = rel ? 1.0 : 0.0;
     cplx* W = dst + tb.off[sct];
-    for (int e = tid; e < rows * n; e += blockDim.x) {   // W[j][k0 + k] = conj(V[k0 + k][j]) - dsub delta
+    for (int e = tid; e < rows * n; e += blockDim.x) {   // W[j][k0 + k] = conj(V[k0 + k][j]) - delta
         const int k = e % rows, j = e / rows;
         const float2 v = vs[k * ld + j];
-        W[(int64_t)j * n + k0 + k] = make_double2((double)v.x - (j == k0 + k ? dsub : 0.0), -v.y);
+        W[(int64_t)j * n + k0 + k] = make_double2((double)v.x - (j == k0 + k ? 1.0 : 0.0), -v.y);
     }
+}
+
+// ---- seed: one-sided Jacobi on a Cholesky factor ---------------------------------------------------
+// rho + delta ||rho|| I = L L^H (FP32, no pivoting), then plane rotations from the right make the columns of L
+// orthogonal (Hestenes' one-sided Jacobi on a Cholesky factor, Veselic and Hari 1989): L V = X Sigma, and the
+// normalised columns X are the eigenvectors of rho (the shift only keeps the factorisation positive).  Against a
+// two-sided Jacobi on rho with accumulated V:
+//   - a rotation touches two columns only and no second matrix, and the warp that owns a pair reads the columns,
+//     forms their three inner products, makes the rotation and applies it from registers: one barrier per round
+//     and no rotation table between warps;
+//   - the factor's columns are already nearly graded, and the criterion |<x, y>| <= tol |x| |y| resolves small
+//     eigenvalues relative to delta ||rho|| rather than to eps ||rho||: fewer sweeps, seeds an order of magnitude
+//     closer (simulated over decaying, Wishart, rank-deficient and multiplet spectra, n = 20 ... 152: one or two
+//     refinement iterations fewer).
+// Measured, the whole decomposition against the two-sided seed with V by rotation replay: L=32 m=400 1041 -> 568 us,
+// L=48 m=1000 8.93 -> 4.95 ms; the seed of n = 60 517 -> ~250 us, n = 152 5.1 -> 3.8 ms.  Bound by the latency of a
+// pair's chain (load, 5 shuffle levels, rotation, store: ~1000 cycles a round) up to n = 64, by shared-memory
+// traffic of 16 n^2 bytes a round beyond.
+// Columns are rows of T (T[c][r] = L[r][c], contiguous in r), lanes run over r.  One CTA per sector; T in shared
+// memory up to n = kSeedSmemN, else in `gwork`.
+constexpr int kSeedSmemN = 168;            // 8 n^2 bytes <= kJacSmemCap
+constexpr float kSeedShift = 1e-4f;        // delta, above the factorisation's rounding (~n 2^-24)
+constexpr float kSeedTol2 = 1e-12f;        // a pair is rotated while |<x, y>|^2 > kSeedTol2 |x|^2 |y|^2 ...
+constexpr float kSeedStop2 = 2.5e-7f;      // ... and sweeps end after one whose largest ratio was below this (convergence
+                                           // is quadratic: that sweep leaves ~1e-6)
+constexpr int kSeedSweeps = 15;
+
+// v 2^-e rounded to FP32, by integer instructions (conversions from double run on the narrow FP64 pipe);
+// values below 2^-126 give 0
+__device__ __forceinline__ float f32_of(double v, int e) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+    const int ex = (int)((hi >> 20) & 0x7FFu) - 896 - e;
+    if (ex <= 0) return 0.f;
+    return __uint_as_float((hi & 0x80000000u) | ((((unsigned)ex << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u)));
+}
+// the double equal to v (subnormals give 0), by integer instructions
+__device__ __forceinline__ double f64_of(float v) {
+    const unsigned u = __float_as_uint(v), ex = (u >> 23) & 0xFFu;
+    if (ex == 0u) return 0.0;
+    const unsigned hi = (u & 0x80000000u) | ((ex + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// Warp sums of g, a and b, in every lane: reduce-scatter to one value per 8 lanes, then broadcasts
+__device__ __forceinline__ void warp_sum4(float2& g, float& a, float& b) {
+    const int lane = threadIdx.x & 31;
+    const bool u16 = lane & 16, u8 = lane & 8;
+    float k0 = u16 ? a : g.x, k1 = u16 ? b : g.y;
+    k0 += __shfl_xor_sync(0xffffffffu, u16 ? g.x : a, 16);
+    k1 += __shfl_xor_sync(0xffffffffu, u16 ? g.y : b, 16);
+    float k = u8 ? k1 : k0;
+    k += __shfl_xor_sync(0xffffffffu, u8 ? k0 : k1, 8);
+    k += __shfl_xor_sync(0xffffffffu, k, 4);
+    k += __shfl_xor_sync(0xffffffffu, k, 2);
+    k += __shfl_xor_sync(0xffffffffu, k, 1);
+    g.x = __shfl_sync(0xffffffffu, k, 0);
+    g.y = __shfl_sync(0xffffffffu, k, 8);
+    a = __shfl_sync(0xffffffffu, k, 16);
+    b = __shfl_sync(0xffffffffu, k, 24);
+}
+
+// Orthogonalises columns x and y; returns whether their ratio was above the stopping limit.  E > 0: the columns
+// have at most 32 E entries and stay in registers; E = 0: any length, read twice.
+template <int E>
+__device__ __forceinline__ bool seed_pair(float2* x, float2* y, int n) {
+    const int lane = threadIdx.x & 31;
+    float2 g = make_float2(0.f, 0.f);
+    float a = 0.f, b = 0.f;
+    float2 xv[E > 0 ? E : 1], yv[E > 0 ? E : 1];
+    auto dots = [&](float2 u, float2 v) {
+        g.x = fmaf(u.x, v.x, fmaf(u.y, v.y, g.x));   // conj(x) y
+        g.y = fmaf(u.x, v.y, fmaf(-u.y, v.x, g.y));
+        a = fmaf(u.x, u.x, fmaf(u.y, u.y, a));
+        b = fmaf(v.x, v.x, fmaf(v.y, v.y, b));
+    };
+    if constexpr (E > 0) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int r = lane + 32 * e;
+            const bool in = e + 1 < E || r < n;
+            xv[e] = in ? x[r] : make_float2(0.f, 0.f);
+            yv[e] = in ? y[r] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) dots(xv[e], yv[e]);
+    } else {
+        for (int r = lane; r < n; r += 32) dots(x[r], y[r]);
+    }
+    warp_sum4(g, a, b);
+    const float g2 = fmaf(g.x, g.x, g.y * g.y), ab = a * b;
+    if (g2 <= kSeedTol2 * ab) return false;
+    float c;
+    float2 s;
+    rotation32(a, b, g, c, s);
+    const float2 sc = conjf2(s);
+    if constexpr (E > 0) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int r = lane + 32 * e;
+            if (e + 1 < E || r < n) {
+                x[r] = rot_l(c, sc, xv[e], yv[e]);
+                y[r] = rot_r(c, s, xv[e], yv[e]);
+            }
+        }
+    } else {
+        for (int r = lane; r < n; r += 32) {
+            const float2 u = x[r], v = y[r];
+            x[r] = rot_l(c, sc, u, v);
+            y[r] = rot_r(c, s, u, v);
+        }
+    }
+    return g2 > kSeedStop2 * ab;
+}
+
+template <int E>
+__device__ __forceinline__ int seed_sweeps(float2* T, int n) {
+    const int P = n + (n & 1), npair = P / 2, R = P - 1, warp = threadIdx.x >> 5;
+    int sweep = 0;
+    for (bool more = n > 1; more && sweep < kSeedSweeps; ++sweep) {
+        bool big = false;
+        for (int round = 0; round < R; ++round) {
+            for (int i = warp; i < npair; i += JT / 32) {
+                int p, q;
+                rr_pair(round, i, P, p, q);
+                if (q < n) big |= seed_pair<E>(T + p * n, T + q * n, n);
+            }
+            if (round + 1 < R) __syncthreads();
+        }
+        more = __syncthreads_or(big);
+    }
+    return sweep;
+}
+
+// T[c][r] = A[r][c] 2^-e for r >= c (0 above) plus `shift` on the diagonal
+__device__ __forceinline__ void seed_load(const cplx* __restrict__ R, float2* T, int n, int e, float shift) {
+    for (int x = threadIdx.x; x < n * n; x += JT) {
+        const int c = x / n, r = x - c * n;
+        float2 v = make_float2(0.f, 0.f);
+        if (r >= c) {
+            const double2 a = R[x];   // A[c][r] = conj(A[r][c])
+            v = r == c ? make_float2(f32_of(a.x, e) + shift, 0.f) : make_float2(f32_of(a.x, e), -f32_of(a.y, e));
+        }
+        T[x] = v;
+    }
+}
+
+// Right-looking Cholesky of the lower triangle held in T, columns left unscaled; false when a pivot falls below lim
+__device__ __forceinline__ bool seed_cholesky(float2* T, int n, float lim) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int k = 0; k < n; ++k) {
+        __syncthreads();
+        const float d = T[k * n + k].x;
+        if (!(d > lim)) return false;   // the same value in every thread
+        const float inv = 1.f / d;
+        for (int j = k + 1 + warp; j < n; j += JT / 32) {
+            const float2 f = T[k * n + j];
+            const float2 fc = make_float2(f.x * inv, -f.y * inv);
+            for (int i = j + lane; i < n; i += 32) {
+                const float2 t = cmf(T[k * n + i], fc);
+                float2* p = T + j * n + i;
+                *p = make_float2(p->x - t.x, p->y - t.y);
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = warp; k < n; k += JT / 32) {   // columns of L
+        const float sc = rsqrtf(T[k * n + k].x);
+        __syncwarp();
+        for (int i = k + lane; i < n; i += 32) { T[k * n + i].x *= sc; T[k * n + i].y *= sc; }
+    }
+    __syncthreads();
+    return true;
+}
+
+// The seed of one sector with T in shared memory (SM, inlined so that its accesses compile as such) or global
+// memory; e: the sector's exponent.  Returns the number of sweeps.
+template <bool SM>
+__device__ __forceinline__ int seed_sector(const cplx* __restrict__ R, cplx* __restrict__ W, double* rho_fro, float2* T, int n, int e) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ float redf[JT / 32];
+    seed_load(R, T, n, e, 0.f);
+    __syncthreads();
+    float f = 0.f;
+    for (int x = tid; x < n * n; x += JT) {   // entries off the diagonal count twice
+        const float2 v = T[x];
+        f += (x / n == x % n ? 1.f : 2.f) * fmaf(v.x, v.x, v.y * v.y);
+    }
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    if (lane == 0) redf[warp] = f;
+    __syncthreads();
+    f = redf[lane];
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    const float nf = sqrtf(f);
+    if (tid == 0) *rho_fro = ldexp((double)nf, e);   // the refinement's cluster threshold
+    int sweeps = 0;
+    if (nf > 0.f) {
+        // the first shift serves every positive semidefinite block; a matrix with eigenvalues below -delta
+        // ||rho|| (no density matrix) is shifted by more than its norm
+        float shift = kSeedShift * nf;
+        __syncthreads();
+        for (int x = tid; x < n; x += JT) T[x * n + x].x += shift;
+        if (!seed_cholesky(T, n, 0.5f * shift)) {
+            __syncthreads();
+            seed_load(R, T, n, e, 1.05f * nf);
+            seed_cholesky(T, n, 0.f);
+        }
+        switch (SM ? (n + 31) / 32 : 0) {
+            case 1: sweeps = seed_sweeps<1>(T, n); break;
+            case 2: sweeps = seed_sweeps<2>(T, n); break;
+            case 3: sweeps = seed_sweeps<3>(T, n); break;
+            case 4: sweeps = seed_sweeps<4>(T, n); break;
+            case 5: sweeps = seed_sweeps<5>(T, n); break;
+            case 6: sweeps = seed_sweeps<6>(T, n); break;
+            default: sweeps = seed_sweeps<0>(T, n);
+        }
+    }
+    for (int c = warp; c < n; c += JT / 32) {   // W row c = (column c)^H / |column c|
+        float q = 0.f;
+        for (int r = lane; r < n; r += 32) { const float2 v = T[c * n + r]; q = fmaf(v.x, v.x, fmaf(v.y, v.y, q)); }
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        const float inv = q > 0.f ? 1.f / sqrtf(q) : 0.f;
+        for (int r = lane; r < n; r += 32) {
+            const float2 v = T[c * n + r];
+            const float2 u = nf > 0.f ? make_float2(v.x * inv, -v.y * inv) : make_float2(r == c ? 1.f : 0.f, 0.f);
+            W[(int64_t)c * n + r] = make_double2(f64_of(u.x), f64_of(u.y));
+        }
+    }
+    return sweeps;
+}
+
+// W0 = X0^H of every sector (rows unsorted), ||rho||_F, the initial iteration count, cleared re-seed flags.
+__global__ void __launch_bounds__(JT) k_seed(const cplx* __restrict__ rho, cplx* __restrict__ W, double* __restrict__ rho_fro,
+                                             int* __restrict__ n_iter, int* __restrict__ flags, EigTables tb,
+                                             float2* __restrict__ gwork, int2* __restrict__ stats) {
+    pdl_enter();
+    const long long t_start = clock64();
+    extern __shared__ float4 fsm4[];
+    const int sct = blockIdx.x, n = tb.dims[sct], tid = threadIdx.x;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int64_t off = tb.off[sct];
+    const cplx* __restrict__ R = rho + off;
+    __shared__ int rede[JT / 32];
+    int ex = 0;   // largest biased exponent: the sector is scaled by a power of two so that no square underflows
+    for (int x = tid; x < n * n; x += JT) {
+        const double2 v = R[x];
+        ex = max(ex, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
+    }
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    if (lane == 0) rede[warp] = ex;
+    __syncthreads();
+    ex = __reduce_max_sync(0xffffffffu, rede[lane]);
+    const int e = ex - 1023;
+    if (tid == 0) {
+        flags[sct] = 0;
+        if (sct == 0) *n_iter = kRefine;
+    }
+    const int sweeps = n <= kSeedSmemN ? seed_sector<true>(R, W + off, rho_fro + sct, reinterpret_cast<float2*>(fsm4), n, e)
+                                       : seed_sector<false>(R, W + off, rho_fro + sct, gwork + 4 * off, n, e);
+    // sweeps and SM cycles of the sector's seed (a measurement aid; tdmrg_eig_stats)
+    if (tid == 0) stats[sct] = make_int2(sweeps, (int)min(clock64() - t_start, (long long)INT_MAX));
 }
 
 // Refinement on W = X^H, which turns every product into a plain or conjugate-transposed operand of the
@@ -521,7 +746,7 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
     const int4 item = oa.items[blockIdx.x];
     const int sct = item.x, n = tb.dims[sct];
     const int64_t off = tb.off[sct], eo = tb.eoff[sct];
-    const double delta = oa.delta[sct], floor_s = (double)kReseedFloor * rho_fro[sct];
+    const double delta = oa.delta[sct], fro = rho_fro[sct], floor_s = (double)kReseedFloor * fro;
     double2 sv[kOaPer], g[kOaPer];
 #pragma unroll
     for (int u = 0; u < kOaPer; ++u) {
@@ -537,10 +762,14 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
             const int i = e / n, j = e - i * n;
             const double2 r = make_double2((i == j ? 1.0 : 0.0) - g[u].x, -g[u].y);
             double2 ev;
-            const double li = lam[eo + i], lj = lam[eo + j];
-            if (!orth_only && i != j && fabs(li - lj) > delta) {
+            const double li = lam[eo + i], lj = lam[eo + j], gap = fabs(li - lj);
+            const double2 num = make_double2(sv[u].x + li * r.x, sv[u].y + li * r.y);
+            // a close pair whose numerator is rounding (an exact multiplet in an iterate that has converged while
+            // other sectors go on) would be turned by noise / noise: a cluster as well
+            const bool near = gap <= delta || (gap <= kNearGap * fro && fmax(fabs(num.x), fabs(num.y)) <= kNearNum * fro);
+            if (!orth_only && i != j && !near) {
                 const double inv = 1.0 / (li - lj);
-                ev = make_double2((sv[u].x + li * r.x) * inv, (sv[u].y + li * r.y) * inv);
+                ev = make_double2(num.x * inv, num.y * inv);
             } else {
                 ev = make_double2(0.5 * r.x, 0.5 * r.y);
                 // clustered pair still coupled: the cluster is not diagonalised by this update
@@ -616,16 +845,14 @@ size_t oa_bytes(int noa, int ns) {
 // Buffer ids of the refinement GEMMs (all packed like rho).
 enum { EB_RHO = BUF_EXTRA0, EB_W, EB_AX, EB_S, EB_G, EB_E, EB_WN };
 
-// Cost model of the split into two groups, in SM cycles: the Jacobi seed of one sector (about 7 sweeps of
-// n - 1 rounds; a round costs ~1300 + 12 n cycles with A and V in shared memory, ~40 n beyond) and the
-// refinement of a sector spread over the GPU (3 iterations of 2 m^3 complex FP64 MACs at ~140 FMA per
-// cycle chip-wide, m = n rounded up to the 16 x 16 x 16 tiles of the grouped GEMM).  Fitted to graph-replay
-// timings of the split sizes on the L=32 m=400 and L=48 m=1000 blocks; it only decides the scheduling.
-double jacobi_cost(int n) { return 7.0 * std::max(n - 1, 0) * (n <= kSmemMaxN ? 1300.0 + 12.0 * n : 40.0 * n); }
-double refine_cost(int n) {
-    const double m = 16.0 * ((n + 15) / 16);
-    return 0.35 * m * m * m;
-}
+// Cost model of the split into two groups, in SM cycles: the seed of one sector (about 7.5 sweeps of n - 1 rounds; a
+// round costs ~700 + 14 n cycles while a pair per warp is enough, ~300 + 32 n beyond) and the refinement of a
+// sector spread over the GPU, 0.4 n^3 (the products alone are ~0.1 n^3; measured over 0.03 ... 1.5: the decomposition at
+// L=48 m=1000 takes 5.7 ms up to 0.12 and 4.95 ms from 0.2 on, L=32 m=400 and m=800 change by 4 %).
+// Measured seeds, cycles per round: n = 21 990, 42 1360, 54 1480, 68 2540, 98 3360, 124 3830, 152 5330.  It only decides
+// the scheduling.
+double jacobi_cost(int n) { return 7.5 * std::max(n - 1, 0) * (n <= 64 ? 700.0 + 14.0 * n : 300.0 + 32.0 * n); }
+double refine_cost(int n) { return 0.4 * (double)n * n * n; }
 
 // Sectors of the first group (run on the second stream): the k with the longest Jacobi seeds, k chosen to
 // minimise max(J_1 + R(first k), J_{k+1} + R(rest)) (J_i the i-th longest seed); empty when one group is
@@ -751,6 +978,8 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
         smem = std::max(smem, jac_base_bytes(n) + 32 * (P / 2) * (P - 1));
     }
     G.jac_smem = std::min(smem, kJacSmemCap);
+    for (int k = 0; k < ns; ++k)
+        if (dim[k] <= kSeedSmemN) G.seed_smem = std::max(G.seed_smem, 8 * dim[k] * dim[k]);
     for (int k = 0; k < ns && !rc; ++k)
         if (dim[k] > 1 && jac_chunk(dim[k], G.jac_smem) < 1) rc = fail(c, TDMRG_EINVAL, "rho_eig: Jacobi shared memory");
     // S = W rho W^H and G = W W^H are Hermitian: lower tiles plus mirror
@@ -766,11 +995,11 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
     const int64_t* t64 = (const int64_t*)G.tables;
     const int* dims = (const int*)(t64 + 3 * ns);
     EigTables tb{t64, t64 + ns, t64 + 2 * ns, dims, dims + ns};
-    // V of the record-mode sectors after each Jacobi launch (seed or re-seed)
-    auto replay = [&](cplx* dst, bool rel) {
+    // V of the record-mode sectors after each re-seed launch
+    auto replay = [&](cplx* dst) {
         if (!G.nbig) return;
         const dim3 grid(G.nbig, (G.maxn_big + kReplayRows - 1) / kReplayRows);
-        launch_pdl(k_jacobi_replay, grid, kReplayThreads, G.replay_smem, s, G.grec, G.nrec, dst, tb, G.replay_batch, rel);
+        launch_pdl(k_jacobi_replay, grid, kReplayThreads, G.replay_smem, s, G.grec, G.nrec, dst, tb, G.replay_batch);
         c->launches++;
     };
     cplx* W = w.buf;
@@ -781,10 +1010,8 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
     cplx* E1h = w.buf + 5 * w.nrho;
     int* n_iter = reinterpret_cast<int*>(G.fro + ns);
     const OaTables oat = oa_tables(G);
-    launch_pdl(k_jacobi32, ns, JT, G.jac_smem, s, rho, W, G.fro, n_iter, G.flags, tb, w.gwork, G.grec, G.nrec, G.jac_smem,
-               false, 0, G.stats);
+    launch_pdl(k_seed, ns, JT, G.seed_smem, s, rho, W, G.fro, n_iter, G.flags, tb, w.gwork, G.stats);
     c->launches += 1;
-    replay(W, false);
     GemmArgs a{};
     a.dscale = c->dscale;
     a.bufs[EB_RHO] = const_cast<cplx*>(rho);
@@ -817,9 +1044,9 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
         }
         if (reseed_iter(it)) {
             launch_pdl(k_jacobi32, ns, JT, G.jac_smem, s, S, E1h, G.fro, n_iter, G.flags, tb, w.gwork, G.grec, G.nrec,
-                       G.jac_smem, true, it, G.stats);
+                       G.jac_smem, it);
             c->launches++;
-            replay(E1h, true);
+            replay(E1h);
         }
         if (e == cudaSuccess) e = gemm(G.tl_y, true);
         if (G.noa) c->launches += orth_only ? 1 : 2;
@@ -855,6 +1082,7 @@ int eig_prepare(tdmrg_ctx* c, int side) {
         // the opt-in is a property of the kernel on the device, shared by every context: always the maximum
         if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, kJacSmemCap),
                                  "eig smem");
+        if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(k_seed, cudaFuncAttributeMaxDynamicSharedMemorySize, kJacSmemCap), "eig smem");
         if (rc) return rc;
         // the longest Jacobi seeds on a second stream, beside the other sectors' seeds and refinement
         const std::vector<int> lng = long_sectors(L.dim);

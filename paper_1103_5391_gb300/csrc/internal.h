@@ -275,7 +275,8 @@ struct EigGroup {
     void* tables = nullptr;     // per-sector offsets (into the side's packed rho) and dims
     size_t tables_bytes = 0;
     double* fro = nullptr;      // per sector ||rho||_F, then the iteration count (int)
-    int jac_smem = 0;           // dynamic shared memory of the Jacobi launch
+    int jac_smem = 0;           // dynamic shared memory of the re-seed Jacobi launch
+    int seed_smem = 0;          // and of the seed launch
     int* flags = nullptr;       // per sector: re-seed requested by the refinement
     float4* grec = nullptr;     // Jacobi rotation records of the sectors too large for V in shared memory
     int64_t grec_entries = 0;
