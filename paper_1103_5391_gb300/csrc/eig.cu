@@ -397,13 +397,19 @@ __global__ void __launch_bounds__(kReplayThreads) k_jacobi_replay(const float4* 
 //     eigenvalues relative to delta ||rho|| rather than to eps ||rho||: fewer sweeps, seeds an order of magnitude
 //     closer (simulated over decaying, Wishart, rank-deficient and multiplet spectra, n = 20 ... 152: one or two
 //     refinement iterations fewer).
-// Measured, the whole decomposition against the two-sided seed with V by rotation replay: L=32 m=400 1041 -> 568 us,
-// L=48 m=1000 8.93 -> 4.95 ms; the seed of n = 60 517 -> ~250 us, n = 152 5.1 -> 3.8 ms.  Bound by the latency of a
-// pair's chain (load, 5 shuffle levels, rotation, store: ~1000 cycles a round) up to n = 64, by shared-memory
-// traffic of 16 n^2 bytes a round beyond.
-// Columns are rows of T (T[c][r] = L[r][c], contiguous in r), lanes run over r.  One CTA per sector; T in shared
-// memory up to n = kSeedSmemN, else in `gwork`.
-constexpr int kSeedSmemN = 168;            // 8 n^2 bytes <= kJacSmemCap
+// Eight lanes own a pair: the reduction, the rotation and the addressing, ~100 instructions whatever n, are then shared by
+// four pairs of a warp (a warp per pair issued 250 instructions a pair at n = 152, 4 x the columns' own work).  A sector
+// above kSeedClusterN columns is spread over a cluster of four CTAs by rows (a round moves 16 n^2 bytes through shared
+// memory, 2900 cycles on one SM at n = 152).
+// Measured, cycles per round: n = 60 1480 (warp per pair) -> 1130, n = 124 3830 -> 3230 (eight lanes) -> 1940 (cluster),
+// n = 152 5330 -> 4610 -> 2510; the decomposition at L=32 m=400 1041 us (two-sided seed with V by rotation replay) -> 568
+// -> 521, at L=48 m=1000 8.93 ms -> 4.95 -> 4.67 -> 3.99.  Bound by the latency of a pair's chain (load, 3 shuffle levels,
+// rotation, store, barrier: ~640 cycles; the cluster's exchange adds ~700) and, from n ~ 100, by instruction issue.
+// Columns are rows of T (T[c][r] = L[r][c], contiguous in r), lanes run over r.  T in shared memory up to n = kSeedSmemN,
+// else in `gwork` (one CTA, a warp per pair).
+constexpr int ST = 640;                    // threads of the seed CTA: 80 pairs of eight lanes
+constexpr int kSeedSmemN = 160;            // largest sector with T in shared memory (2 * ST / 8 columns, 205 KB)
+__host__ __device__ constexpr int seed_ld(int n) { return (n + 15) / 16 * 16; }
 constexpr float kSeedShift = 1e-4f;        // delta, above the factorisation's rounding (~n 2^-24)
 constexpr float kSeedTol2 = 1e-12f;        // a pair is rotated while |<x, y>|^2 > kSeedTol2 |x|^2 |y|^2 ...
 constexpr float kSeedStop2 = 2.5e-7f;      // ... and sweeps end after one whose largest ratio was below this (convergence
@@ -427,88 +433,220 @@ __device__ __forceinline__ double f64_of(float v) {
     return __hiloint2double((int)hi, (int)(u << 29));
 }
 
-// Warp sums of g, a and b, in every lane: reduce-scatter to one value per 8 lanes, then broadcasts
-__device__ __forceinline__ void warp_sum4(float2& g, float& a, float& b) {
-    const int lane = threadIdx.x & 31;
-    const bool u16 = lane & 16, u8 = lane & 8;
-    float k0 = u16 ? a : g.x, k1 = u16 ? b : g.y;
-    k0 += __shfl_xor_sync(0xffffffffu, u16 ? g.x : a, 16);
-    k1 += __shfl_xor_sync(0xffffffffu, u16 ? g.y : b, 16);
-    float k = u8 ? k1 : k0;
-    k += __shfl_xor_sync(0xffffffffu, u8 ? k0 : k1, 8);
-    k += __shfl_xor_sync(0xffffffffu, k, 4);
-    k += __shfl_xor_sync(0xffffffffu, k, 2);
-    k += __shfl_xor_sync(0xffffffffu, k, 1);
-    g.x = __shfl_sync(0xffffffffu, k, 0);
-    g.y = __shfl_sync(0xffffffffu, k, 8);
-    a = __shfl_sync(0xffffffffu, k, 16);
-    b = __shfl_sync(0xffffffffu, k, 24);
+__device__ __forceinline__ float rsqrt_approx(float v) {   // normal arguments only
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+// c and s of rotation32 on the Gram block [[a, g], [conj(g), b]], g != 0, through cos^2 = 1/2 + |x| / 2r; not normalised
+// (a common factor of the two rotated columns drops out when they are normalised at the end).
+__device__ __forceinline__ void seed_rotation(float a, float b, float2 g, float g2, float& c, float2& s) {
+    const float x = b - a;
+    const float ir = rsqrt_approx(fmaf(x, x, 4.f * g2));
+    const float h = fmaf(0.5f * fabsf(x), ir, 0.5f);
+    const float ic = rsqrt_approx(h);
+    c = h * ic;
+    const float f = copysignf(ir * ic, x);
+    s = make_float2(f * g.x, f * g.y);
 }
 
-// Orthogonalises columns x and y; returns whether their ratio was above the stopping limit.  E > 0: the columns
-// have at most 32 E entries and stay in registers; E = 0: any length, read twice.
-template <int E>
-__device__ __forceinline__ bool seed_pair(float2* x, float2* y, int n) {
-    const int lane = threadIdx.x & 31;
-    float2 g = make_float2(0.f, 0.f);
-    float a = 0.f, b = 0.f;
-    float2 xv[E > 0 ? E : 1], yv[E > 0 ? E : 1];
-    auto dots = [&](float2 u, float2 v) {
-        g.x = fmaf(u.x, v.x, fmaf(u.y, v.y, g.x));   // conj(x) y
-        g.y = fmaf(u.x, v.y, fmaf(-u.y, v.x, g.y));
-        a = fmaf(u.x, u.x, fmaf(u.y, u.y, a));
-        b = fmaf(v.x, v.x, fmaf(v.y, v.y, b));
-    };
-    if constexpr (E > 0) {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int r = lane + 32 * e;
-            const bool in = e + 1 < E || r < n;
-            xv[e] = in ? x[r] : make_float2(0.f, 0.f);
-            yv[e] = in ? y[r] : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) dots(xv[e], yv[e]);
-    } else {
-        for (int r = lane; r < n; r += 32) dots(x[r], y[r]);
+// ---- clusters: a sector above kSeedClusterN is shared by the CTAs of a cluster, each holding a slab of rows.  A pair's
+// inner products are summed over the slabs through distributed shared memory (every CTA sends its partial sums to every
+// CTA, counted by an mbarrier there), in the same order everywhere, so that all CTAs make the same rotation from the same bits.
+constexpr int kSeedCluster = 4;
+constexpr int kSeedClusterN = 64;
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// address of this CTA's shared variable at `addr` in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned map_rank(unsigned addr, unsigned rank) {
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(unsigned addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+// 16 bytes into another CTA's shared memory, counted by that CTA's mbarrier
+__device__ __forceinline__ void st_async4(unsigned addr, float4 v, unsigned bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+// Bounded wait for a phase of an mbarrier of this CTA whose bytes come from the cluster
+__device__ __forceinline__ bool mbar_wait_cluster(unsigned bar, unsigned parity) {
+    for (int i = 0; i < (1 << 20); ++i) {
+        unsigned done;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
     }
-    warp_sum4(g, a, b);
-    const float g2 = fmaf(g.x, g.x, g.y * g.y), ab = a * b;
-    if (g2 <= kSeedTol2 * ab) return false;
-    float c;
-    float2 s;
-    rotation32(a, b, g, c, s);
-    const float2 sc = conjf2(s);
-    if constexpr (E > 0) {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int r = lane + 32 * e;
-            if (e + 1 < E || r < n) {
-                x[r] = rot_l(c, sc, xv[e], yv[e]);
-                y[r] = rot_r(c, s, xv[e], yv[e]);
-            }
-        }
-    } else {
-        for (int r = lane; r < n; r += 32) {
-            const float2 u = x[r], v = y[r];
-            x[r] = rot_l(c, sc, u, v);
-            y[r] = rot_r(c, s, u, v);
-        }
-    }
-    return g2 > kSeedStop2 * ab;
+    return false;
 }
 
-template <int E>
-__device__ __forceinline__ int seed_sweeps(float2* T, int n) {
-    const int P = n + (n & 1), npair = P / 2, R = P - 1, warp = threadIdx.x >> 5;
-    int sweep = 0;
-    for (bool more = n > 1; more && sweep < kSeedSweeps; ++sweep) {
+// Sums of g, a and b over LP = 8 or 32 lanes by reduce-scatter: lane l of the group gets component 4 l / LP of
+// (g.x, g.y, a, b); group_sum4 broadcasts them to every lane.
+template <int LP>
+__device__ __forceinline__ float group_scatter4(float2 g, float a, float b) {
+    const int lane = threadIdx.x & 31;
+    const bool up1 = lane & (LP / 2), up2 = lane & (LP / 4);
+    float k0 = up1 ? a : g.x, k1 = up1 ? b : g.y;
+    k0 += __shfl_xor_sync(0xffffffffu, up1 ? g.x : a, LP / 2);
+    k1 += __shfl_xor_sync(0xffffffffu, up1 ? g.y : b, LP / 2);
+    float k = up2 ? k1 : k0;
+    k += __shfl_xor_sync(0xffffffffu, up2 ? k0 : k1, LP / 4);
+#pragma unroll
+    for (int o = LP / 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    return k;
+}
+template <int LP>
+__device__ __forceinline__ void group_sum4(float2& g, float& a, float& b) {
+    const int base = threadIdx.x & 31 & ~(LP - 1);
+    const float k = group_scatter4<LP>(g, a, b);
+    g.x = __shfl_sync(0xffffffffu, k, base);
+    g.y = __shfl_sync(0xffffffffu, k, base + LP / 4);
+    a = __shfl_sync(0xffffffffu, k, base + LP / 2);
+    b = __shfl_sync(0xffffffffu, k, base + 3 * LP / 4);
+}
+
+__device__ __forceinline__ void pair_dots(float2 u, float2 v, float2& g, float& a, float& b) {
+    g.x = fmaf(u.x, v.x, fmaf(u.y, v.y, g.x));   // conj(x) y
+    g.y = fmaf(u.x, v.y, fmaf(-u.y, v.x, g.y));
+    a = fmaf(u.x, u.x, fmaf(u.y, u.y, a));
+    b = fmaf(v.x, v.x, fmaf(v.y, v.y, b));
+}
+
+// Sweeps with T in shared memory, columns zero-padded to ld (a multiple of 16).  Eight lanes own a pair, two rows (16
+// bytes) per lane and step, both columns in registers.  CS = 1: all rows (ld = 16 E), the warps without a pair do not
+// take part.  CS > 1: this CTA's rows [row0, row0 + 16 E) below ld; ex: the exchange buffers [2][CS][ST / 8].
+// bars: an mbarrier per buffer; status: gets a bit when a bounded wait runs out (the sector's seed is then unfinished).
+template <int E, int CS>
+__device__ __forceinline__ int seed_sweeps(float2* T, int n, int ld, int row0, float4* ex, uint64_t* bars, int* status) {
+    const int P = n + (n & 1), npair = P / 2, R = P - 1, nthr = 32 * ((npair + 3) / 4);
+    const int pr = threadIdx.x >> 3, l8 = threadIdx.x & 7;
+    if ((int)threadIdx.x >= nthr || n < 2) return 0;
+    unsigned dst = 0u, dbar = 0u;   // lane l8 < CS sends the pair's sums to CTA l8
+    const unsigned bar0 = (unsigned)__cvta_generic_to_shared(bars);
+    if (CS > 1 && l8 < CS) {
+        dst = map_rank((unsigned)__cvta_generic_to_shared(ex + cluster_rank() * (ST / 8) + pr), l8);
+        dbar = map_rank(bar0, l8);
+    }
+    int phase = 0;    // parity of the current buffer's mbarrier phase
+    bool lost = false;
+    int sweep = 0, par = 1;
+    for (bool more = true; more && sweep < kSeedSweeps; ++sweep) {
         bool big = false;
         for (int round = 0; round < R; ++round) {
-            for (int i = warp; i < npair; i += JT / 32) {
+            par ^= 1;   // the exchange buffer of this round
+            if (CS > 1 && par == 0 && (round > 0 || sweep > 0)) phase ^= 1;
+            int p = 0, q = n;
+            if (pr < npair) rr_pair(round, pr, P, p, q);
+            const bool on = q < n;   // otherwise the group only takes part in its warp's shuffles
+            float4* xp = reinterpret_cast<float4*>(T + p * ld + row0) + l8;
+            float4* yp = reinterpret_cast<float4*>(T + (on ? q : p) * ld + row0) + l8;
+            float4 x[E], y[E];
+            float2 g = make_float2(0.f, 0.f);
+            float a = 0.f, b = 0.f;
+            {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const bool in = CS == 1 || row0 + 16 * e < ld;
+                    x[e] = in ? xp[8 * e] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    y[e] = in ? yp[8 * e] : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    pair_dots(make_float2(x[e].x, x[e].y), make_float2(y[e].x, y[e].y), g, a, b);
+                    pair_dots(make_float2(x[e].z, x[e].w), make_float2(y[e].z, y[e].w), g, a, b);
+                }
+                group_sum4<8>(g, a, b);
+            }
+            if (CS > 1) {
+                // Buffers alternate: one is sent to again two rounds later, after every CTA has had this CTA's sums of the
+                // round between, which follow the barrier at the end of the round that read it.
+                if (threadIdx.x == 0)
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 8 * par),
+                                 "r"(CS * npair * (int)sizeof(float4)) : "memory");
+                if (pr < npair && l8 < CS)
+                    st_async4(dst + par * (unsigned)(CS * (ST / 8) * sizeof(float4)), make_float4(g.x, g.y, a, b), dbar + 8 * par);
+                if (!lost && !mbar_wait_cluster(bar0 + 8 * par, phase)) {
+                    lost = true;
+                    atomicOr(status, 8);
+                }
+                __syncwarp();
+                const float4* in = ex + par * CS * (ST / 8) + pr;
+                float4 t = in[0];
+#pragma unroll
+                for (int k = 1; k < CS; ++k) {
+                    const float4 u = in[k * (ST / 8)];
+                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                }
+                g = make_float2(t.x, t.y);
+                a = t.z;
+                b = t.w;
+            }
+            const float g2 = fmaf(g.x, g.x, g.y * g.y), ab = a * b;
+            if (on && g2 > kSeedTol2 * ab) {
+                big |= g2 > kSeedStop2 * ab;
+                float c;
+                float2 s;
+                seed_rotation(a, b, g, g2, c, s);
+                const float2 sc = conjf2(s);
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    if (CS > 1 && row0 + 16 * e >= ld) continue;
+                    const float2 x0 = make_float2(x[e].x, x[e].y), x1 = make_float2(x[e].z, x[e].w);
+                    const float2 y0 = make_float2(y[e].x, y[e].y), y1 = make_float2(y[e].z, y[e].w);
+                    const float2 u0 = rot_l(c, sc, x0, y0), u1 = rot_l(c, sc, x1, y1);
+                    const float2 v0 = rot_r(c, s, x0, y0), v1 = rot_r(c, s, x1, y1);
+                    xp[8 * e] = make_float4(u0.x, u0.y, u1.x, u1.y);
+                    yp[8 * e] = make_float4(v0.x, v0.y, v1.x, v1.y);
+                }
+            }
+            if (round + 1 < R) asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+        }
+        int any;
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %2, 0;\n bar.red.or.pred q, 1, %1, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+                     : "=r"(any) : "r"(nthr), "r"((int)big) : "memory");
+        more = any != 0;
+    }
+    return sweep;
+}
+
+// Sweeps with T in global memory (row stride n): a warp per pair, the columns read twice
+__device__ __forceinline__ int seed_sweeps_global(float2* T, int n) {
+    const int P = n + (n & 1), npair = P / 2, R = P - 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int sweep = 0;
+    for (bool more = true; more && sweep < kSeedSweeps; ++sweep) {
+        bool big = false;
+        for (int round = 0; round < R; ++round) {
+            for (int i = warp; i < npair; i += ST / 32) {
                 int p, q;
                 rr_pair(round, i, P, p, q);
-                if (q < n) big |= seed_pair<E>(T + p * n, T + q * n, n);
+                if (q >= n) continue;
+                float2* x = T + (int64_t)p * n;
+                float2* y = T + (int64_t)q * n;
+                float2 g = make_float2(0.f, 0.f);
+                float a = 0.f, b = 0.f;
+                for (int r = lane; r < n; r += 32) pair_dots(x[r], y[r], g, a, b);
+                group_sum4<32>(g, a, b);
+                const float g2 = fmaf(g.x, g.x, g.y * g.y), ab = a * b;
+                if (g2 <= kSeedTol2 * ab) continue;
+                big |= g2 > kSeedStop2 * ab;
+                float c;
+                float2 s;
+                seed_rotation(a, b, g, g2, c, s);
+                const float2 sc = conjf2(s);
+                for (int r = lane; r < n; r += 32) {
+                    const float2 u = x[r], v = y[r];
+                    x[r] = rot_l(c, sc, u, v);
+                    y[r] = rot_r(c, s, u, v);
+                }
             }
             if (round + 1 < R) __syncthreads();
         }
@@ -517,13 +655,13 @@ __device__ __forceinline__ int seed_sweeps(float2* T, int n) {
     return sweep;
 }
 
-// T[c][r] = A[r][c] 2^-e for r >= c (0 above) plus `shift` on the diagonal
-__device__ __forceinline__ void seed_load(const cplx* __restrict__ R, float2* T, int n, int e, float shift) {
-    for (int x = threadIdx.x; x < n * n; x += JT) {
-        const int c = x / n, r = x - c * n;
+// T[c][r] = A[r][c] 2^-e for r >= c (0 above and in the padding r >= n) plus `shift` on the diagonal
+__device__ __forceinline__ void seed_load(const cplx* __restrict__ R, float2* T, int n, int ld, int e, float shift) {
+    for (int x = threadIdx.x; x < n * ld; x += ST) {
+        const int c = x / ld, r = x - c * ld;
         float2 v = make_float2(0.f, 0.f);
-        if (r >= c) {
-            const double2 a = R[x];   // A[c][r] = conj(A[r][c])
+        if (r >= c && r < n) {
+            const double2 a = R[(int64_t)c * n + r];   // A[c][r] = conj(A[r][c])
             v = r == c ? make_float2(f32_of(a.x, e) + shift, 0.f) : make_float2(f32_of(a.x, e), -f32_of(a.y, e));
         }
         T[x] = v;
@@ -531,82 +669,111 @@ __device__ __forceinline__ void seed_load(const cplx* __restrict__ R, float2* T,
 }
 
 // Right-looking Cholesky of the lower triangle held in T, columns left unscaled; false when a pivot falls below lim
-__device__ __forceinline__ bool seed_cholesky(float2* T, int n, float lim) {
+__device__ __forceinline__ bool seed_cholesky(float2* T, int n, int ld, float lim) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int k = 0; k < n; ++k) {
         __syncthreads();
-        const float d = T[k * n + k].x;
+        const float d = T[k * ld + k].x;
         if (!(d > lim)) return false;   // the same value in every thread
         const float inv = 1.f / d;
-        for (int j = k + 1 + warp; j < n; j += JT / 32) {
-            const float2 f = T[k * n + j];
+        for (int j = k + 1 + warp; j < n; j += ST / 32) {
+            const float2 f = T[k * ld + j];
             const float2 fc = make_float2(f.x * inv, -f.y * inv);
             for (int i = j + lane; i < n; i += 32) {
-                const float2 t = cmf(T[k * n + i], fc);
-                float2* p = T + j * n + i;
+                const float2 t = cmf(T[k * ld + i], fc);
+                float2* p = T + j * ld + i;
                 *p = make_float2(p->x - t.x, p->y - t.y);
             }
         }
     }
     __syncthreads();
-    for (int k = warp; k < n; k += JT / 32) {   // columns of L
-        const float sc = rsqrtf(T[k * n + k].x);
+    for (int k = warp; k < n; k += ST / 32) {   // columns of L
+        const float sc = rsqrtf(T[k * ld + k].x);
         __syncwarp();
-        for (int i = k + lane; i < n; i += 32) { T[k * n + i].x *= sc; T[k * n + i].y *= sc; }
+        for (int i = k + lane; i < n; i += 32) { T[k * ld + i].x *= sc; T[k * ld + i].y *= sc; }
     }
     __syncthreads();
     return true;
 }
 
-// The seed of one sector with T in shared memory (SM, inlined so that its accesses compile as such) or global
-// memory; e: the sector's exponent.  Returns the number of sweeps.
-template <bool SM>
-__device__ __forceinline__ int seed_sector(const cplx* __restrict__ R, cplx* __restrict__ W, double* rho_fro, float2* T, int n, int e) {
+// The seed of one sector with T in shared memory (inlined so that its accesses compile as such) or global
+// memory; e: the sector's exponent; rank: this CTA's in the cluster (SEED_CLUSTER: every CTA makes the factor, then keeps
+// a slab of rows).  Returns the number of sweeps.
+enum SeedMode { SEED_SMEM = 0, SEED_CLUSTER = 1, SEED_GLOBAL = 2 };
+template <SeedMode MODE>
+__device__ __forceinline__ int seed_sector(const cplx* __restrict__ R, cplx* __restrict__ W, double* rho_fro, float2* T, int n, int e,
+                                           int rank, float4* ex, uint64_t* bars, int* status) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    __shared__ float redf[JT / 32];
-    seed_load(R, T, n, e, 0.f);
+    const int ld = MODE != SEED_GLOBAL ? seed_ld(n) : n;
+    // this CTA's rows
+    const int slab = MODE == SEED_CLUSTER ? 16 * ((ld + 16 * kSeedCluster - 1) / (16 * kSeedCluster)) : ld;
+    const int row0 = MODE == SEED_CLUSTER ? rank * slab : 0, row1 = min(n, row0 + slab);
+    __shared__ float redf[ST / 32];
+    seed_load(R, T, n, ld, e, 0.f);
     __syncthreads();
     float f = 0.f;
-    for (int x = tid; x < n * n; x += JT) {   // entries off the diagonal count twice
+    for (int x = tid; x < n * ld; x += ST) {   // entries off the diagonal count twice
         const float2 v = T[x];
-        f += (x / n == x % n ? 1.f : 2.f) * fmaf(v.x, v.x, v.y * v.y);
+        f += (x / ld == x % ld ? 1.f : 2.f) * fmaf(v.x, v.x, v.y * v.y);
     }
     for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
     if (lane == 0) redf[warp] = f;
     __syncthreads();
-    f = redf[lane];
+    f = lane < ST / 32 ? redf[lane] : 0.f;
     for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
     const float nf = sqrtf(f);
-    if (tid == 0) *rho_fro = ldexp((double)nf, e);   // the refinement's cluster threshold
+    if (tid == 0 && (MODE != SEED_CLUSTER || rank == 0)) *rho_fro = ldexp((double)nf, e);   // the refinement's cluster threshold
     int sweeps = 0;
     if (nf > 0.f) {
         // the first shift serves every positive semidefinite block; a matrix with eigenvalues below -delta
         // ||rho|| (no density matrix) is shifted by more than its norm
         float shift = kSeedShift * nf;
         __syncthreads();
-        for (int x = tid; x < n; x += JT) T[x * n + x].x += shift;
-        if (!seed_cholesky(T, n, 0.5f * shift)) {
+        for (int x = tid; x < n; x += ST) T[x * ld + x].x += shift;
+        if (!seed_cholesky(T, n, ld, 0.5f * shift)) {
             __syncthreads();
-            seed_load(R, T, n, e, 1.05f * nf);
-            seed_cholesky(T, n, 0.f);
+            seed_load(R, T, n, ld, e, 1.05f * nf);
+            seed_cholesky(T, n, ld, 0.f);
         }
-        switch (SM ? (n + 31) / 32 : 0) {
-            case 1: sweeps = seed_sweeps<1>(T, n); break;
-            case 2: sweeps = seed_sweeps<2>(T, n); break;
-            case 3: sweeps = seed_sweeps<3>(T, n); break;
-            case 4: sweeps = seed_sweeps<4>(T, n); break;
-            case 5: sweeps = seed_sweeps<5>(T, n); break;
-            case 6: sweeps = seed_sweeps<6>(T, n); break;
-            default: sweeps = seed_sweeps<0>(T, n);
+        if constexpr (MODE == SEED_SMEM) {
+            switch (ld / 16) {
+                case 1: sweeps = seed_sweeps<1, 1>(T, n, ld, 0, ex, bars, status); break;
+                case 2: sweeps = seed_sweeps<2, 1>(T, n, ld, 0, ex, bars, status); break;
+                case 3: sweeps = seed_sweeps<3, 1>(T, n, ld, 0, ex, bars, status); break;
+                default: sweeps = seed_sweeps<4, 1>(T, n, ld, 0, ex, bars, status);
+            }
+            __syncthreads();   // the warps without a pair wait here
+        } else if constexpr (MODE == SEED_CLUSTER) {
+            sweeps = slab <= 32 ? seed_sweeps<2, kSeedCluster>(T, n, ld, row0, ex, bars, status) : seed_sweeps<3, kSeedCluster>(T, n, ld, row0, ex, bars, status);
+            __syncthreads();
+        } else {
+            sweeps = seed_sweeps_global(T, n);
         }
     }
-    for (int c = warp; c < n; c += JT / 32) {   // W row c = (column c)^H / |column c|
+    // W row c = (column c)^H / |column c|
+    float* norms = reinterpret_cast<float*>(ex);   // cluster: [rank][column] partial squared norms
+    if constexpr (MODE == SEED_CLUSTER) {
+        cluster_sync();   // the exchange buffers are no longer read
+        for (int c = warp; c < n; c += ST / 32) {
+            float q = 0.f;
+            for (int r = row0 + lane; r < row1; r += 32) { const float2 v = T[c * ld + r]; q = fmaf(v.x, v.x, fmaf(v.y, v.y, q)); }
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane < kSeedCluster)
+                st_cluster(map_rank((unsigned)__cvta_generic_to_shared(norms + rank * kSeedSmemN + c), lane), q);
+        }
+        cluster_sync();
+    }
+    for (int c = warp; c < n; c += ST / 32) {
         float q = 0.f;
-        for (int r = lane; r < n; r += 32) { const float2 v = T[c * n + r]; q = fmaf(v.x, v.x, fmaf(v.y, v.y, q)); }
-        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if constexpr (MODE == SEED_CLUSTER) {
+            for (int k = 0; k < kSeedCluster; ++k) q += norms[k * kSeedSmemN + c];
+        } else {
+            for (int r = lane; r < n; r += 32) { const float2 v = T[c * ld + r]; q = fmaf(v.x, v.x, fmaf(v.y, v.y, q)); }
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        }
         const float inv = q > 0.f ? 1.f / sqrtf(q) : 0.f;
-        for (int r = lane; r < n; r += 32) {
-            const float2 v = T[c * n + r];
+        for (int r = row0 + lane; r < row1; r += 32) {
+            const float2 v = T[c * ld + r];
             const float2 u = nf > 0.f ? make_float2(v.x * inv, -v.y * inv) : make_float2(r == c ? 1.f : 0.f, 0.f);
             W[(int64_t)c * n + r] = make_double2(f64_of(u.x), f64_of(u.y));
         }
@@ -614,36 +781,49 @@ __device__ __forceinline__ int seed_sector(const cplx* __restrict__ R, cplx* __r
     return sweeps;
 }
 
-// W0 = X0^H of every sector (rows unsorted), ||rho||_F, the initial iteration count, cleared re-seed flags.
-__global__ void __launch_bounds__(JT) k_seed(const cplx* __restrict__ rho, cplx* __restrict__ W, double* __restrict__ rho_fro,
+// W0 = X0^H of every sector (rows unsorted), ||rho||_F, the initial iteration count, cleared re-seed flags.  items: the
+// sector of every CTA (-1: none), plus kSeedShared when the CTAs of the cluster share it.
+constexpr int kSeedShared = 1 << 20;
+__global__ void __launch_bounds__(ST) k_seed(const cplx* __restrict__ rho, cplx* __restrict__ W, double* __restrict__ rho_fro,
                                              int* __restrict__ n_iter, int* __restrict__ flags, EigTables tb,
-                                             float2* __restrict__ gwork, int2* __restrict__ stats) {
+                                             float2* __restrict__ gwork, int2* __restrict__ stats, const int* __restrict__ items,
+                                             int* __restrict__ status) {
     pdl_enter();
     const long long t_start = clock64();
     extern __shared__ float4 fsm4[];
-    const int sct = blockIdx.x, n = tb.dims[sct], tid = threadIdx.x;
+    __shared__ float4 ex[2 * kSeedCluster * (ST / 8)];
+    __shared__ int rede[ST / 32];
+    __shared__ __align__(8) uint64_t bars[2];
+    const int item = items[blockIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_iter = kRefine;
+    if (item < 0) return;
+    const bool shared = item >= kSeedShared;
+    const int sct = shared ? item - kSeedShared : item, n = tb.dims[sct], tid = threadIdx.x;
+    const int rank = shared ? (int)cluster_rank() : 0;
+    if (shared) {   // every CTA's mbarriers are ready before any CTA sends
+        if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bars + tid)));
+        if (tid < 2) asm volatile("fence.mbarrier_init.release.cluster;");
+        cluster_sync();
+    }
     const int warp = tid >> 5, lane = tid & 31;
     const int64_t off = tb.off[sct];
     const cplx* __restrict__ R = rho + off;
-    __shared__ int rede[JT / 32];
-    int ex = 0;   // largest biased exponent: the sector is scaled by a power of two so that no square underflows
-    for (int x = tid; x < n * n; x += JT) {
+    int ex2 = 0;   // largest biased exponent: the sector is scaled by a power of two so that no square underflows
+    for (int x = tid; x < n * n; x += ST) {
         const double2 v = R[x];
-        ex = max(ex, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
+        ex2 = max(ex2, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
     }
-    ex = __reduce_max_sync(0xffffffffu, ex);
-    if (lane == 0) rede[warp] = ex;
+    ex2 = __reduce_max_sync(0xffffffffu, ex2);
+    if (lane == 0) rede[warp] = ex2;
     __syncthreads();
-    ex = __reduce_max_sync(0xffffffffu, rede[lane]);
-    const int e = ex - 1023;
-    if (tid == 0) {
-        flags[sct] = 0;
-        if (sct == 0) *n_iter = kRefine;
-    }
-    const int sweeps = n <= kSeedSmemN ? seed_sector<true>(R, W + off, rho_fro + sct, reinterpret_cast<float2*>(fsm4), n, e)
-                                       : seed_sector<false>(R, W + off, rho_fro + sct, gwork + 4 * off, n, e);
+    const int e = __reduce_max_sync(0xffffffffu, lane < ST / 32 ? rede[lane] : 0) - 1023;
+    if (tid == 0 && rank == 0) flags[sct] = 0;
+    float2* T = reinterpret_cast<float2*>(fsm4);
+    const int sweeps = shared            ? seed_sector<SEED_CLUSTER>(R, W + off, rho_fro + sct, T, n, e, rank, ex, bars, status)
+                       : n <= kSeedClusterN ? seed_sector<SEED_SMEM>(R, W + off, rho_fro + sct, T, n, e, 0, ex, bars, status)
+                                         : seed_sector<SEED_GLOBAL>(R, W + off, rho_fro + sct, gwork + 4 * off, n, e, 0, ex, bars, status);
     // sweeps and SM cycles of the sector's seed (a measurement aid; tdmrg_eig_stats)
-    if (tid == 0) stats[sct] = make_int2(sweeps, (int)min(clock64() - t_start, (long long)INT_MAX));
+    if (tid == 0 && rank == 0) stats[sct] = make_int2(sweeps, (int)min(clock64() - t_start, (long long)INT_MAX));
 }
 
 // Refinement on W = X^H, which turns every product into a plain or conjugate-transposed operand of the
@@ -764,9 +944,11 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
             double2 ev;
             const double li = lam[eo + i], lj = lam[eo + j], gap = fabs(li - lj);
             const double2 num = make_double2(sv[u].x + li * r.x, sv[u].y + li * r.y);
-            // a close pair whose numerator is rounding (an exact multiplet in an iterate that has converged while
-            // other sectors go on) would be turned by noise / noise: a cluster as well
-            const bool near = gap <= delta || (gap <= kNearGap * fro && fmax(fabs(num.x), fabs(num.y)) <= kNearNum * fro);
+            // the larger numerator of E_ij and E_ji, so that both take the same branch
+            const double nm = fmax(fmax(fabs(num.x), fabs(num.y)), fmax(fabs(sv[u].x + lj * r.x), fabs(sv[u].y + lj * r.y)));
+            // A close pair whose numerator is rounding (an exact multiplet in an iterate that has converged while other
+            // sectors go on) would be turned by noise / noise: a cluster as well.
+            const bool near = gap <= delta || (gap <= kNearGap * fro && nm <= kNearNum * fro);
             if (!orth_only && i != j && !near) {
                 const double inv = 1.0 / (li - lj);
                 ev = make_double2(num.x * inv, num.y * inv);
@@ -846,12 +1028,10 @@ size_t oa_bytes(int noa, int ns) {
 enum { EB_RHO = BUF_EXTRA0, EB_W, EB_AX, EB_S, EB_G, EB_E, EB_WN };
 
 // Cost model of the split into two groups, in SM cycles: the seed of one sector (about 7.5 sweeps of n - 1 rounds; a
-// round costs ~700 + 14 n cycles while a pair per warp is enough, ~300 + 32 n beyond) and the refinement of a
-// sector spread over the GPU, 0.4 n^3 (the products alone are ~0.1 n^3; measured over 0.03 ... 1.5: the decomposition at
-// L=48 m=1000 takes 5.7 ms up to 0.12 and 4.95 ms from 0.2 on, L=32 m=400 and m=800 change by 4 %).
-// Measured seeds, cycles per round: n = 21 990, 42 1360, 54 1480, 68 2540, 98 3360, 124 3830, 152 5330.  It only decides
-// the scheduling.
-double jacobi_cost(int n) { return 7.5 * std::max(n - 1, 0) * (n <= 64 ? 700.0 + 14.0 * n : 300.0 + 32.0 * n); }
+// round costs ~500 + 12 n cycles, in a cluster ~600 + 14 n) and the refinement of a sector spread over the GPU,
+// 0.4 n^3 (the products alone are ~0.1 n^3; measured over 0.03 ... 1.5: the decomposition at L=48 m=1000 took 5.7 ms up
+// to 0.12 and 4.95 ms from 0.2 on, L=32 m=400 and m=800 changed by 4 %).  It only decides the scheduling.
+double jacobi_cost(int n) { return 7.5 * std::max(n - 1, 0) * (n <= kSeedClusterN ? 500.0 + 12.0 * n : 600.0 + 14.0 * n); }
 double refine_cost(int n) { return 0.4 * (double)n * n * n; }
 
 // Sectors of the first group (run on the second stream): the k with the longest Jacobi seeds, k chosen to
@@ -978,8 +1158,23 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
         smem = std::max(smem, jac_base_bytes(n) + 32 * (P / 2) * (P - 1));
     }
     G.jac_smem = std::min(smem, kJacSmemCap);
-    for (int k = 0; k < ns; ++k)
-        if (dim[k] <= kSeedSmemN) G.seed_smem = std::max(G.seed_smem, 8 * dim[k] * dim[k]);
+    // seed CTAs: the shared sectors first, the largest ahead, a cluster each; then one sector per CTA, clusters filled
+    std::vector<int> order(ns), items;
+    for (int k = 0; k < ns; ++k) {
+        order[k] = k;
+        if (dim[k] <= kSeedSmemN) G.seed_smem = std::max(G.seed_smem, 8 * dim[k] * seed_ld(dim[k]));
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return dim[x] > dim[y]; });
+    auto is_shared = [&](int k) { return dim[k] > kSeedClusterN && dim[k] <= kSeedSmemN; };
+    for (int k : order)
+        if (is_shared(k)) items.insert(items.end(), kSeedCluster, k + kSeedShared);
+    G.seed_cluster = items.empty() ? 1 : kSeedCluster;
+    for (int k : order)
+        if (!is_shared(k)) items.push_back(k);
+    while (items.size() % G.seed_cluster) items.push_back(-1);
+    G.nseed = (int)items.size();
+    rc = dev_alloc(c, (void**)&G.seed_items, (size_t)G.nseed * sizeof(int), "eig seed items");
+    if (!rc) rc = cuda_check(c, cudaMemcpy(G.seed_items, items.data(), (size_t)G.nseed * sizeof(int), cudaMemcpyHostToDevice), "eig seed items");
     for (int k = 0; k < ns && !rc; ++k)
         if (dim[k] > 1 && jac_chunk(dim[k], G.jac_smem) < 1) rc = fail(c, TDMRG_EINVAL, "rho_eig: Jacobi shared memory");
     // S = W rho W^H and G = W W^H are Hermitian: lower tiles plus mirror
@@ -1010,8 +1205,10 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
     cplx* E1h = w.buf + 5 * w.nrho;
     int* n_iter = reinterpret_cast<int*>(G.fro + ns);
     const OaTables oat = oa_tables(G);
-    launch_pdl(k_seed, ns, JT, G.seed_smem, s, rho, W, G.fro, n_iter, G.flags, tb, w.gwork, G.stats);
+    cudaError_t e = launch_pdl_cluster(k_seed, G.nseed, ST, G.seed_smem, s, G.seed_cluster, rho, W, G.fro, n_iter, G.flags, tb, w.gwork,
+                                       G.stats, (const int*)G.seed_items, c->dstatus);
     c->launches += 1;
+    if (e != cudaSuccess) return e;
     GemmArgs a{};
     a.dscale = c->dscale;
     a.bufs[EB_RHO] = const_cast<cplx*>(rho);
@@ -1029,7 +1226,6 @@ cudaError_t launch_group(tdmrg_ctx* c, EigWork& w, EigGroup& G, const cplx* rho,
         return corr ? launch_gemm_corr(a, s, skip, it) : launch_gemm_f64(a, s, skip, it);
     };
     const dim3 chunks(ns, kRowChunks);
-    cudaError_t e = cudaGetLastError();
     for (; it < kMaxRefine && e == cudaSuccess; ++it) {
         a.bufs[EB_W] = W; a.bufs[EB_WN] = Wn;
         // the orthonormalisation steps need G = W W^H only (S is formed but not read, lambda stays)
@@ -1078,11 +1274,11 @@ int eig_prepare(tdmrg_ctx* c, int side) {
         w.nrho = r; w.nev = e; w.maxn = maxn; w.ns = ns;
         int rc = dev_alloc(c, (void**)&w.buf, (size_t)6 * r * sizeof(cplx), "eig workspace");
         if (!rc) rc = dev_alloc(c, (void**)&w.lam, (size_t)e * sizeof(double), "eig workspace");
-        if (!rc && maxn > kSmemMaxA) rc = dev_alloc(c, (void**)&w.gwork, (size_t)4 * r * sizeof(float2), "eig workspace");
+        if (!rc && maxn > std::min(kSmemMaxA, kSeedSmemN)) rc = dev_alloc(c, (void**)&w.gwork, (size_t)4 * r * sizeof(float2), "eig workspace");
         // the opt-in is a property of the kernel on the device, shared by every context: always the maximum
         if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, kJacSmemCap),
                                  "eig smem");
-        if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(k_seed, cudaFuncAttributeMaxDynamicSharedMemorySize, kJacSmemCap), "eig smem");
+        if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(k_seed, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kSeedSmemN * seed_ld(kSeedSmemN)), "eig smem");
         if (rc) return rc;
         // the longest Jacobi seeds on a second stream, beside the other sectors' seeds and refinement
         const std::vector<int> lng = long_sectors(L.dim);
@@ -1140,6 +1336,7 @@ void release_eig(tdmrg_ctx* c, int side) {
         dev_free(c, G.stats, (size_t)G.ns * sizeof(int2));
         dev_free(c, G.fro, ((size_t)G.ns + 1) * sizeof(double));
         dev_free(c, G.flags, (size_t)G.ns * sizeof(int));
+        dev_free(c, G.seed_items, (size_t)G.nseed * sizeof(int));
         dev_free(c, G.oa, oa_bytes(G.noa, G.ns));
     }
     dev_free(c, w.buf, (size_t)6 * w.nrho * sizeof(cplx));

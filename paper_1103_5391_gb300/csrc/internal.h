@@ -45,6 +45,27 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
+
+// the same in clusters of `cluster` CTAs
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
+                                      Args&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
 #endif
 
 // Buffer ids a segment or task refers to; the launch passes the base pointers.
@@ -277,6 +298,8 @@ struct EigGroup {
     double* fro = nullptr;      // per sector ||rho||_F, then the iteration count (int)
     int jac_smem = 0;           // dynamic shared memory of the re-seed Jacobi launch
     int seed_smem = 0;          // and of the seed launch
+    int* seed_items = nullptr;  // sector of every CTA of the seed launch (eig.cu)
+    int nseed = 0, seed_cluster = 1;
     int* flags = nullptr;       // per sector: re-seed requested by the refinement
     float4* grec = nullptr;     // Jacobi rotation records of the sectors too large for V in shared memory
     int64_t grec_entries = 0;
