@@ -1084,7 +1084,22 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
     G.nbig = (int)big.size();
     G.maxn_big = maxn_big;
     G.grec_entries = nrec_total;
-    G.tables_bytes = (size_t)ns * (3 * sizeof(int64_t) + sizeof(int)) + big.size() * sizeof(int);
+    // seed CTAs: the shared sectors first, the largest ahead, a cluster each; then one sector per CTA, clusters filled
+    std::vector<int> order(ns), items;
+    for (int k = 0; k < ns; ++k) {
+        order[k] = k;
+        if (dim[k] <= kSeedSmemN) G.seed_smem = std::max(G.seed_smem, 8 * dim[k] * seed_ld(dim[k]));
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return dim[x] > dim[y]; });
+    auto is_shared = [&](int k) { return dim[k] > kSeedClusterN && dim[k] <= kSeedSmemN; };
+    for (int k : order)
+        if (is_shared(k)) items.insert(items.end(), kSeedCluster, k + kSeedShared);
+    G.seed_cluster = items.empty() ? 1 : kSeedCluster;
+    for (int k : order)
+        if (!is_shared(k)) items.push_back(k);
+    while (items.size() % G.seed_cluster) items.push_back(-1);
+    G.nseed = (int)items.size();
+    G.tables_bytes = (size_t)ns * (3 * sizeof(int64_t) + sizeof(int)) + (big.size() + items.size()) * sizeof(int);
     int rc = dev_alloc(c, (void**)&G.tables, G.tables_bytes, "eig tables");
     if (!rc) rc = dev_alloc(c, (void**)&G.fro, ((size_t)ns + 1) * sizeof(double), "eig workspace");
     if (!rc && nrec_total) rc = dev_alloc(c, (void**)&G.grec, (size_t)nrec_total * sizeof(float4), "eig rotation record");
@@ -1099,6 +1114,9 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
     memcpy(h + 2 * ns * sizeof(int64_t), roff.data(), ns * sizeof(int64_t));
     memcpy(h + 3 * ns * sizeof(int64_t), dim.data(), ns * sizeof(int));
     if (!big.empty()) memcpy(h + 3 * ns * sizeof(int64_t) + ns * sizeof(int), big.data(), big.size() * sizeof(int));
+    int* const hi = reinterpret_cast<int*>(h + 3 * ns * sizeof(int64_t) + ns * sizeof(int)) + big.size();
+    memcpy(hi, items.data(), items.size() * sizeof(int));
+    G.seed_items = reinterpret_cast<int*>(static_cast<unsigned char*>(G.tables) + (reinterpret_cast<unsigned char*>(hi) - h));
     rc = cuda_check(c, cudaMemcpy(G.tables, host.data(), host.size(), cudaMemcpyHostToDevice), "eig tables");
     if (rc) return rc;
     {   // work items of the element-wise refinement kernels (counters start at zero)
@@ -1163,23 +1181,6 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
         smem = std::max(smem, jac_base_bytes(n) + 32 * (P / 2) * (P - 1));
     }
     G.jac_smem = std::min(smem, kJacSmemCap);
-    // seed CTAs: the shared sectors first, the largest ahead, a cluster each; then one sector per CTA, clusters filled
-    std::vector<int> order(ns), items;
-    for (int k = 0; k < ns; ++k) {
-        order[k] = k;
-        if (dim[k] <= kSeedSmemN) G.seed_smem = std::max(G.seed_smem, 8 * dim[k] * seed_ld(dim[k]));
-    }
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return dim[x] > dim[y]; });
-    auto is_shared = [&](int k) { return dim[k] > kSeedClusterN && dim[k] <= kSeedSmemN; };
-    for (int k : order)
-        if (is_shared(k)) items.insert(items.end(), kSeedCluster, k + kSeedShared);
-    G.seed_cluster = items.empty() ? 1 : kSeedCluster;
-    for (int k : order)
-        if (!is_shared(k)) items.push_back(k);
-    while (items.size() % G.seed_cluster) items.push_back(-1);
-    G.nseed = (int)items.size();
-    rc = dev_alloc(c, (void**)&G.seed_items, (size_t)G.nseed * sizeof(int), "eig seed items");
-    if (!rc) rc = cuda_check(c, cudaMemcpy(G.seed_items, items.data(), (size_t)G.nseed * sizeof(int), cudaMemcpyHostToDevice), "eig seed items");
     for (int k = 0; k < ns && !rc; ++k)
         if (dim[k] > 1 && jac_chunk(dim[k], G.jac_smem) < 1) rc = fail(c, TDMRG_EINVAL, "rho_eig: Jacobi shared memory");
     // S = W rho W^H and G = W W^H are Hermitian: lower tiles plus mirror
@@ -1341,7 +1342,6 @@ void release_eig(tdmrg_ctx* c, int side) {
         dev_free(c, G.stats, (size_t)G.ns * sizeof(int2));
         dev_free(c, G.fro, ((size_t)G.ns + 1) * sizeof(double));
         dev_free(c, G.flags, (size_t)G.ns * sizeof(int));
-        dev_free(c, G.seed_items, (size_t)G.nseed * sizeof(int));
         dev_free(c, G.oa, oa_bytes(G.noa, G.ns));
     }
     dev_free(c, w.buf, (size_t)6 * w.nrho * sizeof(cplx));

@@ -590,65 +590,111 @@ __global__ void __launch_bounds__(32) k_tridiag_exp_eq(double* __restrict__ tri,
     }
 }
 
-// Lowest eigenpair of the Lanczos tridiagonal T (ground-state targeting, Sec. II.B): one thread, FP64.
-// The eigenvalue by bisection on the Sturm count (number of eigenvalues below x from the signs of the
-// LDL^T pivots of T - x), then the eigenvector by inverse iteration (three tridiagonal solves with the
-// shifted matrix, pivots kept away from zero); coef[0][k] = x_k (normalised, real), tri[T_EMIN] = lambda.
-__global__ void __launch_bounds__(32) k_tridiag_min(double* __restrict__ tri, const int* __restrict__ flags,
-                                                     cplx* __restrict__ coef) {
+// Lowest eigenpair of the Lanczos tridiagonal T (ground-state targeting, Sec. II.B), FP64, n <= 32.
+// The eigenvalue by multisection: x lies below it exactly when the leading minors d_k = det(T_k - x) are all
+// positive, d_k = (alpha_k - x) d_{k-1} - beta_{k-1}^2 d_{k-2} with T scaled by a power of two to norm <= 1 (|d_k| <= 3^k);
+// 128 threads try 128 points of the bracket at once, so it shrinks 129-fold in one chain of n steps.  Bisection on
+// the Sturm count with divisions took ~52 chains of n FP64 divisions (~700 cycles each) in one thread: 650 us at
+// n = 32, 30 us now (bound by the FP64 pipe: three instructions a step and warp).
+// The eigenvector by the twisted factorisation of T - lambda (Dhillon 1997): pivots p_k from the top and m_k from the
+// bottom (ratios of the leading and trailing minors), the twist r where |p_k + m_k - (alpha_k - lambda)| is smallest,
+// z_r = 1, z_k = -(beta_k / p_k) z_{k+1} above and z_k = -(beta_{k-1} / m_k) z_{k-1} below: one lane per component,
+// products by scans.  coef[0][k] = z_k / |z| (real), tri[T_EMIN] = lambda.
+constexpr int kMinThreads = 128;
+__global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict__ tri, const int* __restrict__ flags,
+                                                              cplx* __restrict__ coef) {
     pdl_enter();
-    if (threadIdx.x != 0) return;
-    const int n = flags[0];
-    for (int k = 0; k < 32; ++k) coef[k] = make_double2(0.0, 0.0);
-    if (n <= 0) { tri[T_EMIN] = 0.0; return; }
-    const double* al = tri + T_ALPHA;
-    const double* be = tri + T_BETA;   // be[k] couples k and k + 1
-    double lo = 1e300, hi = -1e300;
-    for (int k = 0; k < n; ++k) {
-        const double r = (k > 0 ? fabs(be[k - 1]) : 0.0) + (k + 1 < n ? fabs(be[k]) : 0.0);
-        lo = fmin(lo, al[k] - r);
-        hi = fmax(hi, al[k] + r);
+    const int n = flags[0], tid = threadIdx.x, l = tid & 31;
+    if (tid < 32) coef[tid] = make_double2(0.0, 0.0);
+    if (n <= 0) {
+        if (tid == 0) tri[T_EMIN] = 0.0;
+        return;
     }
-    const double tiny = 1e-300;
-    for (int it = 0; it < 200 && hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) {
-        const double x = 0.5 * (lo + hi);
-        int cnt = 0;
-        double q = al[0] - x;
-        cnt += q < 0.0;
+    __shared__ double sa[32], sb2[32], sx[kMinThreads + 2], sd[2][32];
+    // every warp: alpha_l, beta_l (couples l and l + 1) and the Gershgorin interval
+    double al = l < n ? tri[T_ALPHA + l] : 0.0, be = l < n - 1 ? tri[T_BETA + l] : 0.0;
+    double bm = __shfl_up_sync(0xffffffffu, be, 1);
+    if (l == 0) bm = 0.0;
+    const double r = fabs(be) + fabs(bm);
+    double lo = l < n ? al - r : 1e300, hi = l < n ? al + r : -1e300;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    const double nrm = fmax(fabs(lo), fabs(hi));
+    int e2 = 0;
+    frexp(nrm, &e2);
+    const double sc = nrm > 0.0 ? ldexp(1.0, -e2) : 1.0, us = nrm > 0.0 ? ldexp(1.0, e2) : 1.0;
+    al *= sc; be *= sc; bm *= sc; lo *= sc; hi *= sc;
+    if (tid < 32) { sa[l] = al; sb2[l] = be * be; }
+    __syncthreads();
+    for (int it = 0; it < 12 && hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) {
+        const double x = fma(hi - lo, (tid + 1) * (1.0 / (kMinThreads + 1)), lo);
+        double d0 = 1.0, d1 = sa[0] - x;
+        bool below = d1 > 0.0;
         for (int k = 1; k < n; ++k) {
-            if (q == 0.0) q = tiny;
-            q = al[k] - x - be[k - 1] * be[k - 1] / q;
-            cnt += q < 0.0;
+            const double d2 = fma(sa[k] - x, d1, -sb2[k - 1] * d0);
+            d0 = d1;
+            d1 = d2;
+            below = below && d2 > 0.0;
         }
-        if (cnt >= 1) hi = x;
-        else lo = x;
+        sx[tid + 1] = x;
+        if (tid == 0) { sx[0] = lo; sx[kMinThreads + 1] = hi; }
+        const int c = __syncthreads_count(below);   // points below the eigenvalue: the first c of them
+        lo = sx[c];
+        hi = sx[c + 1];
+        __syncthreads();
     }
+    if (tid >= 32) return;
     const double lam = 0.5 * (lo + hi);
-    // a pivot that vanishes (lam an exact eigenvalue, e.g. n = 1 when the start vector is already an
-    // eigenvector) is replaced by eps ||T||; each solve is rescaled by its largest entry before the norm
-    const double pmin = 2.2e-16 * fmax(fmax(fabs(lo), fabs(hi)), 1e-300);
-    double v[32], dg[32], up[32];
-    for (int k = 0; k < n; ++k) v[k] = 1.0;
-    for (int r = 0; r < 3; ++r) {   // (T - lam) y = v by elimination down the band, then back substitution
-        for (int k = 0; k < n; ++k) { dg[k] = al[k] - lam; up[k] = k + 1 < n ? be[k] : 0.0; }
+    if (l < 2) {   // lane 0: leading minors, lane 1: trailing minors of T - lambda
+        double d0 = 1.0, d1 = sa[l == 0 ? 0 : n - 1] - lam;
+        sd[l][l == 0 ? 0 : n - 1] = d1;
         for (int k = 1; k < n; ++k) {
-            if (fabs(dg[k - 1]) < pmin) dg[k - 1] = dg[k - 1] < 0.0 ? -pmin : pmin;
-            const double m = be[k - 1] / dg[k - 1];
-            dg[k] -= m * up[k - 1];
-            v[k] -= m * v[k - 1];
+            const int i = l == 0 ? k : n - 1 - k;
+            const double d2 = fma(sa[i] - lam, d1, -sb2[l == 0 ? k - 1 : i] * d0);
+            d0 = d1;
+            d1 = d2;
+            sd[l][i] = d1;
         }
-        if (fabs(dg[n - 1]) < pmin) dg[n - 1] = dg[n - 1] < 0.0 ? -pmin : pmin;
-        v[n - 1] /= dg[n - 1];
-        for (int k = n - 2; k >= 0; --k) v[k] = (v[k] - up[k] * v[k + 1]) / dg[k];
-        double mx = 0.0;
-        for (int k = 0; k < n; ++k) mx = fmax(mx, fabs(v[k]));
-        double nn = 0.0;
-        for (int k = 0; k < n; ++k) { v[k] /= mx; nn += v[k] * v[k]; }
-        const double inv = 1.0 / sqrt(nn);
-        for (int k = 0; k < n; ++k) v[k] *= inv;
     }
-    for (int k = 0; k < n; ++k) coef[k] = make_double2(v[k], 0.0);
-    tri[T_EMIN] = lam;
+    __syncwarp();
+    // a pivot that vanishes (lambda an eigenvalue of a leading or trailing block too, or n = 1) is replaced by eps ||T||
+    constexpr double pmin = 2.2e-16;
+    auto pivot = [&](double d, double prev) {
+        const double q = prev != 0.0 ? d / prev : d;
+        return fabs(q) < pmin ? (q < 0.0 ? -pmin : pmin) : q;
+    };
+    const bool in = l < n;
+    const double p = in ? pivot(sd[0][l], l > 0 ? sd[0][l - 1] : 1.0) : 1.0;
+    const double m = in ? pivot(sd[1][l], l < n - 1 ? sd[1][l + 1] : 1.0) : 1.0;
+    double g = in ? fabs(p + m - (al - lam)) : 1e300;
+    int tw = l;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {   // the smallest, ties to the first
+        const double og = __shfl_xor_sync(0xffffffffu, g, o);
+        const int ot = __shfl_xor_sync(0xffffffffu, tw, o);
+        if (og < g || (og == g && ot < tw)) { g = og; tw = ot; }
+    }
+    double up = l < tw ? -be / p : 1.0;                 // z_l = product of up over l .. tw - 1
+    double dn = in && l > tw ? -bm / m : 1.0;           // z_l = product of dn over tw + 1 .. l
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_down_sync(0xffffffffu, up, o), d = __shfl_up_sync(0xffffffffu, dn, o);
+        if (l + o < 32) up *= u;
+        if (l >= o) dn *= d;
+    }
+    const double z = in ? (l < tw ? up : dn) : 0.0;
+    double mx = fabs(z);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const double zs = z / mx;   // mx >= |z_tw| = 1
+    double nn = zs * zs;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
+    if (in) coef[l] = make_double2(zs / sqrt(nn), 0.0);
+    if (l == 0) tri[T_EMIN] = lam * us;
 }
 
 struct TargetPtrs { cplx* p[16]; };
@@ -966,7 +1012,7 @@ int ground_state(tdmrg_ctx* c, int a, int b, cplx* psi, int nk, int restarts, do
     for (int r = 0; r < restarts; ++r) {
         int rc = lanczos_build(c, a, b, psi, nk, &k);
         if (rc) return rc;
-        launch_pdl(k_tridiag_min, 1, 32, 0, c->stream, k->tri, k->flags, k->coef);
+        launch_pdl(k_tridiag_min, 1, kMinThreads, 0, c->stream, k->tri, k->flags, k->coef);
         TargetPtrs tg{};
         tg.p[0] = psi;
         const int grid = (int)std::min<int64_t>((k->n + 255) / 256, 4L * c->num_sms);
