@@ -382,9 +382,9 @@ int tdmrg_overlap_op(tdmrg_ctx* ctx, int opL, int opR, int n_up1, int n_dn1, con
  *   out_d[i * nR + j] = <phi1| opL[i] opR[j] |phi2>   (not normalised), i < nL, j < nR,
  * each product with the fermion sign of tdmrg_apply_op (-1 = identity on that block, not both in one
  * product); phi2_d lives in sector Q2 = (n_up2, n_dn2) and every product must map it to Q1 =
- * (n_up1, n_dn1), the sector of phi1_d.  out_d: nL * nR device tdmrg_c64.  The whole grid runs as two
- * grouped FP64 launches into library-owned scratch (nL * nR vectors of sector Q1 plus the
- * intermediates) and one fixed-order reduction per entry.  The plan and scratch are built by the first
+ * (n_up1, n_dn1), the sector of phi1_d.  out_d: nL * nR device tdmrg_c64.  The whole grid runs as one
+ * grouped FP64 launch of nL + nR products into library-owned vectors (A_i^dag phi1 and phi2 B_j^T, nL + nR
+ * of them) and one fixed-order reduction per entry.  The plan and vectors are built by the first
  * call for a given (operator lists, sectors), which allocates and synchronises; later calls do neither
  * and may be captured in a CUDA graph.  Errors: EINVAL, ESTATE, ESECTOR, ENOMEM, ECUDA. */
 int tdmrg_correlation(tdmrg_ctx* ctx, int nL, const int32_t* opL, int nR, const int32_t* opR, int n_up1, int n_dn1,

@@ -232,15 +232,17 @@ struct Plan {
     TaskList thin[2];
 };
 
-// The correlation grid <phi1| A_i B_j |phi2>: every product of the grid compiled into one pair of task
-// lists (stage 1 into per-product scratch, stage 2 into per-product output vectors W_ij), then dots.
+// The correlation grid <phi1| A_i B_j |phi2> (correlation.cu): the products Z_i and T_j on a common block list as one
+// task list, copies for identity operators, then dots.
+struct CorrCopy { int64_t src, dst, len; int32_t right; };
 struct CorrPlan {
-    TaskList s1, s2;
-    int npairs = 0;
-    int64_t n1 = 0, scratch = 0;
-    cplx* T = nullptr;          // stage-1 intermediates of all products
-    cplx* W = nullptr;          // npairs vectors of sector Q1
-    double2* part = nullptr;    // dot partials, npairs x kCorrChunks
+    TaskList tl;
+    int nL = 0, nR = 0, ncopies = 0;
+    int64_t n = 0;              // entries of one Z_i or T_j
+    cplx* Z = nullptr;          // nL vectors A_i^dag phi1
+    cplx* T = nullptr;          // nR vectors +-phi2 B_j^T
+    CorrCopy* copies = nullptr;
+    double2* part = nullptr;    // dot partials, nL nR x kCorrChunks
 };
 constexpr int kCorrChunks = 32;
 
@@ -415,7 +417,7 @@ void dev_free(tdmrg_ctx* c, void* p, size_t bytes);
 
 // plan.cu
 int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qin0, int qin1, int qout0, int qout1,
-               Plan* out, bool to_device = true);
+               Plan* out);
 int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn);
 void make_tiles(TaskList& tl);
 void make_corr_tiles(TaskList& tl, int ksplit);

@@ -217,7 +217,7 @@ std::vector<PairInfo> pairs_of(const tdmrg_ctx* c, int a, int b) {
 
 }  // namespace
 
-int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int oa, int ob, Plan* p, bool to_device) {
+int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int oa, int ob, Plan* p) {
     const Side& L = c->side[0];
     p->qin[0] = qa; p->qin[1] = qb; p->qout[0] = oa; p->qout[1] = ob;
     std::vector<PairInfo> pin = pairs_of(c, qa, qb), pout = pairs_of(c, oa, ob);
@@ -336,7 +336,6 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
     make_tiles(s2);
     p->scratch = scr;
     p->flops = s1.flops + s2.flops;
-    if (!to_device) return TDMRG_OK;   // host task lists only (merged into a larger launch by the caller)
     int urc = upload(c, s1);
     if (!urc) urc = upload(c, s2);
     if (urc) return urc;
