@@ -182,8 +182,8 @@ int tdmrg_create(tdmrg_ctx** out, const tdmrg_opts* o) {
     cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, o->device);
     int rc = dev_alloc(c, (void**)&c->red, 2 * 64 * kRedBlocks * sizeof(double2), "reduction workspace");
     if (!rc) rc = dev_alloc(c, (void**)&c->dscale, 64 * sizeof(double), "scale workspace");
-    if (!rc) rc = dev_alloc(c, (void**)&c->dstatus, sizeof(int), "status word");
-    if (!rc) rc = cuda_check(c, cudaMemset(c->dstatus, 0, sizeof(int)), "status word");
+    if (!rc) rc = dev_alloc(c, (void**)&c->dstatus, 32 * sizeof(int), "status word");
+    if (!rc) rc = cuda_check(c, cudaMemset(c->dstatus, 0, 32 * sizeof(int)), "status word");
     if (rc) {
         g_err = c->err;
         tdmrg_destroy(c);
@@ -207,8 +207,8 @@ int tdmrg_destroy(tdmrg_ctx* c) {
     dev_free(c, c->red, 2 * 64 * kRedBlocks * sizeof(double2));
     dev_free(c, c->dsum_dscale, c->dsum_dscale_bytes);
     dev_free(c, c->dscale, 64 * sizeof(double));
-    dev_free(c, c->dstatus, sizeof(int));
-    dev_free(c, c->trunc_tables, c->trunc_tables_bytes);
+    dev_free(c, c->dstatus, 32 * sizeof(int));
+    for (auto& t : c->trunc) dev_free(c, t.d, t.bytes);
     delete c;
     return TDMRG_OK;
 }
@@ -253,6 +253,7 @@ int tdmrg_set_block(tdmrg_ctx* c, int side, int nsec, const int32_t* qn, const i
     DeviceGuard g(c->opts.device);
     cudaStreamSynchronize(c->stream);
     release_eig(c, side);
+    c->trunc[side].valid = false;
     c->side[side] = s;
     c->ops[side].clear();
     c->dsum_src[0].clear();

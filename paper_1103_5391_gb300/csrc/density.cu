@@ -20,16 +20,43 @@ constexpr int NB = kRedBlocks;
 
 struct Weights { double w[12]; };
 
-__global__ void k_weight_scale(const double2* __restrict__ part, int nt, double* __restrict__ dscale, Weights ws) {
+// dscale[l] = w_l / ||psi_l||^2 (0 for a zero state) for all targets in one launch: block (b, l) sums a chunk of target l,
+// the last block of a target (ticket) the chunks in order, one warp.  One norm launch per target and one for the
+// scales were six launches of ~5 us each.
+struct NormList { const cplx* p[12]; int64_t n[12]; int nb[12]; };
+__global__ void __launch_bounds__(256) k_weight_scale(NormList nl, double* __restrict__ part, int* __restrict__ tickets,
+                                                      double* __restrict__ dscale, Weights ws) {
     pdl_enter();
-    // one warp per target: dscale[l] = w_l / ||psi_l||^2 (0 for a zero state)
-    const int l = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (l >= nt) return;
+    const int l = blockIdx.y, nb = nl.nb[l];
+    if ((int)blockIdx.x >= nb) return;
+    __shared__ double sh[8];
+    __shared__ int last;
+    const int64_t ch = (nl.n[l] + nb - 1) / nb, lo = min(nl.n[l], (int64_t)blockIdx.x * ch), hi = min(nl.n[l], lo + ch);
+    const cplx* __restrict__ x = nl.p[l];
     double s = 0.0;
-    for (int b = lane; b < NB; b += 32) s += part[(int64_t)l * NB + b].x;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += 256) { const double2 v = x[i]; s = fma(v.x, v.x, fma(v.y, v.y, s)); }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) dscale[l] = s > 0.0 ? ws.w[l] / s : 0.0;
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += sh[k];
+        part[l * NB + blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(tickets + l, 1) == nb - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    s = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 32) s += __ldcg(part + l * NB + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) {
+        dscale[l] = s > 0.0 ? ws.w[l] / s : 0.0;
+        tickets[l] = 0;   // ready for the next launch
+    }
 }
 
 // Real-basis variant: Re rho_L = sum_l w_l (Re Psi_l Re Psi_l^T + Im Psi_l Im Psi_l^T) / <psi_l|psi_l>, the
@@ -130,15 +157,16 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
     } else {
         // norms of the targets -> dscale[l] = w_l / ||psi_l||^2; partials in the upper half of the reduction
         // workspace, apart from those of tdmrg_expect / tdmrg_overlap_op (which may run beside on another stream)
-        double2* nred = c->red + 64 * (int64_t)NB;
+        NormList nl{};
+        int gx = 1;
         for (int l = 0; l < nt; ++l) {
-            const int64_t nl = sector_size(c, Q[2 * l], Q[2 * l + 1]);
-            if (nl == 0) return fail(c, TDMRG_ESECTOR, "density_matrix: target in an empty sector");
-            cudaError_t e = launch_norm2(psi[l], nl, nred + (int64_t)l * NB, NB, s);
-            c->launches++;
-            if (e != cudaSuccess) return cuda_check(c, e, "density_matrix norms");
+            nl.p[l] = psi[l];
+            nl.n[l] = sector_size(c, Q[2 * l], Q[2 * l + 1]);
+            if (nl.n[l] == 0) return fail(c, TDMRG_ESECTOR, "density_matrix: target in an empty sector");
+            nl.nb[l] = (int)std::min<int64_t>((nl.n[l] + 1023) / 1024, NB);   // four elements a thread while the blocks last
+            gx = std::max(gx, nl.nb[l]);
         }
-        launch_pdl(k_weight_scale, 1, 32 * 12, 0, s, nred, nt, c->dscale, wl);
+        launch_pdl(k_weight_scale, dim3(gx, nt), 256, 0, s, nl, (double*)(c->red + 64 * (int64_t)NB), c->dstatus + 16, c->dscale, wl);
         c->launches++;
     }
     // task list: one task per sector of the side, compiled once per (side, set of target sectors, order);

@@ -385,12 +385,12 @@ struct tdmrg_ctx {
     int schedule = -1;             // tile schedule of the persistent tensor kernel: -1 autotuned, 0 static, 1 queue
     int tile_m = 0;                // tile M of the persistent tensor kernel: 0 autotuned, 64, 128
     int orth_per_sm = 0;           // blocks per SM of the cooperative orthogonalisation (0: the default)
-    void* trunc_tables = nullptr;  // sector tables of tdmrg_truncate
-    size_t trunc_tables_bytes = 0;
+    struct TruncTables { void* d = nullptr; size_t bytes = 0; bool valid = false; int64_t nev = 0; };
+    TruncTables trunc[2];          // per side: sector tables of tdmrg_truncate
     int thin_dim = 12;
     int real_basis = 0;            // tdmrg_density_matrix forms Re rho_L (targets' real and imaginary parts apart)
     const tdmrg::cplx* dcoef = nullptr;   // caller's device array of connection coefficients (null: static)             // tensor path: sector products with min(M, N) below this run on FP64 warps
-    int* dstatus = nullptr;        // device word: bit 0 set when a bounded device wait ran out
+    int* dstatus = nullptr;        // device word: nonzero when a bounded device wait ran out; 16 tickets follow at +16
     tdmrg::EigWork eig[2];         // per side (rho_L, rho_R)
 };
 
@@ -452,7 +452,6 @@ int ground_state(tdmrg_ctx* c, int n_up, int n_dn, cplx* psi, int nk, int restar
 int evolve_segments(tdmrg_ctx* c, int n_up, int n_dn, const cplx* phi, int nseg, const int64_t* seg_len, int n_v,
                     const double* t_x, int nk, cplx* const* targets);
 int segments_info(tdmrg_ctx* c, int n_up, int n_dn, int nk, int nseg, int* nk_used, double* err);
-cudaError_t launch_norm2(const cplx* x, int64_t n, double2* partials, int nblk, cudaStream_t s);
 cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* partials, int nblk,
                              cplx* out, int normalise, cudaStream_t s);
 constexpr int kRedBlocks = 304;   // 2 x 152 SMs: fixed, so reductions are deterministic

@@ -909,12 +909,6 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
 
 }  // namespace
 
-cudaError_t launch_norm2(const cplx* x, int64_t n, double2* partials, int nblk, cudaStream_t s) {
-    (void)nblk;
-    launch_pdl(k_norm2, NB, NT, 0, s, x, n, partials);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* partials, int nblk, cplx* out,
                              int normalise, cudaStream_t s) {
     (void)nblk;
