@@ -268,7 +268,7 @@ int tdmrg_truncate_side(tdmrg_ctx* ctx, int side, const double* evals_d, int m, 
  * (the layout of tdmrg_rho_eig); kept (host, one int per sector of that side) the kept counts k(q).
  * out_d (device) receives, for every block of the operator in the order it was set whose two kept
  * counts are nonzero, the k(q_out) x k(q_in) block row-major, concatenated; *nblk_out (host, nullable)
- * their number.  FP64 grouped products; allocates a scratch buffer and synchronises the stream.
+ * their number.  FP64 grouped products; scratch from a buffer the context keeps; synchronises the stream.
  * Errors: EINVAL (unknown op id, kept count outside 0..dim), ESTATE, ENOMEM, ECUDA. */
 int tdmrg_renormalize_op(tdmrg_ctx* ctx, int side, int op_id, const tdmrg_c64* U_d, const int32_t* kept,
                          tdmrg_c64* out_d, int* nblk_out);
@@ -353,7 +353,7 @@ int tdmrg_set_op_adjoint(tdmrg_ctx* ctx, int side, int op_id, int src_id);
  *
  * psi_d: the target in `from`'s sector Q = (n_up, n_dn); out_d: the result in `to`'s sector Q (cleared
  * first).  No fermion sign arises (the moved site keeps its place in the lattice order).  Two grouped FP64
- * launches on `from`'s stream; allocates scratch and synchronises.  Errors: EINVAL (null, kept counts
+ * launches on `from`'s stream; scratch from a buffer the context keeps; synchronises.  Errors: EINVAL (null, kept counts
  * outside 0..dim), ESTATE, ESECTOR (the block tables do not match the move), ENOMEM, ECUDA. */
 int tdmrg_wft_right(tdmrg_ctx* from, int n_up, int n_dn, const tdmrg_c64* psi_d, const tdmrg_c64* U_d,
                     const int32_t* kept, const tdmrg_c64* V_d, const int32_t* kept_next, tdmrg_ctx* to,

@@ -31,9 +31,16 @@ int cuda_check(tdmrg_ctx* c, cudaError_t e, const char* what) {
 int dev_alloc(tdmrg_ctx* c, void** p, size_t bytes, const char* what) {
     *p = nullptr;
     if (bytes == 0) return TDMRG_OK;
-    if (c->opts.hbm_budget && c->allocated + bytes > c->opts.hbm_budget)
-        return fail(c, TDMRG_ENOMEM, std::string(what) + ": HBM budget exceeded");
-    cudaError_t e = cudaMalloc(p, bytes);
+    const bool over = c->opts.hbm_budget && c->allocated + bytes > c->opts.hbm_budget;
+    cudaError_t e = over ? cudaSuccess : cudaMalloc(p, bytes);
+    if ((over || e != cudaSuccess) && c->transient) {   // give the transient buffer back (idle between calls) and try again
+        if (e != cudaSuccess) cudaGetLastError();
+        dev_free(c, c->transient, c->transient_bytes);
+        c->transient = nullptr;
+        c->transient_bytes = 0;
+        return dev_alloc(c, p, bytes, what);
+    }
+    if (over) return fail(c, TDMRG_ENOMEM, std::string(what) + ": HBM budget exceeded");
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -209,6 +216,7 @@ int tdmrg_destroy(tdmrg_ctx* c) {
     dev_free(c, c->dscale, 64 * sizeof(double));
     dev_free(c, c->dstatus, 32 * sizeof(int));
     for (auto& t : c->trunc) dev_free(c, t.d, t.bytes);
+    dev_free(c, c->transient, c->transient_bytes);
     delete c;
     return TDMRG_OK;
 }

@@ -392,6 +392,8 @@ struct tdmrg_ctx {
     const tdmrg::cplx* dcoef = nullptr;   // caller's device array of connection coefficients (null: static)             // tensor path: sector products with min(M, N) below this run on FP64 warps
     int* dstatus = nullptr;        // device word: nonzero when a bounded device wait ran out; 16 tickets follow at +16
     tdmrg::EigWork eig[2];         // per side (rho_L, rho_R)
+    void* transient = nullptr;     // task lists and scratch of calls that do not keep a plan (run_transient)
+    size_t transient_bytes = 0;
 };
 
 namespace tdmrg {
@@ -423,6 +425,9 @@ void make_tiles(TaskList& tl);
 void make_corr_tiles(TaskList& tl, int ksplit);
 int upload(tdmrg_ctx* c, TaskList& tl);
 void release(tdmrg_ctx* c, TaskList& tl);
+// The task lists (tiles made, not uploaded) run one after another on c->stream with g's buffers, `scratch` complex entries
+// as BUF_SCRATCH, from the context's transient buffer; synchronises the stream.
+int run_transient(tdmrg_ctx* c, TaskList* const* lists, int nlists, int64_t scratch, GemmArgs g, const char* what);
 int run_plan(tdmrg_ctx* c, const Plan& p, const cplx* in, cplx* out, const int* skip_flag, int skip_step);
 
 // gemm_f64.cu: grouped complex FP64 GEMM (one output per lane), and the correction C = (I + A) B with A B in FP32

@@ -54,6 +54,57 @@ void release(tdmrg_ctx* c, TaskList& tl) {
     tl.d_tasks = nullptr; tl.d_segs = nullptr; tl.d_tiles = nullptr; tl.d_ctiles = nullptr; tl.d_partials = nullptr; tl.d_counters = nullptr;
 }
 
+int run_transient(tdmrg_ctx* c, TaskList* const* lists, int nlists, int64_t scratch, GemmArgs g, const char* what) {
+    // one device buffer: scratch | per list: tasks, segments, tiles | tickets | partial sums.  It stays with the context
+    // (grown when a call needs more), so that a call costs one copy and no allocation; dev_alloc gives it back
+    // when memory runs out.  One copy per call from a host image of the tables and zeroed tickets.
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    struct Off { size_t tasks, segs, tiles, tick, part; };
+    std::vector<Off> off(nlists);
+    const size_t b_scr = al((size_t)scratch * sizeof(cplx));
+    size_t pos = b_scr;
+    for (int k = 0; k < nlists; ++k) {
+        off[k].tasks = pos; pos += al(lists[k]->tasks.size() * sizeof(Task));
+        off[k].segs = pos; pos += al(lists[k]->segs.size() * sizeof(Seg));
+        off[k].tiles = pos; pos += al(lists[k]->tiles.size() * sizeof(Tile));
+        off[k].tick = pos; pos += al((size_t)lists[k]->nsplit * sizeof(int));
+    }
+    const size_t b_tab = pos - b_scr;
+    for (int k = 0; k < nlists; ++k) { off[k].part = pos; pos += al((size_t)lists[k]->npartial * sizeof(cplx)); }
+    if (c->transient_bytes < pos) {
+        dev_free(c, c->transient, c->transient_bytes);
+        c->transient = nullptr;
+        c->transient_bytes = 0;
+        int rc = dev_alloc(c, &c->transient, pos, what);
+        if (rc) return rc;
+        c->transient_bytes = pos;
+    }
+    unsigned char* base = static_cast<unsigned char*>(c->transient);
+    std::vector<unsigned char> host(b_tab, 0);
+    for (int k = 0; k < nlists; ++k) {
+        const TaskList& tl = *lists[k];
+        if (!tl.tasks.empty()) memcpy(host.data() + off[k].tasks - b_scr, tl.tasks.data(), tl.tasks.size() * sizeof(Task));
+        if (!tl.segs.empty()) memcpy(host.data() + off[k].segs - b_scr, tl.segs.data(), tl.segs.size() * sizeof(Seg));
+        if (!tl.tiles.empty()) memcpy(host.data() + off[k].tiles - b_scr, tl.tiles.data(), tl.tiles.size() * sizeof(Tile));
+    }
+    int rc = b_tab ? cuda_check(c, cudaMemcpyAsync(base + b_scr, host.data(), b_tab, cudaMemcpyHostToDevice, c->stream), what) : TDMRG_OK;
+    g.bufs[BUF_SCRATCH] = reinterpret_cast<cplx*>(base);
+    for (int k = 0; k < nlists && !rc; ++k) {
+        if (lists[k]->tiles.empty()) continue;
+        g.tasks = reinterpret_cast<const Task*>(base + off[k].tasks);
+        g.segs = reinterpret_cast<const Seg*>(base + off[k].segs);
+        g.tiles = reinterpret_cast<const Tile*>(base + off[k].tiles);
+        g.ntiles = (int)lists[k]->tiles.size();
+        g.counters = reinterpret_cast<int*>(base + off[k].tick);
+        g.partials = reinterpret_cast<cplx*>(base + off[k].part);
+        c->launches++;
+        rc = cuda_check(c, launch_gemm_f64(g, c->stream, nullptr, 0), what);
+    }
+    // the products are done before the buffer and the host image are used again
+    const int rc2 = cuda_check(c, cudaStreamSynchronize(c->stream), what);
+    return rc ? rc : rc2;
+}
+
 int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
     const Side& L = c->side[0];
     const Side& R = c->side[1];

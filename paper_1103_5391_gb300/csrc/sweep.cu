@@ -92,34 +92,16 @@ int run_stages(tdmrg_ctx* from, TaskList& s1, TaskList& s2, int64_t scr, const t
     DeviceGuard g(from->opts.device);
     make_tiles(s1);
     make_tiles(s2);
-    cplx* P1 = nullptr;
-    const size_t sb = (size_t)std::max<int64_t>(scr, 1) * sizeof(cplx);
-    int rc = dev_alloc(from, (void**)&P1, sb, "wft scratch");
-    if (!rc) rc = upload(from, s1);
-    if (!rc) rc = upload(from, s2);
-    if (!rc) rc = cuda_check(from, cudaMemsetAsync(out, 0, (size_t)nout * sizeof(cplx), from->stream), "wft clear");
-    if (!rc) {
-        GemmArgs ga{};
-        ga.bufs[BUF_IN] = (cplx*)psi;
-        ga.bufs[BUF_SCRATCH] = P1;
-        ga.bufs[BUF_OUT] = (cplx*)out;
-        ga.bufs[BU] = (cplx*)U;
-        ga.bufs[BV] = (cplx*)V;
-        ga.dscale = from->dscale;
-        for (TaskList* tl : {&s1, &s2}) {
-            if (tl->tiles.empty()) continue;
-            ga.tasks = tl->d_tasks; ga.segs = tl->d_segs; ga.tiles = tl->d_tiles; ga.ntiles = (int)tl->tiles.size();
-            ga.partials = tl->d_partials; ga.counters = tl->d_counters;
-            from->launches++;
-            rc = cuda_check(from, launch_gemm_f64(ga, from->stream, nullptr, 0), "wft launch");
-            if (rc) break;
-        }
-    }
-    const int rc2 = cuda_check(from, cudaStreamSynchronize(from->stream), "wft");
-    release(from, s1);
-    release(from, s2);
-    dev_free(from, P1, sb);
-    return rc ? rc : rc2;
+    int rc = cuda_check(from, cudaMemsetAsync(out, 0, (size_t)nout * sizeof(cplx), from->stream), "wft clear");
+    if (rc) return rc;
+    GemmArgs ga{};
+    ga.bufs[BUF_IN] = (cplx*)psi;
+    ga.bufs[BUF_OUT] = (cplx*)out;
+    ga.bufs[BU] = (cplx*)U;
+    ga.bufs[BV] = (cplx*)V;
+    ga.dscale = from->dscale;
+    TaskList* const lists[2] = {&s1, &s2};
+    return run_transient(from, lists, 2, std::max<int64_t>(scr, 1), ga, "wft");
 }
 
 Seg seg(int64_t a_off, int8_t a_buf, int lda, int opa, int64_t b_off, int8_t b_buf, int ldb, int8_t opb, int K) {

@@ -270,30 +270,13 @@ extern "C" int tdmrg_renormalize_op(tdmrg_ctx* c, int side, int op_id, const tdm
     if (prev != c->opts.device) cudaSetDevice(c->opts.device);
     make_tiles(s1);
     make_tiles(s2);
-    cplx* T = nullptr;
-    int rc = dev_alloc(c, (void**)&T, (size_t)scr * sizeof(cplx), "renormalisation scratch");
-    if (!rc) rc = upload(c, s1);
-    if (!rc) rc = upload(c, s2);
-    if (!rc) {
-        GemmArgs g{};
-        g.bufs[BUF_OPS] = c->pool;
-        g.bufs[BUF_IN] = (cplx*)U;
-        g.bufs[BUF_SCRATCH] = T;
-        g.bufs[BUF_OUT] = (cplx*)out;
-        g.dscale = c->dscale;
-        for (TaskList* tl : {&s1, &s2}) {
-            g.tasks = tl->d_tasks; g.segs = tl->d_segs; g.tiles = tl->d_tiles; g.ntiles = (int)tl->tiles.size();
-            g.partials = tl->d_partials; g.counters = tl->d_counters;
-            c->launches++;
-            rc = cuda_check(c, launch_gemm_f64(g, c->stream, nullptr, 0), "renormalisation launch");
-            if (rc) break;
-        }
-    }
-    // the task lists and the scratch are released once the products are done
-    int rc2 = cuda_check(c, cudaStreamSynchronize(c->stream), "renormalisation");
-    release(c, s1);
-    release(c, s2);
-    dev_free(c, T, (size_t)scr * sizeof(cplx));
+    GemmArgs g{};
+    g.bufs[BUF_OPS] = c->pool;
+    g.bufs[BUF_IN] = (cplx*)U;
+    g.bufs[BUF_OUT] = (cplx*)out;
+    g.dscale = c->dscale;
+    TaskList* const lists[2] = {&s1, &s2};
+    const int rc = run_transient(c, lists, 2, scr, g, "renormalisation");
     if (prev >= 0 && prev != c->opts.device) cudaSetDevice(prev);
-    return rc ? rc : rc2;
+    return rc;
 }
