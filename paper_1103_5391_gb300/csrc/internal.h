@@ -280,12 +280,13 @@ struct KrylovWork {     // device workspace of tdmrg_evolve for one (Q, nk)
     double* tri = nullptr;      // alpha[32], beta[32], beta0, resid, err
     int* flags = nullptr;       // n_used
     cplx* coef = nullptr;       // [x][k] Krylov coefficients
-    unsigned* bar = nullptr;    // grid barrier of the fused orthogonalisation
-    int orth_grid = 0;
+    unsigned* bar = nullptr;    // ticket of the tridiagonal exponential
+    int orth_grid = 0, orth_per_sm = 1;   // blocks of the fused orthogonalisation at most
     // segmented mode (independent problems side by side in one vector): per-segment tridiagonals, flags
     // and coefficients, and the CTA partition of the vector, in one device allocation
     int nseg = 0;
     std::vector<int64_t> seg_len;
+    int64_t seg_emax = 1;       // elements of a CTA at most
     void* segmem = nullptr;
     size_t segmem_bytes = 0;
 };

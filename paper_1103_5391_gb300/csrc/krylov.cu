@@ -24,7 +24,7 @@ namespace {
 
 constexpr int NB = kRedBlocks;   // reduction blocks
 constexpr int kCoefWords = (16 + 32) * 32;   // Krylov coefficients of 16 targets + step exponential columns
-constexpr int kBarWords = 4;                  // grid barrier counter, exponential ticket
+constexpr int kBarWords = 4;                  // exponential ticket in word 2
 constexpr int NT = 256;          // threads per reduction block
 enum { T_ALPHA = 0, T_BETA = 32, T_BETA0 = 64, T_RESID = 65, T_ERR = 66, T_EMIN = 67 };
 
@@ -88,10 +88,24 @@ __global__ void __launch_bounds__(NT) k_norm2(const cplx* __restrict__ x, int64_
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
+// The partial-sum slots of the orthogonalisation steps, emptied before a Lanczos run (rows of grid blocks: the first
+// pass's two, then both buffers of the second pass's).
+struct OrthSlots { double2 *partA, *partB0, *partB1; int rows, grid; };
+__device__ __forceinline__ void clear_slots(const OrthSlots& sl) {
+    const double e = __longlong_as_double(0x7ff4dead7ff4deadll);
+    const int n = sl.rows * sl.grid;
+    for (int i = blockIdx.x * NT + threadIdx.x; i < n; i += gridDim.x * NT) {
+        sl.partB0[i] = make_double2(e, e);
+        sl.partB1[i] = make_double2(e, e);
+        if (i < 2 * sl.grid) sl.partA[i] = make_double2(e, e);
+    }
+}
+
 __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, int64_t n, const double2* __restrict__ part,
                                                  cplx* __restrict__ v0, double* __restrict__ tri, int* __restrict__ flags,
-                                                 int nk) {
+                                                 int nk, OrthSlots slots) {
     pdl_enter();
+    clear_slots(slots);
     __shared__ double2 h[1];
     reduce_coeffs(part, 1, h);
     const double b0 = sqrt(h[0].x);
@@ -107,17 +121,35 @@ __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, in
 }
 
 // ---- one Lanczos orthogonalisation step in a single cooperative launch -----------------------
-// Two grid barriers separate: (A) the first-pass dots h1_k = <v_k|w>; (B) w' = w - sum h1_k v_k, the
-// second-pass dots h2_k = <v_k|w'> and ||w'||^2; (C) beta = ||w' - sum h2_k v_k|| and
+// Two exchanges of partial sums between all blocks separate: (A) the first-pass dots h1_k = <v_k|w>; (B) w' = w -
+// sum h1_k v_k, the second-pass dots h2_k = <v_k|w'> and ||w'||^2; (C) beta = ||w' - sum h2_k v_k|| and
 // v_{j+1} = (w' - sum h2_k v_k) / beta.  Since h2 holds the projections of w' on orthonormal v_k,
 // ||w' - sum h2_k v_k||^2 = ||w'||^2 - sum |h2_k|^2 (h2 is at rounding level after the first pass, so
-// the difference loses nothing), which saves the barrier of a separate norm pass.  Every block
-// reduces the partials of all blocks in the same fixed order, so results do not depend on
-// scheduling.  FP64 throughput per SM is low on this GPU, so the warp reductions are
-// reduce-scatter (16 FP64 adds for 16 values instead of 80).  The barrier spins are bounded: when one
-// runs out the kernel sets a status bit and finishes.
+// the difference loses nothing), which saves the exchange of a separate norm pass.  Every block
+// reduces the partials of all blocks in the same fixed order, so results do not depend on scheduling.
+//
+// What bounds it is FP64 issue (a warp-wide FP64 instruction holds a sub-partition ~64 cycles) and, for short vectors,
+// the chain of latencies.  Hence:
+//   - the block's slices of w and of the newest Krylov vectors come into shared memory by bulk copies issued at the
+//     start and are read from there by all three passes (what does not fit is read from global memory);
+//   - blocks own whole multiples of 128 elements (four warps' worth, one per sub-partition), no more blocks than that
+//     gives: fewer partials for every block to sum;
+//   - the second-pass dots are split over the warps by vector, not by element: a warp's five FP64 shuffle-adds then serve
+//     all of the block's elements, and no cross-warp sum follows;
+//   - a partial sum is its own flag: its slot holds a NaN pattern that no arithmetic produces until the block stores the
+//     value, and readers poll the values themselves.  Against a counter barrier this saves the arrival's round trip
+//     twice.  Slots are cleared a phase later, when every block is known to have read them.
+// Polls are bounded: when one runs out the kernel sets a status bit and finishes.
+// Measured, cycles at j = 8 (D = 5000 / 46,868), before (dots by element, a counter barrier and then the partials, loads
+// where used) -> now: pass A with its loads 3000 / 3800 -> 3500 / 4000, its exchange 6700 / 6000 -> 3700 / 8000, pass B
+// 14200 / 20400 -> 6700 / 14500, its exchange 10300 / 10700 -> 3900 / 6000, pass C 8400 / 13700 -> 4500 / 11500; the launch
+// 23.4 / 26.8 -> 13.6 / 19.9 us on average over a run.  What remains at D = 46,868 is FP64 issue in B and C.
 constexpr int OB = 256;   // threads per block of the fused kernel
-constexpr long kBarrierSpin = 1L << 24;
+constexpr long kPollLimit = 1L << 20;
+constexpr int kOrthAlign = 128;              // elements of a block: a multiple of this
+constexpr int kOrthSmem = 220 * 1024;        // dynamic shared memory of a block at most
+constexpr int kPartRowsB1 = 8;               // second buffer of the second-pass partials: rows of partA from here on
+constexpr unsigned long long kEmpty = 0x7ff4dead7ff4deadull;   // a signalling NaN: arithmetic gives quiet ones
 
 // Segmented mode: the vector holds independent problems side by side (a direct sum of superblocks);
 // CTA b works on elements [lo_b, hi_b) of segment seg_b, and each segment has its own partial sums,
@@ -137,140 +169,65 @@ struct OrthArgs {
     int64_t n;
     int nv, j, nk;
     double tol;
-    double2* partA;
-    double2* partB;
+    double2* partA;    // first-pass partials, rows k of gridDim.x blocks
+    double2* partB;    // second-pass partials of this step (empty)
+    double2* partNext; // those of the next step (used by the step before): cleared here
     double* tri;
     int* flags;
-    unsigned* bar;     // [0] grid barrier counter (top bit flips at each barrier)
     int* status;
+    int chunk;         // elements of a block (one problem)
+    int rows;          // newest Krylov vectors staged in shared memory (STAGED)
+    int emax;          // elements of a block at most (shared-memory row)
     SegTab seg;        // seg.nseg == 0: one problem over the whole vector
 };
 
-// Grid barrier of the co-resident (cooperative) grid on one counter word whose low 31 bits stay zero:
-// block 0 adds 2^31 - (G - 1), every other block 1, so the top bit flips exactly when the last block
-// arrives, and each block waits until the top bit differs from the value it saw at its own arrival.  The
-// last arrival releases everyone directly (no reset, no second word).  Bounded wait: status bit 2.
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ double2 ld_slot(const double2* p) {   // two independent 8-byte values
+    double2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void grid_barrier(unsigned* bar, int* status) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned add = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u;
-        __threadfence();
-        const unsigned old = atomicAdd(bar, add);
-        long it = 0;
-        while (((old ^ ld_acquire_u32(bar)) & 0x80000000u) == 0u) {
-            if (++it > kBarrierSpin) { atomicOr(status, 2); break; }
-        }
-        __threadfence();
-    }
-    __syncthreads();
+__device__ __forceinline__ void st_slot(double* p, double v) {
+    asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
+__device__ __forceinline__ bool is_empty(double v) { return (unsigned long long)__double_as_longlong(v) == kEmpty; }
 
-// Block sums of NK complex values in a fixed order; the result is in out[0..NK-1].  Warp level:
-// reduce-scatter over ND = 2 * pow2ceil(NK) doubles (log2 ND halving levels, then a butterfly over the
-// remaining lane bits), after which lane l holds the warp total of double l >> (5 - log2 ND).
-template <int NK>
-__device__ void block_sum(double2 (&v)[NK], double* sh /* [OB/32][16] */, double2* out) {
-    constexpr int ND = NK <= 1 ? 2 : NK <= 2 ? 4 : NK <= 4 ? 8 : 16;
-    constexpr int LV = ND == 2 ? 1 : ND == 4 ? 2 : ND == 8 ? 3 : 4;
-    double d[ND];
+// h = sum of part[b0 .. b1) in a fixed order (lane l holds blocks b0 + l, b0 + l + 32, ...), waiting for each value; one warp.
+// Lanes 0-15 return the real, 16-31 the imaginary part.
+__device__ __forceinline__ double poll_sum(const double2* part, int b0, int b1, int* status) {
+    constexpr int U = 5;   // values in flight per lane
+    const int l = threadIdx.x & 31;
+    double re = 0.0, im = 0.0;
+    for (int c0 = b0; c0 < b1; c0 += 32 * U) {
+        double2 x[U];
 #pragma unroll
-    for (int k = 0; k < ND / 2; ++k) {
-        d[2 * k] = k < NK ? v[k < NK ? k : 0].x : 0.0;
-        d[2 * k + 1] = k < NK ? v[k < NK ? k : 0].y : 0.0;
-    }
-    const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+        for (int u = 0; u < U; ++u) x[u] = c0 + l + 32 * u < b1 ? ld_slot(part + c0 + l + 32 * u) : make_double2(0.0, 0.0);
+        for (long it = 0;; ++it) {   // only what is still empty is read again: all blocks poll the same few lines
+            bool ok = true;
 #pragma unroll
-    for (int lv = 0; lv < LV; ++lv) {
-        const int half = ND >> (lv + 1), o = 16 >> lv;
-        const bool up = (l & o) != 0;   // keep the upper half of the remaining values
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const double lo_v = d[i], hi_v = d[i + half];
-            const double send = up ? lo_v : hi_v;
-            d[i] = (up ? hi_v : lo_v) + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-#pragma unroll
-    for (int o = 16 >> LV; o > 0; o >>= 1) d[0] += __shfl_xor_sync(0xffffffffu, d[0], o);
-    __syncthreads();
-    if ((l & ((32 >> LV) - 1)) == 0) sh[w * 16 + (l >> (5 - LV))] = d[0];
-    __syncthreads();
-    if (threadIdx.x < 2 * NK) {
-        double s = 0.0;
-        for (int ww = 0; ww < OB / 32; ++ww) s += sh[ww * 16 + threadIdx.x];
-        reinterpret_cast<double*>(out)[threadIdx.x] = s;
-    }
-    __syncthreads();
-}
-
-// Deterministic block sum of one double (result in every thread).
-__device__ double block_sum1(double x, double* sh) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
-    __syncthreads();
-    double s = 0.0;
-    for (int k = 0; k < OB / 32; ++k) s += sh[k];
-    __syncthreads();
-    return s;
-}
-
-// partials[k * gridDim + b] for k < nv and b in [b0, b1)  ->  every block's h[k] (same order everywhere)
-__device__ void sum_partials(const double2* __restrict__ part, int nv, double2* h, int b0 = 0, int b1 = -1) {
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (b1 < 0) b1 = (int)gridDim.x;
-    for (int k = w; k < nv; k += OB / 32) {
-        double2 s = make_double2(0.0, 0.0);
-        for (int b = b0 + l; b < b1; b += 32) { s.x += part[(int64_t)k * gridDim.x + b].x; s.y += part[(int64_t)k * gridDim.x + b].y; }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-        }
-        if (l == 0) h[k] = s;
-    }
-    __syncthreads();
-}
-
-// Dots <v_k|x> over this block's chunk for k in [k0, k0 + NK), written as partials.  With
-// h != nullptr the chunk is first updated in place, x <- x - sum_u h_u v_{ju + u} over u < nu, and
-// ||x||^2 of the updated chunk is returned (this happens in the group k0 = 0 only).  NK is the exact
-// count: predicated-off FP64 instructions would still take issue slots of the slow FP64 pipe.
-template <int NK>
-__device__ double chunk_dots_n(const cplx* __restrict__ V, cplx* __restrict__ w, int64_t n, int ju, int nu, int k0,
-                               int64_t lo, int64_t hi, const double2* h, double2* part, double* sh, double2* red8) {
-    double2 acc[NK];
-#pragma unroll
-    for (int k = 0; k < NK; ++k) acc[k] = make_double2(0.0, 0.0);
-    double nn = 0.0;
-    const cplx* __restrict__ Vk = V + (int64_t)k0 * n;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += OB) {
-        double2 x = w[i];
-        if (h != nullptr && k0 == 0) {
-            for (int k = 0; k < nu; ++k) {
-                const double2 v = V[(int64_t)(ju + k) * n + i];
-                x.x = fma(-h[k].x, v.x, fma(h[k].y, v.y, x.x));
-                x.y = fma(-h[k].x, v.y, fma(-h[k].y, v.x, x.y));
+            for (int u = 0; u < U; ++u)
+                if (is_empty(x[u].x) || is_empty(x[u].y)) {
+                    x[u] = ld_slot(part + c0 + l + 32 * u);
+                    ok = false;
+                }
+            if (__all_sync(0xffffffffu, ok)) break;
+            if (it > kPollLimit) {
+                if (l == 0) atomicOr(status, 2);
+                break;
             }
-            w[i] = x;
-            nn = fma(x.x, x.x, fma(x.y, x.y, nn));
         }
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const double2 v = Vk[(int64_t)k * n + i];   // acc += conj(v) x
-            acc[k].x = fma(v.x, x.x, fma(v.y, x.y, acc[k].x));
-            acc[k].y = fma(v.x, x.y, fma(-v.y, x.x, acc[k].y));
+        for (int u = 0; u < U; ++u) {
+            if (c0 + 32 * u >= b1) break;   // uniform: no FP64 instructions for absent values
+            re += x[u].x;
+            im += x[u].y;
         }
     }
-    block_sum<NK>(acc, sh, red8);
-    if (threadIdx.x < NK) part[(int64_t)(k0 + threadIdx.x) * gridDim.x + blockIdx.x] = red8[threadIdx.x];
-    return nn;
+    // lanes 0-15 take the real, 16-31 the imaginary part; then a butterfly over 16 lanes
+    const bool up = l & 16;
+    double v = (up ? im : re) + __shfl_xor_sync(0xffffffffu, up ? re : im, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // FP32 value of a double by truncating its mantissa to 23 bits, on the integer pipe (conversions and FP64
@@ -282,67 +239,38 @@ __device__ __forceinline__ float f32_trunc(double x) {
     return ex <= 896u ? 0.f : __uint_as_float((hi & 0x80000000u) | ((ex - 896u) << 23) | mant);
 }
 
-// First-pass dots <v_k|w> over this block's chunk in FP32 (k in [k0, k0 + NK)), written as FP64
-// partials.  The second pass (FP64, chunk_dots_n with h) removes what this pass leaves along V to FP64
-// accuracy, and alpha is the sum of both passes' coefficients, so only the first pass's FP64 work goes.
-template <int NK>
-__device__ void chunk_dots_f32_n(const cplx* __restrict__ V, const cplx* __restrict__ w, int64_t n, int k0, int64_t lo,
-                                 int64_t hi, double2* part, double* sh, double2* red8) {
-    float2 fa[NK];
-#pragma unroll
-    for (int k = 0; k < NK; ++k) fa[k] = make_float2(0.f, 0.f);
-    const cplx* __restrict__ Vk = V + (int64_t)k0 * n;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += OB) {
-        const double2 x = w[i];
-        const float xr = f32_trunc(x.x), xi = f32_trunc(x.y);
-#pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const double2 v = Vk[(int64_t)k * n + i];   // acc += conj(v) x
-            const float vr = f32_trunc(v.x), vi = f32_trunc(v.y);
-            fa[k].x = fmaf(vr, xr, fmaf(vi, xi, fa[k].x));
-            fa[k].y = fmaf(vr, xi, fmaf(-vi, xr, fa[k].y));
-        }
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool wait_bulk(uint32_t bar) {
+    for (long i = 0; i < kPollLimit; ++i) {
+        uint32_t done;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(bar) : "memory");
+        if (done) return true;
     }
-    double2 acc[NK];
-#pragma unroll
-    for (int k = 0; k < NK; ++k) acc[k] = make_double2((double)fa[k].x, (double)fa[k].y);
-    block_sum<NK>(acc, sh, red8);
-    if (threadIdx.x < NK) part[(int64_t)(k0 + threadIdx.x) * gridDim.x + blockIdx.x] = red8[threadIdx.x];
+    return false;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-__device__ void chunk_dots_f32(const cplx* __restrict__ V, const cplx* __restrict__ w, int64_t n, int nv, int k0,
-                               int64_t lo, int64_t hi, double2* part, double* sh, double2* red8) {
-    switch (min(8, nv - k0)) {
-        case 1: return chunk_dots_f32_n<1>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 2: return chunk_dots_f32_n<2>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 3: return chunk_dots_f32_n<3>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 4: return chunk_dots_f32_n<4>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 5: return chunk_dots_f32_n<5>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 6: return chunk_dots_f32_n<6>(V, w, n, k0, lo, hi, part, sh, red8);
-        case 7: return chunk_dots_f32_n<7>(V, w, n, k0, lo, hi, part, sh, red8);
-        default: return chunk_dots_f32_n<8>(V, w, n, k0, lo, hi, part, sh, red8);
+// <v|x> over one warp's elements (lane, lane + 32, ...) of [0, E)
+__device__ __forceinline__ double2 warp_dot(const double2* v, const double2* x, int E) {
+    double2 s = make_double2(0.0, 0.0), t = make_double2(0.0, 0.0);
+    for (int i = threadIdx.x & 31; i < E; i += 32) {
+        const double2 a = v[i], b = x[i];
+        s.x = fma(a.x, b.x, s.x);
+        t.x = fma(a.y, b.y, t.x);
+        s.y = fma(a.x, b.y, s.y);
+        t.y = fma(a.y, b.x, t.y);
     }
+    return make_double2(s.x + t.x, s.y - t.y);
 }
 
-__device__ double chunk_dots(const cplx* __restrict__ V, cplx* __restrict__ w, int64_t n, int nv, int ju, int nu, int k0,
-                             int64_t lo, int64_t hi, const double2* h, double2* part, double* sh, double2* red8) {
-    switch (min(8, nv - k0)) {
-        case 1: return chunk_dots_n<1>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 2: return chunk_dots_n<2>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 3: return chunk_dots_n<3>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 4: return chunk_dots_n<4>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 5: return chunk_dots_n<5>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 6: return chunk_dots_n<6>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        case 7: return chunk_dots_n<7>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-        default: return chunk_dots_n<8>(V, w, n, ju, nu, k0, lo, hi, h, part, sh, red8);
-    }
-}
-
-template <bool SEG>
-__global__ void __launch_bounds__(OB) k_lanczos_orth_t(OrthArgs a) {
+template <bool SEG, bool STAGED>
+__global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(OrthArgs a) {
     pdl_enter();
-    // one problem: the whole grid stops together.  Segments: a stopped segment's blocks stay for the grid
-    // barriers and do nothing else.
+    // one problem: the whole grid stops together.  Segments: nobody waits for a stopped segment's blocks.
     int sg = 0, b0 = 0, b1 = (int)gridDim.x;
     int64_t lo, hi;
     if (SEG) {
@@ -352,73 +280,192 @@ __global__ void __launch_bounds__(OB) k_lanczos_orth_t(OrthArgs a) {
         lo = a.seg.cta_lo[blockIdx.x];
         hi = a.seg.cta_hi[blockIdx.x];
     } else {
-        const int64_t ch = (a.n + gridDim.x - 1) / gridDim.x;
-        lo = min(a.n, (int64_t)blockIdx.x * ch);
-        hi = min(a.n, lo + ch);
+        lo = min(a.n, (int64_t)blockIdx.x * a.chunk);
+        hi = min(a.n, lo + a.chunk);
     }
     double* tri = a.tri + (SEG ? (int64_t)sg * kTriStride : 0);
     int* flags = a.flags + (SEG ? sg * kFlagStride : 0);
-    const bool active = a.j < flags[0];   // uniform per segment: the flag only changes after the last barrier
-    if (!SEG && !active) return;
-    __shared__ double sh[(OB / 32) * 16];
-    __shared__ double2 red8[8];
-    __shared__ double2 h[33];
-    __shared__ double alpha1;   // the first pass's coefficient of v_j (alpha = pass 1 + pass 2)
-    // (A) first-pass dots (FP32) with v_{j-1} and v_j only: H v_j has components above rounding along
-    // these two alone (the three-term recurrence), so the first pass skips the older vectors
+    if (a.j >= flags[0]) return;   // stopped (uniform per segment: the flag only changes after the last exchange)
+    extern __shared__ double2 osm[];   // STAGED: w, then the newest `rows` Krylov vectors, emax elements each
+    __shared__ double2 h[34];
+    __shared__ double alpha1, sc[2];
+    __shared__ __align__(8) uint64_t bars[2];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int E = (int)(hi - lo), nv = a.nv, G = (int)gridDim.x;
+    const int s0 = STAGED ? nv - a.rows : nv;   // vectors s0 .. nv - 1 are staged
+    const cplx* gV = a.V + lo;
+    double2* w = STAGED ? osm : a.w + lo;
+    auto staged = [&](int k) -> const double2* { return osm + (int64_t)(1 + k - s0) * a.emax; };
     const int j0 = a.j > 0 ? a.j - 1 : 0, na = a.j - j0 + 1;
-    if (active) chunk_dots_f32(a.V + (int64_t)j0 * a.n, a.w, a.n, na, 0, lo, hi, a.partA, sh, red8);
-    grid_barrier(a.bar, a.status);
-    // (B) w' = w - h1_{j-1} v_{j-1} - h1_j v_j, second-pass dots with every v_k (FP64), ||w'||^2
-    double nn = 0.0;
-    if (active) {
-        sum_partials(a.partA, na, h, b0, b1);
-        if (threadIdx.x == 0) alpha1 = h[na - 1].x;
-        for (int k0 = 0; k0 < a.nv; k0 += 8) {
-            nn += chunk_dots(a.V, a.w, a.n, a.nv, j0, na, k0, lo, hi, h, a.partB, sh, red8);
-            __syncthreads();   // h is read by every thread of the first group
+    if (STAGED) {
+        if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bars + tid)));
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid == 0 && E > 0) {   // w, v_{j-1} and v_j first
+            const uint32_t bytes = (uint32_t)E * 16u;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bars)), "r"((1 + na) * bytes) : "memory");
+            bulk_load(smem_addr(osm), a.w + lo, bytes, smem_addr(bars));
+            for (int k = j0; k < nv; ++k) bulk_load(smem_addr(staged(k)), gV + (int64_t)k * a.n, bytes, smem_addr(bars));
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bars + 1)), "r"((j0 - s0) * bytes) : "memory");
+            for (int k = s0; k < j0; ++k) bulk_load(smem_addr(staged(k)), gV + (int64_t)k * a.n, bytes, smem_addr(bars + 1));
         }
-        nn = block_sum1(nn, sh);
-        if (threadIdx.x == 0) a.partB[(int64_t)a.nv * gridDim.x + blockIdx.x] = make_double2(nn, 0.0);
+        if (E > 0 && !wait_bulk(smem_addr(bars))) atomicOr(a.status, 2);
     }
-    grid_barrier(a.bar, a.status);
-    if (!active) return;
-    // (C) beta, stop test, v_{j+1} = (w' - sum h2_k v_k) / beta; the scalars by one thread (FP64
-    // instructions of the other warps would only repeat them on the slow FP64 pipe)
-    sum_partials(a.partB, a.nv + 1, h, b0, b1);
-    __shared__ double sc[2];
-    if (threadIdx.x == 0) {
-        double b2 = h[a.nv].x;
-        for (int k = 0; k < a.nv; ++k) b2 -= h[k].x * h[k].x + h[k].y * h[k].y;
-        const double bt = sqrt(fmax(b2, 0.0));
-        const double alpha = alpha1 + h[a.j].x;
-        if (blockIdx.x == b0) tri[T_ALPHA + a.j] = alpha;
-        const bool st = (a.j == a.nk - 1) || (bt <= a.tol * fmax(1.0, fabs(alpha)));
-        sc[0] = bt;
-        sc[1] = st ? 0.0 : 1.0 / bt;
+    // (A) first-pass dots (FP32, summed in FP64 from the warps on) with v_{j-1} and v_j only: H v_j has components
+    // above rounding along these two alone (the three-term recurrence), so the first pass skips the older vectors
+    const double2* v0 = STAGED ? staged(j0) : gV + (int64_t)j0 * a.n;
+    const double2* v1 = STAGED ? staged(a.j) : gV + (int64_t)a.j * a.n;
+    {
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = tid; i < E; i += OB) {
+            const double2 x = w[i], p = v0[i], q = v1[i];
+            const float xr = f32_trunc(x.x), xi = f32_trunc(x.y);
+            const float pr = f32_trunc(p.x), pi = f32_trunc(p.y), qr = f32_trunc(q.x), qi = f32_trunc(q.y);
+            f.x = fmaf(pr, xr, fmaf(pi, xi, f.x));
+            f.y = fmaf(pr, xi, fmaf(-pi, xr, f.y));
+            f.z = fmaf(qr, xr, fmaf(qi, xi, f.z));
+            f.w = fmaf(qr, xi, fmaf(-qi, xr, f.w));
+        }
+        double r = 0.0;   // lane l ends with component l / 8 of the warp's sums
+        if (warp * 32 < E) {
+            const bool u16 = lane & 16, u8 = lane & 8;
+            double k0 = u16 ? (double)f.z : (double)f.x, k1 = u16 ? (double)f.w : (double)f.y;
+            k0 += __shfl_xor_sync(0xffffffffu, u16 ? (double)f.x : (double)f.z, 16);
+            k1 += __shfl_xor_sync(0xffffffffu, u16 ? (double)f.y : (double)f.w, 16);
+            r = (u8 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, u8 ? k0 : k1, 8);
+            r += __shfl_xor_sync(0xffffffffu, r, 4);
+            r += __shfl_xor_sync(0xffffffffu, r, 2);
+            r += __shfl_xor_sync(0xffffffffu, r, 1);
+        }
+        double* shd = reinterpret_cast<double*>(h);   // [component][warp]
+        if ((lane & 7) == 0) shd[(lane >> 3) * 8 + warp] = r;
+        __syncthreads();
+        if (warp == 0) {   // lane = 8 component + warp
+            double t = shd[lane];
+            t += __shfl_xor_sync(0xffffffffu, t, 4);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            // components 0, 1: v_{j-1}; 2, 3: v_j (row na - 1; with j = 0 both are v_0, stored once)
+            const int row = na == 2 ? lane >> 4 : 0;
+            if ((lane & 7) == 0 && (na == 2 || lane >= 16))
+                st_slot(reinterpret_cast<double*>(a.partA + (int64_t)row * G + blockIdx.x) + ((lane >> 3) & 1), t);
+        }
     }
     __syncthreads();
-    const double beta = sc[0];
-    const bool stop = sc[1] == 0.0;
-    if (stop) {
-        if (blockIdx.x == b0 && threadIdx.x == 0) {
-            tri[T_BETA + a.j] = beta;
-            tri[T_RESID] = beta;
-            flags[0] = a.j + 1;   // read by later kernels only (every block is past its check)
-        }
-        return;
+    if (warp < na) {
+        const double v = poll_sum(a.partA + (int64_t)warp * G, b0, b1, a.status);
+        if (lane == 0) h[warp].x = v;
+        if (lane == 16) h[warp].y = v;
     }
-    if (blockIdx.x == b0 && threadIdx.x == 0) tri[T_BETA + a.j] = beta;
-    const double inv = sc[1];
-    cplx* vnext = const_cast<cplx*>(a.V) + (int64_t)(a.j + 1) * a.n;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += OB) {
-        double2 x = a.w[i];
-        for (int k = 0; k < a.nv; ++k) {
-            const double2 v = a.V[(int64_t)k * a.n + i];
-            x.x = fma(-h[k].x, v.x, fma(h[k].y, v.y, x.x));
-            x.y = fma(-h[k].x, v.y, fma(-h[k].y, v.x, x.y));
+    __syncthreads();
+    // (B) w' = w - h1_{j-1} v_{j-1} - h1_j v_j
+    {
+        const double2 p = h[0], q = na == 2 ? h[1] : make_double2(0.0, 0.0);
+        if (tid == 0) alpha1 = h[na - 1].x;
+        for (int i = tid; i < E; i += OB) {
+            double2 x = w[i];
+            const double2 u = v0[i];
+            x.x = fma(-p.x, u.x, fma(p.y, u.y, x.x));
+            x.y = fma(-p.x, u.y, fma(-p.y, u.x, x.y));
+            if (na == 2) {
+                const double2 v = v1[i];
+                x.x = fma(-q.x, v.x, fma(q.y, v.y, x.x));
+                x.y = fma(-q.x, v.y, fma(-q.y, v.x, x.y));
+            }
+            w[i] = x;
         }
-        vnext[i] = make_double2(x.x * inv, x.y * inv);
+    }
+    if (STAGED && E > 0 && !wait_bulk(smem_addr(bars + 1))) atomicOr(a.status, 2);
+    __syncthreads();
+    // second-pass dots with every v_k and ||w'||^2 (row nv), FP64: a warp per row
+    for (int k = warp; k <= nv; k += OB / 32) {
+        double2 d = make_double2(0.0, 0.0);
+        if (k == nv) {
+            double s = 0.0, t = 0.0;
+            for (int i = lane; i < E; i += 32) {
+                const double2 x = w[i];
+                s = fma(x.x, x.x, s);
+                t = fma(x.y, x.y, t);
+            }
+            d.x = s + t;
+        } else if (STAGED && k >= s0) {
+            d = warp_dot(staged(k), osm, E);
+        } else {
+            d = warp_dot(gV + (int64_t)k * a.n, w, E);
+        }
+        const bool up = lane & 16;
+        double v = (up ? d.y : d.x) + __shfl_xor_sync(0xffffffffu, up ? d.x : d.y, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0) st_slot(reinterpret_cast<double*>(a.partB + (int64_t)k * G + blockIdx.x) + (lane >> 4), v);
+    }
+    for (int k = warp; k <= nv; k += OB / 32) {
+        const double v = poll_sum(a.partB + (int64_t)k * G, b0, b1, a.status);
+        if (lane == 0) h[k].x = v;
+        if (lane == 16) h[k].y = v;
+    }
+    // every block of the problem has stored its second-pass partials, so it has read the first-pass ones, and the step
+    // before has ended: its own slots of both are cleared for the next step
+    __syncthreads();
+    if (tid < 2 * na) st_slot(reinterpret_cast<double*>(a.partA + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), __longlong_as_double((long long)kEmpty));
+    if (tid < 2 * (nv + 1)) st_slot(reinterpret_cast<double*>(a.partNext + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), __longlong_as_double((long long)kEmpty));
+    // (C) beta, stop test and 1 / beta by the last warp (h2 in parallel, one FP64 square root), beside the others'
+    // update x = w' - sum h2_k v_k
+    if (warp == OB / 32 - 1) {
+        double q = lane < nv ? fma(h[lane].x, h[lane].x, h[lane].y * h[lane].y) : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) {
+            const double bt = sqrt(fmax(h[nv].x - q, 0.0));
+            const double alpha = alpha1 + h[a.j].x;
+            const bool st = (a.j == a.nk - 1) || (bt <= a.tol * fmax(1.0, fabs(alpha)));
+            sc[0] = bt;
+            sc[1] = st ? 0.0 : 1.0 / bt;
+            if ((int)blockIdx.x == b0) {
+                tri[T_ALPHA + a.j] = alpha;
+                tri[T_BETA + a.j] = bt;
+                if (st) {
+                    tri[T_RESID] = bt;
+                    flags[0] = a.j + 1;   // read by later kernels only (every block is past its check)
+                }
+            }
+        }
+    }
+    const bool last_step = a.j == a.nk - 1;   // no next vector
+    cplx* vnext = const_cast<cplx*>(a.V) + (int64_t)(a.j + 1) * a.n + lo;
+    bool have_sc = false;
+    for (int i0 = 0; i0 < E && !last_step; i0 += OB) {
+        const int i = i0 + tid;
+        double2 x = make_double2(0.0, 0.0);
+        if (i < E) {
+            x = w[i];
+            int k = 0;
+            for (; k + 4 <= s0; k += 4) {   // not staged: four loads in flight
+                double2 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = gV[(int64_t)(k + u) * a.n + i];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    x.x = fma(-h[k + u].x, v[u].x, fma(h[k + u].y, v[u].y, x.x));
+                    x.y = fma(-h[k + u].x, v[u].y, fma(-h[k + u].y, v[u].x, x.y));
+                }
+            }
+            for (; k < s0; ++k) {
+                const double2 v = gV[(int64_t)k * a.n + i];
+                x.x = fma(-h[k].x, v.x, fma(h[k].y, v.y, x.x));
+                x.y = fma(-h[k].x, v.y, fma(-h[k].y, v.x, x.y));
+            }
+            if (STAGED)
+#pragma unroll 4
+                for (; k < nv; ++k) {
+                    const double2 v = staged(k)[i];
+                    x.x = fma(-h[k].x, v.x, fma(h[k].y, v.y, x.x));
+                    x.y = fma(-h[k].x, v.y, fma(-h[k].y, v.x, x.y));
+                }
+        }
+        if (!have_sc) { __syncthreads(); have_sc = true; }   // sc
+        if (sc[1] == 0.0) return;
+        if (i < E) vnext[i] = make_double2(x.x * sc[1], x.y * sc[1]);
     }
 }
 
@@ -763,8 +810,9 @@ __global__ void __launch_bounds__(NT) k_norm2_seg(const cplx* __restrict__ x, Se
 
 __global__ void __launch_bounds__(NT) k_init_v0_seg(const cplx* __restrict__ phi, SegTab tb, const double2* __restrict__ part,
                                                     cplx* __restrict__ v0, double* __restrict__ tri, int* __restrict__ flags,
-                                                    int nk) {
+                                                    int nk, OrthSlots slots) {
     pdl_enter();
+    clear_slots(slots);
     __shared__ double b0s;
     const int sg = tb.cta_seg[blockIdx.x], c0 = tb.seg_cta0[sg], c1 = tb.seg_cta0[sg + 1];
     if (threadIdx.x < 32) {   // the segment's partials in a fixed order
@@ -882,14 +930,18 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
     if (!rc) rc = dev_alloc(c, (void**)&k.flags, 4 * sizeof(int), "Krylov flags");
     // coefficients [x][k] of 16 targets, then the columns of the step exponential (32 x 32)
     if (!rc) rc = dev_alloc(c, (void**)&k.coef, kCoefWords * sizeof(cplx), "Krylov coefficients");
-    // grid barrier counter (word 0), then the ticket of k_tridiag_exp_eq (word 2)
-    if (!rc) rc = dev_alloc(c, (void**)&k.bar, kBarWords * sizeof(unsigned), "Krylov grid barrier");
-    if (!rc) rc = cuda_check(c, cudaMemset(k.bar, 0, kBarWords * sizeof(unsigned)), "Krylov grid barrier");
+    // the ticket of k_tridiag_exp_eq (word 2)
+    if (!rc) rc = dev_alloc(c, (void**)&k.bar, kBarWords * sizeof(unsigned), "Krylov ticket");
+    if (!rc) rc = cuda_check(c, cudaMemset(k.bar, 0, kBarWords * sizeof(unsigned)), "Krylov ticket");
     if (!rc) {   // co-resident grid of the fused orthogonalisation: at most one block per SM, at most NB
         int per_sm = 0;
-        rc = cuda_check(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lanczos_orth_t<true>, OB, 0), "occupancy");
+        rc = cuda_check(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lanczos_orth_t<true, false>, OB, 0), "occupancy");
         const int want = c->orth_per_sm > 0 ? c->orth_per_sm : 1;   // blocks per SM of the fused orthogonalisation
-        k.orth_grid = std::max(1, std::min({c->num_sms * std::max(per_sm, 1), c->num_sms * want, NB}));
+        k.orth_per_sm = std::max(1, std::min(want, std::max(per_sm, 1)));
+        k.orth_grid = std::max(1, std::min(c->num_sms * k.orth_per_sm, NB));
+        // the opt-in is a property of the kernels on the device: always the maximum
+        for (const void* f : {(const void*)k_lanczos_orth_t<false, true>, (const void*)k_lanczos_orth_t<true, true>})
+            if (!rc) rc = cuda_check(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kOrthSmem), "orthogonalisation smem");
     }
     if (rc) {
         dev_free(c, k.V, (size_t)(nk + 1) * n * sizeof(cplx));
@@ -917,6 +969,42 @@ cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* p
     return cudaGetLastError();
 }
 
+// Partial-sum slots of a Lanczos run on `grid` blocks with nk steps; norm partials of the start vector are in row 2 of partA.
+static OrthSlots orth_slots(const KrylovWork* k, int grid, int nk) {
+    return OrthSlots{k->partA, k->partB, k->partA + kPartRowsB1 * (int64_t)kRedBlocks, nk + 1, grid};
+}
+static double2* norm_slots(const KrylovWork* k) { return k->partA + 2 * (int64_t)kRedBlocks; }
+
+// One orthogonalisation step on `grid` co-resident blocks of at most emax elements.
+static cudaError_t launch_orth(tdmrg_ctx* c, const KrylovWork* k, OrthArgs a, int grid, int emax) {
+    const OrthSlots sl = orth_slots(k, grid, a.nk);
+    a.partA = sl.partA;
+    a.partB = (a.j & 1) ? sl.partB1 : sl.partB0;
+    a.partNext = (a.j & 1) ? sl.partB0 : sl.partB1;
+    a.emax = emax;
+    // shared memory: w and as many of the newest vectors as fit; at least v_{j-1} and v_j, else nothing is staged
+    const size_t row = (size_t)std::max(emax, 1) * sizeof(cplx), cap = (size_t)kOrthSmem / k->orth_per_sm;
+    const int fit = (int)std::min<size_t>(cap / row, 64) - 1;
+    const bool staged = fit >= std::min(a.nv, 2);
+    a.rows = staged ? std::min(a.nv, fit) : 0;
+    const size_t smem = staged ? (size_t)(1 + a.rows) * row : 0;
+    void* params[] = {&a};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(OB);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const void* f = a.seg.nseg > 0 ? (staged ? (const void*)k_lanczos_orth_t<true, true> : (const void*)k_lanczos_orth_t<true, false>)
+                                   : (staged ? (const void*)k_lanczos_orth_t<false, true> : (const void*)k_lanczos_orth_t<false, false>);
+    c->launches += 1;
+    return cudaLaunchKernelExC(&cfg, f, params);
+}
+
 // The Lanczos recursion of n_K steps started at phi (Sec. II.A): V, the tridiagonal and the flags in the
 // Krylov workspace of (Q, nk).
 int lanczos_build(tdmrg_ctx* c, int a, int b, const cplx* phi, int nk, KrylovWork** out) {
@@ -930,29 +1018,22 @@ int lanczos_build(tdmrg_ctx* c, int a, int b, const cplx* phi, int nk, KrylovWor
     if (rc) return rc;
     *out = k;
     cudaStream_t s = c->stream;
-    launch_pdl(k_norm2, NB, NT, 0, s, phi, n, k->partA);
-    launch_pdl(k_init_v0, NB, NT, 0, s, phi, n, k->partA, k->V, k->tri, k->flags, nk);
+    // blocks own multiples of kOrthAlign elements, at most one block per SM
+    const int64_t units = (n + kOrthAlign - 1) / kOrthAlign;
+    const int chunk = (int)(kOrthAlign * ((units + k->orth_grid - 1) / k->orth_grid));
+    const int grid = (int)((n + chunk - 1) / chunk);
+    launch_pdl(k_norm2, NB, NT, 0, s, phi, n, norm_slots(k));
+    launch_pdl(k_init_v0, NB, NT, 0, s, phi, n, (const double2*)norm_slots(k), k->V, k->tri, k->flags, nk, orth_slots(k, grid, nk));
     c->launches += 2;
     for (int j = 0; j < nk; ++j) {
         cplx* vj = k->V + (int64_t)j * n;
         rc = run_plan(c, *p, vj, k->w, k->flags, j);
         if (rc) return rc;
-        OrthArgs oa{k->V, k->w, n, j + 1, j, nk, c->opts.breakdown_tol, k->partA, k->partB, k->tri, k->flags,
-                    k->bar, c->dstatus};
-        void* params[] = {&oa};
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(k->orth_grid);
-        cfg.blockDim = dim3(OB);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        cudaError_t le = cudaLaunchKernelExC(&cfg, (const void*)k_lanczos_orth_t<false>, params);
+        OrthArgs oa{};
+        oa.V = k->V; oa.w = k->w; oa.n = n; oa.nv = j + 1; oa.j = j; oa.nk = nk; oa.tol = c->opts.breakdown_tol;
+        oa.tri = k->tri; oa.flags = k->flags; oa.status = c->dstatus; oa.chunk = chunk;
+        const cudaError_t le = launch_orth(c, k, oa, grid, (int)std::min<int64_t>(chunk, n));
         if (le != cudaSuccess) return cuda_check(c, le, "Lanczos orthogonalisation launch");
-        c->launches += 1;
     }
     return TDMRG_OK;
 }
@@ -1065,6 +1146,8 @@ static int ensure_segments(tdmrg_ctx* c, KrylovWork* k, int nseg, const int64_t*
             off += seg_len[s];
         }
         c0[nseg] = (int)cta_seg.size();
+        k->seg_emax = 1;
+        for (size_t b = 0; b < lo.size(); ++b) k->seg_emax = std::max(k->seg_emax, hi[b] - lo[b]);
         if (k->segmem_bytes < bytes) {
             dev_free(c, k->segmem, k->segmem_bytes);
             k->segmem = nullptr;
@@ -1127,28 +1210,18 @@ int evolve_segments(tdmrg_ctx* c, int a, int b, const cplx* phi, int nseg, const
     rc = ensure_segments(c, k, nseg, seg_len, &tb, &tri, &flags, &coef, &G);
     if (rc) return rc;
     cudaStream_t s = c->stream;
-    launch_pdl(k_norm2_seg, G, NT, 0, s, phi, tb, k->partA);
-    launch_pdl(k_init_v0_seg, G, NT, 0, s, phi, tb, k->partA, k->V, tri, flags, nk);
+    launch_pdl(k_norm2_seg, G, NT, 0, s, phi, tb, norm_slots(k));
+    launch_pdl(k_init_v0_seg, G, NT, 0, s, phi, tb, (const double2*)norm_slots(k), k->V, tri, flags, nk, orth_slots(k, G, nk));
     c->launches += 2;
     for (int j = 0; j < nk; ++j) {
         cplx* vj = k->V + (int64_t)j * n;
         rc = run_plan(c, *p, vj, k->w, nullptr, 0);   // every segment's product (a stopped one's is ignored)
         if (rc) return rc;
-        OrthArgs oa{k->V, k->w, n, j + 1, j, nk, c->opts.breakdown_tol, k->partA, k->partB, tri, flags, k->bar,
-                    c->dstatus, tb};
-        void* params[] = {&oa};
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(G);
-        cfg.blockDim = dim3(OB);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        cudaError_t le = cudaLaunchKernelExC(&cfg, (const void*)k_lanczos_orth_t<true>, params);
+        OrthArgs oa{};
+        oa.V = k->V; oa.w = k->w; oa.n = n; oa.nv = j + 1; oa.j = j; oa.nk = nk; oa.tol = c->opts.breakdown_tol;
+        oa.tri = tri; oa.flags = flags; oa.status = c->dstatus; oa.seg = tb;
+        const cudaError_t le = launch_orth(c, k, oa, G, (int)k->seg_emax);
         if (le != cudaSuccess) return cuda_check(c, le, "segmented Lanczos launch");
-        c->launches += 1;
     }
     Times tt{};
     for (int x = 0; x < n_v; ++x) tt.t[x] = t_x[x];
