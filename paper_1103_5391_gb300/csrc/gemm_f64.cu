@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
     __shared__ double2 red[GT];
     __shared__ int last;
     const Tile tile = args.tiles[blockIdx.x];
-    const Task task = args.tasks[tile.task];
+    const Task task = args.tasks[tile.task];   // used at the end only
     const int tid = threadIdx.x;
     const int nseg = tile.seg_hi - tile.seg_lo;
     if (tid < nseg) {
@@ -128,14 +128,14 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
     int m = 0, n = 0;
     if (active) {
         const int o = tile.o0 + lo;
-        if (task.herm) {   // row m of the lower triangle starts at m (m + 1) / 2
+        if (tile.N == 0) {   // row m of the lower triangle starts at m (m + 1) / 2
             m = (int)((sqrtf(8.f * (float)o + 1.f) - 1.f) * 0.5f);
             while ((m + 1) * (m + 2) / 2 <= o) ++m;
             while (m * (m + 1) / 2 > o) --m;
             n = o - m * (m + 1) / 2;
         } else {
-            m = o / task.N;
-            n = o - m * task.N;
+            m = o / tile.N;
+            n = o - m * tile.N;
         }
     }
     const int kspan = tile.k1 - tile.k0;

@@ -107,7 +107,8 @@ struct Tile {
     int32_t task, o0, cnt, ks;
     int32_t seg_lo, seg_hi, k0, k1;
     int32_t split, part, nparts, split_base;
-    int32_t cost, pad;        // complex MACs, for ordering
+    int32_t cost;             // complex MACs, for ordering
+    int32_t N;                // columns of the task's output (0: lower triangle), so that its outputs need no second load
 };
 // 16 x 16 output tile of the correction kernel (eigen-refinement), segments [seg_lo, seg_hi); K parts as above,
 // partial tiles at partials[(split_base + part) * 256].

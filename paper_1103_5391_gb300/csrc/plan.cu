@@ -116,11 +116,13 @@ int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
     return n;
 }
 
-// Tiles of the grouped FP64 GEMM.  The K range one warp runs through aims at a sixth of the launch's work per
-// FP64 pipe (152 SMs x 4), between 8 and 192: small launches are cut finely so that every pipe has work and no
-// chain is long, large ones into tiles of 256 outputs whose operands are reused by all of the CTA's warps.
-// Measured: a floor of 4 or 16 instead of 8 makes a Krylov advance at L=16 m=120 614 or 542 us instead of 527, a cap of
-// 64 instead of 192 rho_L at L=48 m=1000 607 us instead of 581.
+// Tiles of the grouped FP64 GEMM.  The K range one warp runs through aims at half the launch's work per FP64 pipe
+// (152 SMs x 4), between 8 and 192: small launches are cut finely so that every pipe has work and no chain is long,
+// but not more finely than that needs, as a CTA's fixed latency (its tables, the first operands, the sums of its
+// shares: ~6000 cycles) is that of ~25 complex k of a warp.  Measured with half / a sixth of the work: ground state
+// L=16 m=200 4.86 / 6.09 ms, eigendecomposition L=32 m=400 458 / 500 us; a floor of 4 or 16 instead of 8 makes a
+// Krylov advance at L=16 m=120 614 or 542 us instead of 527, a cap of 64 instead of 192 rho_L at L=48 m=1000 607 us
+// instead of 581.
 // A task's K is divided first among the warps of a CTA (ks = 1, 2, 4, 8 shares, 256 / ks outputs), then over CTAs.
 void make_tiles(TaskList& tl) {
     tl.tiles.clear();
@@ -139,7 +141,7 @@ void make_tiles(TaskList& tl) {
         }
         work += (double)outs[t] * (double)ks[t];
     }
-    const int64_t per_warp = (int64_t)std::min(192.0, std::max(8.0, work / (32.0 * 608.0 * 6.0)));
+    const int64_t per_warp = (int64_t)std::min(192.0, std::max(8.0, work / (32.0 * 608.0 * 2.0)));
     for (size_t t = 0; t < tl.tasks.size(); ++t) {
         const Task& k = tl.tasks[t];
         if (outs[t] <= 0) continue;
@@ -177,6 +179,7 @@ void make_tiles(TaskList& tl) {
             for (int p = 0; p < np; ++p) {
                 Tile tile{};
                 tile.task = (int32_t)t; tile.o0 = (int32_t)o0; tile.cnt = cnt; tile.ks = cks;
+                tile.N = k.herm ? 0 : k.N;
                 tile.seg_lo = parts[p].seg_lo; tile.seg_hi = parts[p].seg_hi;
                 tile.k0 = (int32_t)parts[p].k0; tile.k1 = (int32_t)parts[p].k1;
                 tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = (int32_t)base;
