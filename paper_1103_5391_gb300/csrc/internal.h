@@ -423,7 +423,7 @@ void dev_free(tdmrg_ctx* c, void* p, size_t bytes);
 int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qin0, int qin1, int qout0, int qout1,
                Plan* out);
 int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn);
-void make_tiles(TaskList& tl);
+void make_tiles(TaskList& tl, const std::vector<int>* group = nullptr);
 void make_corr_tiles(TaskList& tl, int ksplit);
 int upload(tdmrg_ctx* c, TaskList& tl);
 void release(tdmrg_ctx* c, TaskList& tl);

@@ -123,13 +123,15 @@ int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
 // L=16 m=200 4.86 / 6.09 ms, eigendecomposition L=32 m=400 458 / 500 us; a floor of 4 or 16 instead of 8 makes a
 // Krylov advance at L=16 m=120 614 or 542 us instead of 527, a cap of 64 instead of 192 rho_L at L=48 m=1000 607 us
 // instead of 581.
+// With groups (group[t] of task t) the work is that of the task's group alone, so that the sums of a group's outputs do
+// not depend on what else is launched with it.
 // A task's K is divided first among the warps of a CTA (ks = 1, 2, 4, 8 shares, 256 / ks outputs), then over CTAs.
-void make_tiles(TaskList& tl) {
+void make_tiles(TaskList& tl, const std::vector<int>* group) {
     tl.tiles.clear();
     tl.flops = 0.0;
     tl.nsplit = 0;
     tl.npartial = 0;
-    double work = 0.0;
+    std::vector<double> work(1, 0.0);
     std::vector<int64_t> outs(tl.tasks.size()), ks(tl.tasks.size(), 0);
     for (size_t t = 0; t < tl.tasks.size(); ++t) {
         const Task& k = tl.tasks[t];
@@ -139,12 +141,14 @@ void make_tiles(TaskList& tl) {
             // 8 real flops per complex multiply-add, 4 when one operand is real
             tl.flops += (tl.segs[s].rflags ? 4.0 : 8.0) * (double)k.M * k.N * (double)tl.segs[s].K;
         }
-        work += (double)outs[t] * (double)ks[t];
+        const size_t gr = group ? (size_t)(*group)[t] : 0;
+        if (gr >= work.size()) work.resize(gr + 1, 0.0);
+        work[gr] += (double)outs[t] * (double)ks[t];
     }
-    const int64_t per_warp = (int64_t)std::min(192.0, std::max(8.0, work / (32.0 * 608.0 * 2.0)));
     for (size_t t = 0; t < tl.tasks.size(); ++t) {
         const Task& k = tl.tasks[t];
         if (outs[t] <= 0) continue;
+        const int64_t per_warp = (int64_t)std::min(192.0, std::max(8.0, work[group ? (*group)[t] : 0] / (32.0 * 608.0 * 2.0)));
         const int64_t shares = std::max<int64_t>(1, (ks[t] + per_warp - 1) / per_warp);
         const int cks = shares <= 1 ? 1 : shares <= 2 ? 2 : shares <= 4 ? 4 : 8;
         const int area = kTileOut / cks;
@@ -280,9 +284,20 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
     std::vector<int> out_of_q(L.dim.size(), -1);
     for (size_t k = 0; k < pout.size(); ++k) out_of_q[pout[k].qi] = (int)k;
 
+    // left sectors that the terms connect: the superblocks of a direct sum stay apart, and every one gets the K parts (so
+    // the bits) that it has alone; without the groups H psi of the jobs of a batch differed from theirs alone in
+    // the last bit, and with parts by a task's own size instead H psi at L=16 m=200 takes 40 to 49 us instead of 41, the
+    // ground state 4.84 to 5.99 ms instead of 4.87, a Krylov advance at L=16 m=120 427 to 466 us instead of 429
+    std::vector<int> root(L.dim.size());
+    for (size_t k = 0; k < root.size(); ++k) root[k] = (int)k;
+    auto find_root = [&](int q) {
+        while (root[q] != q) q = root[q] = root[root[q]];
+        return q;
+    };
     std::vector<std::vector<Seg>> direct(pout.size()), left(pout.size());
     std::vector<Task> s1_inter;
     std::vector<Seg> s1_inter_seg;
+    std::vector<int> s1_inter_q, g1, g2;   // left sectors of the intermediates, groups of the tasks
     int64_t scr = 0;
     const cplx one = make_double2(1.0, 0.0);
 
@@ -313,6 +328,7 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
                 for (auto& b : bl) {
                     if (b.first != po.ri) continue;
                     if (!A && !B) return fail(c, TDMRG_EINVAL, "a term needs an operator on at least one block");
+                    root[find_root(a.first)] = find_root(pi.qi);
                     if (!A) {          // Psi'_q += sc * Psi_q B^T, written by stage 1
                         Seg s{};
                         s.a_off = pi.off; s.a_buf = BUF_IN; s.lda = pi.dr;
@@ -339,6 +355,7 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
                         s.K = pi.dr; s.scale = one; s.dscale = -1;
                         s.rflags = b_real;
                         s1_inter.push_back(tk);
+                        s1_inter_q.push_back(pi.qi);
                         s1_inter_seg.push_back(s);
                         Seg s2{};
                         s2.a_off = a.second; s2.a_buf = BUF_OPS; s2.lda = pi.dl;
@@ -366,6 +383,7 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         for (auto& s : direct[k]) s1.segs.push_back(s);
         tk.seg_end = (int)s1.segs.size();
         s1.tasks.push_back(tk);
+        g1.push_back(find_root(pout[k].qi));
     }
     for (size_t k = 0; k < s1_inter.size(); ++k) {
         Task tk = s1_inter[k];
@@ -373,6 +391,7 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         s1.segs.push_back(s1_inter_seg[k]);
         tk.seg_end = (int)s1.segs.size();
         s1.tasks.push_back(tk);
+        g1.push_back(find_root(s1_inter_q[k]));
     }
     // stage 2: one task per output block that still needs left products or a zero fill
     for (size_t k = 0; k < pout.size(); ++k) {
@@ -385,9 +404,10 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         for (auto& s : left[k]) s2.segs.push_back(s);
         tk.seg_end = (int)s2.segs.size();
         s2.tasks.push_back(tk);
+        g2.push_back(find_root(pout[k].qi));
     }
-    make_tiles(s1);
-    make_tiles(s2);
+    make_tiles(s1, &g1);
+    make_tiles(s2, &g2);
     p->scratch = scr;
     p->flops = s1.flops + s2.flops;
     int urc = upload(c, s1);
