@@ -27,12 +27,12 @@
 // is what limits the accuracy, so it suits small corrections only, not full products.  It works on 16 x 16
 // output tiles staged through shared memory.
 #include "internal.h"
+#include "lane_mac.cuh"
 
 namespace tdmrg {
 namespace {
 
 constexpr int GT = 256;               // threads of a CTA of the grouped GEMM
-constexpr int UK = 4;                 // k steps loaded ahead
 
 // Sign flip of a double on the integer pipe
 __device__ __forceinline__ double neg(double x) { return __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63)); }
@@ -46,44 +46,6 @@ struct SegView {
     double ca, cb;                    // -1: conjugated operand
     double sr, si;                    // factor
 };
-
-// s0 += Re a Re b, s1 += Im a Im b, s2 += Re a Im b, s3 += Im a Re b over k in [k0, k1)
-template <int MODE>
-__device__ __forceinline__ void seg_mac(const double2* __restrict__ pa, const double2* __restrict__ pb, int ak, int bk, int nk,
-                                        double (&s)[4]) {
-    auto mac = [&](double2 a, double2 b) {
-        s[0] = fma(a.x, b.x, s[0]);
-        if (MODE == 0) s[1] = fma(a.y, b.y, s[1]);
-        if (MODE != 2) s[2] = fma(a.x, b.y, s[2]);
-        if (MODE != 1) s[3] = fma(a.y, b.x, s[3]);
-    };
-    int k = 0;
-    if (nk >= UK) {
-        double2 a[UK], b[UK];
-#pragma unroll
-        for (int u = 0; u < UK; ++u) { a[u] = __ldg(pa + u * ak); b[u] = __ldg(pb + u * bk); }
-        for (k = UK; k + UK <= nk; k += UK) {
-            pa += (int64_t)UK * ak;
-            pb += (int64_t)UK * bk;
-            double2 na[UK], nb[UK];
-#pragma unroll
-            for (int u = 0; u < UK; ++u) { na[u] = __ldg(pa + u * ak); nb[u] = __ldg(pb + u * bk); }
-#pragma unroll
-            for (int u = 0; u < UK; ++u) mac(a[u], b[u]);
-#pragma unroll
-            for (int u = 0; u < UK; ++u) { a[u] = na[u]; b[u] = nb[u]; }
-        }
-        pa += (int64_t)UK * ak;
-        pb += (int64_t)UK * bk;
-#pragma unroll
-        for (int u = 0; u < UK; ++u) mac(a[u], b[u]);
-    }
-    for (; k < nk; ++k) {
-        mac(__ldg(pa), __ldg(pb));
-        pa += ak;
-        pb += bk;
-    }
-}
 
 __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const int* skip_flag, int skip_step) {
     pdl_enter();
@@ -152,9 +114,9 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
             const double2* pa = w.a + (int64_t)m * w.am + (int64_t)k0 * w.ak;
             const double2* pb = w.b + (int64_t)n * w.bn + (int64_t)k0 * w.bk;
             double q[4] = {0.0, 0.0, 0.0, 0.0};
-            if (w.mode == 0) seg_mac<0>(pa, pb, w.ak, w.bk, k1 - k0, q);
-            else if (w.mode == 1) seg_mac<1>(pa, pb, w.ak, w.bk, k1 - k0, q);
-            else seg_mac<2>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            if (w.mode == 0) seg_mac<0, 4>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            else if (w.mode == 1) seg_mac<1, 4>(pa, pb, w.ak, w.bk, k1 - k0, q);
+            else seg_mac<2, 4>(pa, pb, w.ak, w.bk, k1 - k0, q);
             const double pr = fma(-w.ca * w.cb, q[1], q[0]), pi = fma(w.cb, q[2], w.ca * q[3]);
             const double sr = w.sr, si = w.si;
             if (si == 0.0) {

@@ -147,9 +147,11 @@ struct OzTask {            // one complex GEMM C (+)= A op(B), all of its segmen
     int8_t c_buf, beta, trans, pad1;
 };
 struct OzTile { int32_t task, m0, n0, cost; };
-// An 8 x 8 output block of a thin sector-pair product (min(M, N) below the thin threshold), computed in
-// FP64 by the thin warps of the persistent tensor kernel; task indexes the stage's FP64 thin tasks.
-struct ThinItem { int32_t task, m0, n0, cost; };
+// Outputs of thin sector-pair products (min(M, N) below the thin threshold), entries [out0, out0 + cnt) of the stage's
+// output list (task, flattened index), for one thin warp of the persistent tensor kernel: each output on 2^(lps + lpk)
+// lanes, which take every 2^lps-th segment and one of 2^lpk parts of its K.
+struct ThinItem { int32_t out0, cnt, cost; int16_t lps, lpk; };
+
 struct OzSliceJob {        // slices the rows of A' (role 0) or columns of B' (role 1) of one operand
     int32_t role, nvec, seg_begin, seg_end, row0, exp0, ktot, use_scale, vec_prefix;
 };
@@ -173,6 +175,7 @@ struct OzGemmArgs {
     const Task* ttasks;       // thin tasks (FP64 warps): tasks, segments, items grouped by CTA
     const Seg* tsegs;
     const ThinItem* titems;
+    const int2* touts;
     const int* tcta;          // items of CTA b: titems[tcta[b] .. tcta[b + 1]) (null: none)
 };
 struct OzStage {
@@ -205,10 +208,12 @@ struct OzStage {
     std::vector<Task> ttasks;
     std::vector<Seg> tsegs;
     std::vector<ThinItem> titems;
+    std::vector<int2> touts;
     std::vector<int> tcta;
     Task* d_ttasks = nullptr;
     Seg* d_tsegs = nullptr;
     ThinItem* d_titems = nullptr;
+    int2* d_touts = nullptr;
     int* d_tcta = nullptr;
     double thin_flops = 0.0;   // algorithmic flops of the thin products (8 per complex MAC)
     CUtensorMap mapA, mapB, mapA128;

@@ -24,6 +24,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "lane_mac.cuh"
 
 namespace tdmrg {
 namespace {
@@ -465,7 +466,9 @@ template <int TMW> __host__ __device__ constexpr int ws_aboxw() { return TMW * K
 template <int TMW> __host__ __device__ constexpr int ws_nst() { return TMW == 128 ? 2 : 3; }  // shared-memory stages
 constexpr int EPIW = 16;                   // epilogue warps: four per TMEM lane quarter, 16 accumulator columns each
 constexpr int THINW = 2;                   // FP64 warps for the thin sector-pair products
-constexpr int kThinMaxKsteps = 8;          // a thin block's m8n8k4 steps at most (K <= 32 over all its segments)
+constexpr int kThinMaxKsteps = 8;          // steps of four k at most (each segment rounded up) for a thin product
+constexpr int kThinChain = 24;             // k-steps of one lane above which an output is shared by more lanes
+constexpr int kThinLog2Parts = 3;
 constexpr int WS_THREADS = 64 + 32 * EPIW + 32 * THINW;
 constexpr int RT = 4;                      // tile-index ring between the producer and the consumers
 constexpr long kWaitWS = 1L << 22;
@@ -485,65 +488,67 @@ __device__ __forceinline__ bool mbar_wait_ws(uint32_t bar, uint32_t parity, vola
 // ---- thin sector-pair products (K3): FP64 on the warps the tensor pipeline leaves idle ---------------
 // A product whose output block has fewer than thin_dim rows or columns fills a small part of a 64-row
 // tensor tile, so it would cost a whole tile (TMA boxes, S(S+1)/2 MMAs per k-step, TMEM readout) for
-// little work.  Such products run instead on THINW extra warps of the persistent kernel, in FP64 with
-// the FP64 tensor MMA (mma.sync m8n8k4), straight from the FP64 operands (no slicing): the FP64 pipe is
-// otherwise idle during the tensor pipeline, and these operands need neither slices nor TMA boxes.
-// One warp computes one 8 x 8 output block over all segments of its task; items are assigned to CTAs
-// at plan build, longest first onto the least loaded CTA.
-__device__ __forceinline__ void dmma_f64(double& c0, double& c1, double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
-                 : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
-}
-__device__ __forceinline__ double neg_f64(double x) { return __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63)); }
-
-__device__ __forceinline__ void thin_block(const ThinItem& it, const Task& tk, const Seg* __restrict__ segs,
-                                           const GemmArgs& g, int lane) {
-    const int gid = lane >> 2, tig = lane & 3;   // fragment layout of m8n8k4: A[gid][tig], B[tig][gid]
-    const int r = it.m0 + gid, cb = it.n0 + gid;
-    const bool rv = r < tk.M, cv = cb < tk.N;
-    double cre0 = 0.0, cre1 = 0.0, cim0 = 0.0, cim1 = 0.0;
-    for (int si = tk.seg_begin; si < tk.seg_end; ++si) {
-        const Seg sg = segs[si];
-        const cplx* __restrict__ A = g.bufs[sg.a_buf] + sg.a_off + (int64_t)r * sg.lda;
-        const cplx* __restrict__ B = g.bufs[sg.b_buf] + sg.b_off;
-        const bool bn = sg.opb == OPB_N, bc = sg.opb == OPB_C;
-        const cplx* __restrict__ Bc = bn ? B + cb : B + (int64_t)cb * sg.ldb;   // column cb of op(B)
-        const int64_t bk = bn ? sg.ldb : 1;                                         // its step along k
-        double pre0 = 0.0, pre1 = 0.0, pim0 = 0.0, pim1 = 0.0;
-        const bool a_real = (sg.rflags & 1) != 0, b_real = (sg.rflags & 2) != 0;   // zero imaginary products skipped
-#pragma unroll 2
-        for (int k0 = 0; k0 < sg.K; k0 += 4) {
-            const int k = k0 + tig;
-            double2 a = make_double2(0.0, 0.0), b = make_double2(0.0, 0.0);
-            if (rv && k < sg.K) a = A[k];
-            if (cv && k < sg.K) b = Bc[(int64_t)k * bk];
-            if (bc) b.y = neg_f64(b.y);
-            dmma_f64(pre0, pre1, a.x, b.x);           // Re += Re a Re b - Im a Im b
-            if (!a_real && !b_real) dmma_f64(pre0, pre1, neg_f64(a.y), b.y);
-            if (!b_real) dmma_f64(pim0, pim1, a.x, b.y);   // Im += Re a Im b + Im a Re b
-            if (!a_real) dmma_f64(pim0, pim1, a.y, b.x);
+// little work.  Such products run instead in FP64 straight from the FP64 operands (no slices, no TMA boxes) on THINW
+// extra warps of the persistent kernel, joined by the epilogue warps after the CTA's last tile.  One output per lane:
+// the outputs of all thin tasks of a stage are put in order of segments and K, and an item is a warp of consecutive ones,
+// of one task or of several, so that blocks of a few entries fill their warps; items go to CTAs at plan build, longest
+// first onto the least loaded.  What bounds them is latency (tables and operands, one segment after the other, and 4 FP64
+// instructions of 64 cycles per complex k), so an output whose chain is above kThinChain k-steps (a segment as 4) is
+// shared by up to 2^kThinLog2Parts lanes, over segments first.  Measured, stage 1 of six batched jobs (where the thin
+// products are the longest chain) and L = 32, m = 400 H psi: 8 x 8 blocks of m8n8k4 MMAs (3 x padding) 57 us, 46 us;
+// a warp per task and 32 outputs 60 us, 46 us; outputs packed over tasks 51 us; the epilogue warps joining in 29 us,
+// 47.4 us; the split over lanes 29 us, 46.3 us; the CTA's range passed on in shared memory 29 us, 45.8 us.
+__device__ __forceinline__ void thin_item(const ThinItem& it, int lane, const OzGemmArgs& oa, const GemmArgs& g) {
+    const int W = 32 >> (it.lps + it.lpk);   // outputs of the item; lanes of part p of every output: p W .. p W + W - 1
+    const int oi = lane & (W - 1), part = lane / W;
+    const int ps = part >> it.lpk, pk = part & ((1 << it.lpk) - 1);
+    double re = 0.0, im = 0.0;
+    Task tk;
+    int r = 0, n = 0;
+    if (oi < it.cnt) {
+        const int2 out = oa.touts[it.out0 + oi];
+        tk = oa.ttasks[out.x];
+        if (tk.trans) { n = out.y / tk.M; r = out.y - n * tk.M; }   // neighbouring lanes store neighbouring elements
+        else { r = out.y / tk.N; n = out.y - r * tk.N; }
+        for (int si = tk.seg_begin + ps; si < tk.seg_end; si += 1 << it.lps) {
+            const Seg sg = oa.tsegs[si];
+            const bool bn = sg.opb == OPB_N;
+            const int k0 = (sg.K * pk) >> it.lpk, nk = ((sg.K * (pk + 1)) >> it.lpk) - k0;
+            const int bk = bn ? sg.ldb : 1;
+            const cplx* A = g.bufs[sg.a_buf] + sg.a_off + (int64_t)r * sg.lda + k0;
+            const cplx* B = g.bufs[sg.b_buf] + sg.b_off + (bn ? (int64_t)n : (int64_t)n * sg.ldb) + (int64_t)k0 * bk;
+            double q[4] = {0.0, 0.0, 0.0, 0.0};
+            if (sg.rflags & 1) seg_mac<1, 2>(A, B, 1, bk, nk, q);          // zero imaginary products skipped
+            else if (sg.rflags & 2) seg_mac<2, 2>(A, B, 1, bk, nk, q);
+            else seg_mac<0, 2>(A, B, 1, bk, nk, q);
+            const bool bc = sg.opb == OPB_C;
+            const double pr = bc ? q[0] + q[1] : q[0] - q[1], pi = bc ? q[3] - q[2] : q[2] + q[3];
+            double sr = sg.scale.x, si2 = sg.scale.y;   // segment factor on the sums
+            if (sg.dcoef >= 0 && g.dcoef != nullptr) {   // run-time coefficient of a connection term
+                const cplx d = g.dcoef[sg.dcoef];
+                const double tr = sr * d.x - si2 * d.y;
+                si2 = sr * d.y + si2 * d.x;
+                sr = tr;
+            }
+            if (si2 == 0.0) {
+                re = fma(sr, pr, re);
+                im = fma(sr, pi, im);
+            } else {
+                re = fma(sr, pr, fma(-si2, pi, re));
+                im = fma(sr, pi, fma(si2, pr, im));
+            }
         }
-        double sr = sg.scale.x, si2 = sg.scale.y;   // segment factor on the block's partial product
-        if (sg.dcoef >= 0 && g.dcoef != nullptr) {   // run-time coefficient of a connection term
-            const cplx d = g.dcoef[sg.dcoef];
-            const double tr = sr * d.x - si2 * d.y;
-            si2 = sr * d.y + si2 * d.x;
-            sr = tr;
-        }
-        cre0 += sr * pre0 - si2 * pim0; cim0 += sr * pim0 + si2 * pre0;
-        cre1 += sr * pre1 - si2 * pim1; cim1 += sr * pim1 + si2 * pre1;
     }
-    if (!rv) return;
-    cplx* __restrict__ C = g.bufs[tk.c_buf] + tk.c_off;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int n = it.n0 + 2 * tig + e;
-        if (n < tk.N) {
-            cplx* p = tk.trans ? C + (int64_t)n * tk.ldc + r : C + (int64_t)r * tk.ldc + n;
-            double2 v = e ? make_double2(cre1, cim1) : make_double2(cre0, cim0);
-            if (tk.beta) { const double2 o = *p; v.x += o.x; v.y += o.y; }
-            *p = v;
-        }
+    __syncwarp();
+    for (int off = W; off < 32; off <<= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, off);
+        im += __shfl_xor_sync(0xffffffffu, im, off);
+    }
+    if (part == 0 && oi < it.cnt) {
+        cplx* __restrict__ C = g.bufs[tk.c_buf] + tk.c_off;
+        cplx* p = tk.trans ? C + (int64_t)n * tk.ldc + r : C + (int64_t)r * tk.ldc + n;
+        if (tk.beta) { const double2 old = *p; re += old.x; im += old.y; }
+        *p = make_double2(re, im);
     }
 }
 
@@ -572,9 +577,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
     __shared__ int sExp[EPIW][16];   // column exponents of the epilogue warps' current tile
     __shared__ uint32_t tmem_base;
     __shared__ volatile int failed;
+    __shared__ int thin_next;             // thin items of this CTA taken so far
+    __shared__ volatile int thin_rng[2];  // its range of items, once a thin warp has read it (else -1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         failed = 0;
+        thin_next = 0;
+        thin_rng[0] = thin_rng[1] = -1;
         for (int i = 0; i < NST; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&full[i])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&empty[i])));
@@ -689,15 +698,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
                 }
             }
         }
-    } else if (warp >= 2 + EPIW) {   // ----------------------------------------------------------- thin FP64 warps
-        if (oa.tcta != nullptr) {
-            const int i1 = oa.tcta[blockIdx.x + 1];
-            for (int i = oa.tcta[blockIdx.x] + (warp - 2 - EPIW); i < i1; i += THINW) {
-                const ThinItem it = oa.titems[i];
-                thin_block(it, oa.ttasks[it.task], oa.tsegs, g, lane);
-            }
-        }
-    } else {   // ------------------------------------------------------------------------ epilogue warps 2..17
+    } else if (warp < 2 + EPIW) {   // ------------------------------------------------------ epilogue warps 2..17
         const int quad = warp & 3;            // TMEM lanes 32 * quad .. 32 * quad + 31 (M = 64: 16 of them hold rows)
         const int part = (warp - 2) >> 2;     // accumulator columns 16 * part .. 16 * part + 15
         const int row = (TMW == 128 ? 32 : 16) * quad + lane;
@@ -782,6 +783,23 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
                 }
             }
             __syncwarp();   // sExp is rewritten for the next tile
+        }
+    }
+    // thin FP64 items of this CTA, longest first: the thin warps from the start, the epilogue warps after their last tile
+    if (warp >= 2 && oa.tcta != nullptr) {
+        int i0 = thin_rng[0], i1 = thin_rng[1];
+        if (__any_sync(0xffffffffu, i0 < 0 || i1 < 0)) {
+            i0 = oa.tcta[blockIdx.x];
+            i1 = oa.tcta[blockIdx.x + 1];
+            if (warp == 2 + EPIW && lane == 0) { thin_rng[0] = i0; thin_rng[1] = i1; }
+        }
+        for (;;) {
+            int i = 0;
+            if (lane == 0) i = atomicAdd(&thin_next, 1);
+            i = i0 + __shfl_sync(0xffffffffu, i, 0);
+            if (i >= i1) break;
+            const ThinItem it = oa.titems[i];
+            thin_item(it, lane, oa, g);
         }
     }
     __syncwarp();   // the producer and MMA threads rejoin their warps: the barrier below waits for every thread
@@ -903,6 +921,7 @@ void release_oz(tdmrg_ctx* c, OzPlan& oz) {
         dev_free(c, st.d_ttasks, st.ttasks.size() * sizeof(Task));
         dev_free(c, st.d_tsegs, st.tsegs.size() * sizeof(Seg));
         dev_free(c, st.d_titems, st.titems.size() * sizeof(ThinItem));
+        dev_free(c, st.d_touts, st.touts.size() * sizeof(int2));
         dev_free(c, st.d_tcta, st.tcta.size() * sizeof(int));
         st = OzStage();
     }
@@ -1006,8 +1025,8 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
             int ktot = 0;
             bool dev_scale = false;
             for (int s = tk.seg_begin; s < tk.seg_end; ++s) { ktot += tl.segs[s].K; dev_scale |= tl.segs[s].dscale >= 0; }
-            // thin product: on the FP64 warps of the persistent kernel (S <= 4), in 8 x 8 output blocks, if one
-            // block's FP64 chain is short (GB300 runs an m8n8k4 FP64 MMA in ~640 cycles of a sub-partition)
+            // thin product: on the FP64 warps of the persistent kernel (S <= 4), if an output's FP64 chain is short (256
+            // cycles of a sub-partition per complex k)
             int ksteps_all = 0;
             for (int s = tk.seg_begin; s < tk.seg_end; ++s) ksteps_all += (tl.segs[s].K + 3) / 4;
             if (S <= 4 && c->thin_dim > 0 && nseg > 0 && !dev_scale && std::min(tk.M, tk.N) < c->thin_dim &&
@@ -1018,10 +1037,6 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
                 nt.seg_end = (int)st.tsegs.size();
                 const int ti = (int)st.ttasks.size();
                 st.ttasks.push_back(nt);
-                int ksteps = 0;   // m8n8k4 steps of one block over all segments
-                for (int s = tk.seg_begin; s < tk.seg_end; ++s) ksteps += (tl.segs[s].K + 3) / 4;
-                for (int m0 = 0; m0 < tk.M; m0 += 8)
-                    for (int n0 = 0; n0 < tk.N; n0 += 8) st.titems.push_back({ti, m0, n0, std::max(ksteps, 1)});
                 st.thin_flops += 8.0 * tk.M * tk.N * (double)ktot;
                 continue;
             }
@@ -1102,6 +1117,37 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
         }
         std::stable_sort(st.tiles.begin(), st.tiles.end(), [](const OzTile& a, const OzTile& b) { return a.cost > b.cost; });
         std::stable_sort(st.tiles128.begin(), st.tiles128.end(), [](const OzTile& a, const OzTile& b) { return a.cost > b.cost; });
+        // thin outputs in order of (segments, K, real operands), 32 per item; an item costs its longest chain and the latency
+        // of its tables and operands
+        if (!st.ttasks.empty()) {
+            struct Key { int nseg, k, mode, task; };
+            std::vector<Key> keys;
+            for (size_t t = 0; t < st.ttasks.size(); ++t) {
+                const Task& tk = st.ttasks[t];
+                Key kk{tk.seg_end - tk.seg_begin, 0, 0, (int)t};
+                for (int s = tk.seg_begin; s < tk.seg_end; ++s) { kk.k += st.tsegs[s].K; kk.mode = kk.mode * 4 + (st.tsegs[s].rflags & 3); }
+                keys.push_back(kk);
+            }
+            std::stable_sort(keys.begin(), keys.end(), [](const Key& x, const Key& y) {
+                return std::make_tuple(-x.nseg, -x.k, x.mode) < std::make_tuple(-y.nseg, -y.k, y.mode);
+            });
+            for (const Key& kk : keys)
+                for (int o = 0; o < st.ttasks[kk.task].M * st.ttasks[kk.task].N; ++o) {
+                    if (st.titems.empty() || st.titems.back().cnt == 32 >> (st.titems.back().lps + st.titems.back().lpk)) {
+                        ThinItem it{(int)st.touts.size(), 0, 0, 0, 0};
+                        auto cost = [&] {   // k-steps in a row, segments in a row and the first loads
+                            return kk.k / (1 << (it.lps + it.lpk)) + 4 * ((kk.nseg + (1 << it.lps) - 1) >> it.lps) + 4;
+                        };
+                        while (it.lps + it.lpk < kThinLog2Parts && cost() > kThinChain)
+                            if ((1 << it.lps) < kk.nseg) ++it.lps;
+                            else ++it.lpk;
+                        it.cost = cost();
+                        st.titems.push_back(it);
+                    }
+                    st.touts.push_back(make_int2(kk.task, o));
+                    ++st.titems.back().cnt;
+                }
+        }
         // persistent grid: one CTA per SM when thin items exist (their warps ride along), else one per tile
         st.grid = st.titems.empty() ? std::max(1, std::min((int)st.tiles.size(), c->num_sms)) : c->num_sms;
         if (!st.titems.empty()) {   // thin items: longest first onto the least loaded CTA, grouped by CTA
@@ -1142,10 +1188,11 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
             rc = upload_vec(c, st.ttasks, &st.d_ttasks, "thin tasks");
             if (!rc) rc = upload_vec(c, st.tsegs, &st.d_tsegs, "thin segments");
             if (!rc) rc = upload_vec(c, st.titems, &st.d_titems, "thin items");
+            if (!rc) rc = upload_vec(c, st.touts, &st.d_touts, "thin items");
             if (!rc) rc = upload_vec(c, st.tcta, &st.d_tcta, "thin items");
             if (rc) return rc;
         }
-        st.args.ttasks = st.d_ttasks; st.args.tsegs = st.d_tsegs; st.args.titems = st.d_titems; st.args.tcta = st.d_tcta;
+        st.args.ttasks = st.d_ttasks; st.args.tsegs = st.d_tsegs; st.args.titems = st.d_titems; st.args.touts = st.d_touts; st.args.tcta = st.d_tcta;
         st.args.status = oz.status;
         if (!st.tasks.empty() || !st.titems.empty()) {   // work-queue counters (also for a stage of thin items only)
             rc = dev_alloc(c, (void**)&st.d_sched, 2 * sizeof(unsigned), "ozaki work queue");
