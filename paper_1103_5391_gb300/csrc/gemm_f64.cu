@@ -48,17 +48,19 @@ struct SegView {
 };
 
 __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const int* skip_flag, int skip_step) {
-    pdl_enter();
-    if (skip_flag != nullptr && skip_step >= *skip_flag) return;   // Krylov space already complete
     __shared__ SegView sv[kTileSegs];
     __shared__ double2 red[GT];
     __shared__ int last;
+    // the tables before the wait for the previous kernel: they are the plan's, no kernel writes them
     const Tile tile = args.tiles[blockIdx.x];
     const Task task = args.tasks[tile.task];   // used at the end only
     const int tid = threadIdx.x;
     const int nseg = tile.seg_hi - tile.seg_lo;
+    Seg seg{};
+    if (tid < nseg) seg = args.segs[tile.seg_lo + tid];
+    pdl_enter();
+    if (skip_flag != nullptr && skip_step >= *skip_flag) return;   // Krylov space already complete
     if (tid < nseg) {
-        const Seg seg = args.segs[tile.seg_lo + tid];
         SegView w;
         w.a = args.bufs[seg.a_buf] + seg.a_off;
         w.b = args.bufs[seg.b_buf] + seg.b_off;

@@ -23,7 +23,11 @@ typedef double2 cplx;   // {re, im}, same layout as tdmrg_c64
 // Programmatic dependent launch.  Kernels are launched with the programmatic-serialisation attribute and
 // every kernel of the library starts with pdl_enter(), which waits until the previous grid of the stream
 // has completed and its memory is visible: the launch of a kernel overlaps the end of the previous one,
-// while every global memory access still follows the previous kernel's completion.  No kernel signals
+// while every global memory access still follows the previous kernel's completion, except the reads of a plan's tables in
+// the slicer and the grouped FP64 GEMM: no kernel writes those, and an upload is no kernel, so a launch behind one waits for
+// it as a whole.  Their two or three loads in a row then run beside the end of the previous kernel (H psi at L=8 8.7 -> 8.2
+// us, at L=32 m=400 with four slices 44.4 -> 44.0 us).  The same for the setup and first tile of the tensor kernel gave
+// nothing, for the segments of the slicer it spilled, for the correction GEMM it cost the launches that are skipped.  No kernel signals
 // its dependents early (measured: blocks parked in the wait beside a running kernel slow it down).
 // Without the launch attribute the wait returns at once.
 #ifdef __CUDACC__

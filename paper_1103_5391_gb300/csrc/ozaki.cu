@@ -125,12 +125,13 @@ __device__ __forceinline__ double2 view_load(const SegView& w, int k, bool use_s
 
 template <int S>
 __global__ void __launch_bounds__(kSliceCT) k_slice(OzSliceArgs sa, GemmArgs g, const int* skip_flag, int skip_step) {
-    pdl_enter();
-    if (skip_flag != nullptr && skip_step >= *skip_flag) return;
     const int gv = blockIdx.x;   // the vector; block-uniform
     if (gv >= sa.nvec_total) return;
     const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+    // the plan's tables before the wait for the previous kernel: no kernel writes them
     const OzSliceJob job = sa.jobs[sa.vjob[gv]];
+    pdl_enter();
+    if (skip_flag != nullptr && skip_step >= *skip_flag) return;
     const int v = gv - job.vec_prefix;
     __shared__ SegView sv[kSegCache];
     __shared__ int spre[kSegCache + 1];
@@ -724,6 +725,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
             long long acc[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) acc[j] = 0;
+            // the exponents while the products are formed (after them: H psi at L=32 m=400 45.0 instead of 44.4 us): a row's in a register, the columns' in a per-warp row of shared
+            // memory; accumulator columns 2j, 2j + 1 hold Re and Im of output column j: this warp's 16 columns are output
+            // columns 8 part .. 8 part + 7
+            const int Ei = row_lane && tile.m0 + row < task.M ? oa.expA[task.aexp0 + tile.m0 + row] - 7 * (S + 1) : 0;
+            if (lane < 16) {
+                const int j = 8 * part + (lane >> 1);
+                sExp[warp - 2][lane] = j < nval ? oa.expB[task.bexp0 + tile.n0 + j] : 0;
+            }
+            __syncwarp();
             bool ok = true;
             for (int k0 = 0; k0 < task.kchunks; k0 += kReadoutChunks, ++b) {
                 const int buf = b & 1;
@@ -748,21 +758,12 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&tempty[buf])) : "memory");
             }
             if (!ok) break;
-            // loads ahead of the stores (a load behind a store to C may not be reordered above it, so
-            // loads inside the store loop would cost one memory latency each): the column exponents
-            // through a per-warp row of shared memory, the beta operands eight at a time
-            {   // accumulator columns 2j, 2j + 1 hold Re and Im of output column j: this warp's 16 columns
-                // are output columns 8 part .. 8 part + 7
-                const int j = 8 * part + (lane >> 1);
-                if (lane < 16) sExp[warp - 2][lane] = j < nval ? oa.expB[task.bexp0 + tile.n0 + j] : 0;
-            }
-            __syncwarp();
             if (row_lane && tile.m0 + row < task.M) {
-                const int Ei = oa.expA[task.aexp0 + tile.m0 + row] - 7 * (S + 1);
                 const int64_t rs = task.trans ? 1 : task.ldc, cs = task.trans ? task.ldc : 1;   // row / column strides
                 double* C = (double*)(g.bufs[task.c_buf] + task.c_off + (int64_t)(tile.m0 + row) * rs + (int64_t)tile.n0 * cs);
 #pragma unroll
-                for (int c4 = 0; c4 < 8; c4 += 4) {   // the beta operands four at a time, ahead of their stores
+                for (int c4 = 0; c4 < 8; c4 += 4) {   // the beta operands four at a time, ahead of their stores (a load behind a
+                                                      // store to C may not be reordered above it)
                     double2 old[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
