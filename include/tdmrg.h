@@ -67,7 +67,7 @@ enum tdmrg_side { TDMRG_LEFT = 0, TDMRG_RIGHT = 1 };
 /* Arithmetic of the superblock products (H psi, excitations, expectation values).
  * Lanczos orthogonalisation, norms, the tridiagonal exponential and rho_L always run in FP64. */
 enum tdmrg_prec {
-    TDMRG_FP64 = 0,        /* complex FP64 products (DMMA tensor-core path)                          */
+    TDMRG_FP64 = 0,        /* complex FP64 products (grouped GEMM on the FP64 units)                  */
     TDMRG_OZAKI_BF16 = 1   /* FP64 operands split into bf16 slices, exact FP32 tensor-core products,
                               FP64 recombination; accuracy set by ozaki_slices                       */
 };
@@ -159,7 +159,7 @@ int tdmrg_evolve(tdmrg_ctx* ctx, int n_up, int n_dn, const tdmrg_c64* phi_d, int
 
 /* Ground state in sector Q (the ground-state targeting of Sec. II.B, needed at every DMRG step):
  * `restarts` times, nk Lanczos steps started at psi_d (full re-orthogonalisation, FP64), the lowest
- * eigenvector of the tridiagonal (bisection on its Sturm count, then inverse iteration, FP64) combined
+ * eigenvector of the tridiagonal (multisection on its Sturm count, a twisted factorisation, FP64) combined
  * in place into psi_d, normalised.  psi_d (device, sector Q) is the start vector on entry and the ground
  * state on return; *energy (host, nullable) receives the lowest Ritz value of the last restart.  The
  * call synchronises the stream once at the end.  Errors: EINVAL (nk outside 2..nk_max, restarts < 1),
@@ -231,8 +231,8 @@ int tdmrg_density_matrix_side(tdmrg_ctx* ctx, int side, int ntargets, const int3
 int tdmrg_rho_size_side(tdmrg_ctx* ctx, int side, int64_t* rho_entries, int64_t* n_evals);
 
 /* Eigendecomposition of a packed rho_L (as written by tdmrg_density_matrix) to FP64 accuracy per sector
- * (dL <= 512): FP32 Jacobi seed, FP64 iterative refinement (Ogita-Aishima) with re-seeding of coupled
- * clusters.
+ * (dL <= 512): FP32 one-sided Jacobi seed on a Cholesky factor, FP64 iterative refinement (Ogita-Aishima)
+ * with one re-seeding of coupled clusters.
  * evals_d (sum dL doubles) gets each sector's eigenvalues in descending order; evecs_d (packed like
  * rho) gets U with rho(q) = U diag(evals) U^dag, column k of U the k-th eigenvector.  This feeds the
  * truncation of Sec. II.B.  Errors: EINVAL, ESTATE, ECUDA. */

@@ -71,7 +71,7 @@ int tdmrg_set_orth_per_sm(tdmrg_ctx* ctx, int k);
 int tdmrg_hpsi_tuning(tdmrg_ctx* ctx, int n_up, int n_dn, int32_t* out);
 
 /* Per sector of one block (side 0: left, 1: right), from the last tdmrg_rho_eig[_side] there: the
- * number of sweeps of the FP32 Jacobi seed and the SM cycles its CTA took (host arrays of the side's
+ * number of sweeps of the FP32 Jacobi seed and the SM cycles its CTA (the first of its cluster) took (host arrays of the side's
  * sector count).  Synchronises the stream.  Errors: EINVAL, ESTATE (no eigendecomposition yet). */
 int tdmrg_eig_stats(tdmrg_ctx* ctx, int side, int32_t* sweeps, int64_t* cycles);
 

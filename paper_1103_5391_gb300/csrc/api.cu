@@ -148,8 +148,8 @@ int check_device_status(tdmrg_ctx* c) {
     if (rc) return rc;
     if (st) {
         cudaMemset(c->dstatus, 0, sizeof(int));
-        return fail(c, TDMRG_ETIMEOUT, "a bounded device wait ran out (tensor-core mbarrier, Lanczos grid barrier or "
-                                       "the wait probe); results are invalid");
+        return fail(c, TDMRG_ETIMEOUT, "a bounded device wait ran out (tensor-core or seed mbarrier, Lanczos "
+                                       "exchange or the wait probe); results are invalid");
     }
     return TDMRG_OK;
 }
