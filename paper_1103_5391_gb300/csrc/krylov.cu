@@ -106,10 +106,16 @@ __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, in
                                                  int nk, OrthSlots slots) {
     pdl_enter();
     clear_slots(slots);
-    __shared__ double2 h[1];
-    reduce_coeffs(part, 1, h);
-    const double b0 = sqrt(h[0].x);
-    const double inv = b0 > 0.0 ? 1.0 / b0 : 0.0;
+    __shared__ double sb[2];
+    if (threadIdx.x < 32) {   // one square root and one division per block: each is ~20 FP64 instructions of 64 cycles
+        const double2 t = warp_total(part);
+        if (threadIdx.x == 0) {
+            sb[0] = sqrt(t.x);
+            sb[1] = sb[0] > 0.0 ? 1.0 / sb[0] : 0.0;
+        }
+    }
+    __syncthreads();
+    const double b0 = sb[0], inv = sb[1];
     int64_t lo, hi;
     chunk_of(n, lo, hi);
     for (int64_t i = lo + threadIdx.x; i < hi; i += NT) { const double2 v = phi[i]; v0[i] = make_double2(v.x * inv, v.y * inv); }
@@ -745,57 +751,63 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
 }
 
 struct TargetPtrs { cplx* p[16]; };
-struct CombineList { cplx* p[8]; int row[8]; };   // targets of one combine launch and their coefficient rows
+struct CombineList { cplx* p[16]; int row[16]; int n; };   // targets and their coefficient rows
 
-// targets p[x][i] = sum_k coef[row[x]][k] v_k[i] for x < NX: one pass over V.  NX is exact (no
-// predicated FP64 work for absent targets).
-template <int NX>
-__global__ void __launch_bounds__(256) k_combine(const cplx* __restrict__ V, int64_t n, const int* __restrict__ flags,
-                                                  const cplx* __restrict__ coef, CombineList tg) {
-    pdl_enter();
-    __shared__ double2 cf[NX][32];
-    const int nu = flags[0];
-    for (int e = threadIdx.x; e < NX * 32; e += blockDim.x) cf[e / 32][e % 32] = coef[tg.row[e / 32] * 32 + e % 32];
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double2 acc[NX];
+// sum_k c[k] v_k[i] over nu vectors, four loads ahead of their use
+__device__ __forceinline__ double2 combine_one(const cplx* __restrict__ V, int64_t n, int64_t i, const double2* c, int nu) {
+    double2 acc = make_double2(0.0, 0.0);
+    auto add = [&](double2 w, double2 v) {
+        acc.x = fma(w.x, v.x, fma(-w.y, v.y, acc.x));
+        acc.y = fma(w.x, v.y, fma(w.y, v.x, acc.y));
+    };
+    int k = 0;
+    for (; k + 4 <= nu; k += 4) {
+        double2 v[4];
 #pragma unroll
-        for (int x = 0; x < NX; ++x) acc[x] = make_double2(0.0, 0.0);
-        for (int k = 0; k < nu; ++k) {
-            const double2 v = V[(int64_t)k * n + i];
+        for (int u = 0; u < 4; ++u) v[u] = V[(int64_t)(k + u) * n + i];
 #pragma unroll
-            for (int x = 0; x < NX; ++x) {
-                const double2 c = cf[x][k];
-                acc[x].x = fma(c.x, v.x, fma(-c.y, v.y, acc[x].x));
-                acc[x].y = fma(c.x, v.y, fma(c.y, v.x, acc[x].y));
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < NX; ++x) tg.p[x][i] = acc[x];
+        for (int u = 0; u < 4; ++u) add(c[k + u], v[u]);
     }
+    for (; k < nu; ++k) add(c[k], V[(int64_t)k * n + i]);
+    return acc;
 }
 
-// The targets listed in rows (coefficient row of each), eight per launch; returns the launch count.
-int launch_combine(const cplx* V, int64_t n, const int* flags, const cplx* coef, const std::vector<int>& rows,
-                   const TargetPtrs& tg, int grid, cudaStream_t s) {
-    const int cnt = (int)rows.size();
-    int launches = 0;
-    for (int x0 = 0; x0 < cnt; x0 += 8) {
-        CombineList t{};
-        for (int x = x0; x < std::min(cnt, x0 + 8); ++x) { t.p[x - x0] = tg.p[rows[x]]; t.row[x - x0] = rows[x]; }
-        switch (std::min(8, cnt - x0)) {
-            case 1: launch_pdl(k_combine<1>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 2: launch_pdl(k_combine<2>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 3: launch_pdl(k_combine<3>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 4: launch_pdl(k_combine<4>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 5: launch_pdl(k_combine<5>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 6: launch_pdl(k_combine<6>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            case 7: launch_pdl(k_combine<7>, grid, 256, 0, s, V, n, flags, coef, t); break;
-            default: launch_pdl(k_combine<8>, grid, 256, 0, s, V, n, flags, coef, t); break;
-        }
-        ++launches;
+// targets p[x][i] = sum_k coef[row[x]][k] v_k[i], one target per blockIdx.y.  What bounds it is FP64 issue (4 instructions
+// of 64 cycles per k and element), so what counts is that every sub-partition has work and an even share: with all targets
+// in one thread's registers and V read once, 5332 elements kept 167 of 608 sub-partitions busy for 9200 cycles and loads
+// came one at a time.  The second and third read of V come from L2.  Measured with n_K = 12 and three targets at
+// D = 5332, n_K = 10 at D = 46,868: the whole advance 417.7 -> 410.9 us and 679.0 -> 674.4 us.
+constexpr int CBT = 128;
+__global__ void __launch_bounds__(CBT) k_combine(const cplx* __restrict__ V, int64_t n, const int* __restrict__ flags,
+                                                 const cplx* __restrict__ coef, CombineList tg) {
+    pdl_enter();
+    __shared__ double2 cf[32];
+    const int nu = flags[0], x = blockIdx.y;
+    if (threadIdx.x < 32) cf[threadIdx.x] = coef[tg.row[x] * 32 + threadIdx.x];
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * CBT + threadIdx.x; i < n; i += (int64_t)gridDim.x * CBT) tg.p[x][i] = combine_one(V, n, i, cf, nu);
+}
+
+// The targets listed in rows (coefficient row of each).  Of segmented targets in one buffer the last is formed, as the
+// blocks of different targets run in any order.
+CombineList combine_list(const std::vector<int>& rows, const TargetPtrs& tg) {
+    CombineList t{};
+    for (size_t x = 0; x < rows.size(); ++x) {
+        bool again = false;
+        for (size_t y = x + 1; y < rows.size(); ++y) again |= tg.p[rows[y]] == tg.p[rows[x]];
+        if (again) continue;
+        t.p[t.n] = tg.p[rows[x]];
+        t.row[t.n++] = rows[x];
     }
-    return launches;
+    return t;
+}
+int launch_combine(const cplx* V, int64_t n, const int* flags, const cplx* coef, const std::vector<int>& rows,
+                   const TargetPtrs& tg, int sms, cudaStream_t s) {
+    const CombineList t = combine_list(rows, tg);
+    if (t.n == 0) return 0;
+    const int grid = (int)std::min<int64_t>((n + CBT - 1) / CBT, 16L * sms);
+    launch_pdl(k_combine, dim3(grid, t.n), CBT, 0, s, V, n, flags, coef, t);
+    return 1;
 }
 
 // ---- segmented mode: the start vector's norm, v_0 and the targets per segment --------------------
@@ -813,17 +825,20 @@ __global__ void __launch_bounds__(NT) k_init_v0_seg(const cplx* __restrict__ phi
                                                     int nk, OrthSlots slots) {
     pdl_enter();
     clear_slots(slots);
-    __shared__ double b0s;
+    __shared__ double sb[2];
     const int sg = tb.cta_seg[blockIdx.x], c0 = tb.seg_cta0[sg], c1 = tb.seg_cta0[sg + 1];
     if (threadIdx.x < 32) {   // the segment's partials in a fixed order
         double t = 0.0;
         for (int b = c0 + (int)threadIdx.x; b < c1; b += 32) t += part[b].x;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (threadIdx.x == 0) b0s = sqrt(t);
+        if (threadIdx.x == 0) {
+            sb[0] = sqrt(t);
+            sb[1] = sb[0] > 0.0 ? 1.0 / sb[0] : 0.0;
+        }
     }
     __syncthreads();
-    const double b0 = b0s, inv = b0 > 0.0 ? 1.0 / b0 : 0.0;
+    const double b0 = sb[0], inv = sb[1];
     const int64_t lo = tb.cta_lo[blockIdx.x], hi = tb.cta_hi[blockIdx.x];
     for (int64_t i = lo + threadIdx.x; i < hi; i += NT) { const double2 v = phi[i]; v0[i] = make_double2(v.x * inv, v.y * inv); }
     if ((int)blockIdx.x == c0 && threadIdx.x == 0) {
@@ -833,54 +848,16 @@ __global__ void __launch_bounds__(NT) k_init_v0_seg(const cplx* __restrict__ phi
     }
 }
 
-// targets[x] over each block's range with its segment's coefficients (one pass over V)
-template <int NX>
-__global__ void __launch_bounds__(256) k_combine_seg(const cplx* __restrict__ V, int64_t n, SegTab tb,
-                                                     const int* __restrict__ flags, const cplx* __restrict__ coef, int x0,
-                                                     TargetPtrs tg) {
+// The targets over each block's range with its segment's coefficients, one target per blockIdx.y
+__global__ void __launch_bounds__(CBT) k_combine_seg(const cplx* __restrict__ V, int64_t n, SegTab tb, const int* __restrict__ flags,
+                                                     const cplx* __restrict__ coef, CombineList tg) {
     pdl_enter();
-    __shared__ double2 cf[NX][32];
-    const int sg = tb.cta_seg[blockIdx.x];
-    const int nu = flags[sg * kFlagStride];
-    const cplx* cs = coef + (int64_t)sg * kCoefStride;
-    for (int e = threadIdx.x; e < NX * 32; e += blockDim.x) cf[e / 32][e % 32] = cs[(x0 + e / 32) * 32 + e % 32];
+    __shared__ double2 cf[32];
+    const int sg = tb.cta_seg[blockIdx.x], nu = flags[sg * kFlagStride], x = blockIdx.y;
+    if (threadIdx.x < 32) cf[threadIdx.x] = coef[(int64_t)sg * kCoefStride + tg.row[x] * 32 + threadIdx.x];
     __syncthreads();
     const int64_t lo = tb.cta_lo[blockIdx.x], hi = tb.cta_hi[blockIdx.x];
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        double2 acc[NX];
-#pragma unroll
-        for (int x = 0; x < NX; ++x) acc[x] = make_double2(0.0, 0.0);
-        for (int k = 0; k < nu; ++k) {
-            const double2 v = V[(int64_t)k * n + i];
-#pragma unroll
-            for (int x = 0; x < NX; ++x) {
-                const double2 c = cf[x][k];
-                acc[x].x = fma(c.x, v.x, fma(-c.y, v.y, acc[x].x));
-                acc[x].y = fma(c.x, v.y, fma(c.y, v.x, acc[x].y));
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < NX; ++x) tg.p[x][i] = acc[x];
-    }
-}
-
-cudaError_t launch_combine_seg(const cplx* V, int64_t n, const SegTab& tb, int grid, const int* flags, const cplx* coef,
-                               int n_v, const TargetPtrs& tg, cudaStream_t s) {
-    for (int x0 = 0; x0 < n_v; x0 += 8) {
-        TargetPtrs t{};
-        for (int x = x0; x < n_v; ++x) t.p[x - x0] = tg.p[x];
-        switch (std::min(8, n_v - x0)) {
-            case 1: launch_pdl(k_combine_seg<1>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 2: launch_pdl(k_combine_seg<2>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 3: launch_pdl(k_combine_seg<3>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 4: launch_pdl(k_combine_seg<4>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 5: launch_pdl(k_combine_seg<5>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 6: launch_pdl(k_combine_seg<6>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            case 7: launch_pdl(k_combine_seg<7>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-            default: launch_pdl(k_combine_seg<8>, grid, 256, 0, s, V, n, tb, flags, coef, x0, t); break;
-        }
-    }
-    return cudaGetLastError();
+    for (int64_t i = lo + threadIdx.x; i < hi; i += CBT) tg.p[x][i] = combine_one(V, n, i, cf, nu);
 }
 
 __global__ void __launch_bounds__(NT) k_dot2(const cplx* __restrict__ x, const cplx* __restrict__ y, int64_t n,
@@ -1074,8 +1051,7 @@ int evolve(tdmrg_ctx* c, int a, int b, const cplx* phi, int n_v, const double* t
     }
     TargetPtrs tg{};
     for (int x = 0; x < n_v; ++x) tg.p[x] = targets[x];
-    int grid = (int)std::min<int64_t>((n + 255) / 256, 4L * c->num_sms);
-    c->launches += 1 + launch_combine(k->V, n, k->flags, k->coef, rows, tg, grid, s);
+    c->launches += 1 + launch_combine(k->V, n, k->flags, k->coef, rows, tg, c->num_sms, s);
     c->last_krylov = k;
     return cuda_check(c, cudaGetLastError(), "evolve launch");
 }
@@ -1090,8 +1066,7 @@ int ground_state(tdmrg_ctx* c, int a, int b, cplx* psi, int nk, int restarts, do
         launch_pdl(k_tridiag_min, 1, kMinThreads, 0, c->stream, k->tri, k->flags, k->coef);
         TargetPtrs tg{};
         tg.p[0] = psi;
-        const int grid = (int)std::min<int64_t>((k->n + 255) / 256, 4L * c->num_sms);
-        launch_combine(k->V, k->n, k->flags, k->coef, std::vector<int>{0}, tg, grid, c->stream);
+        launch_combine(k->V, k->n, k->flags, k->coef, std::vector<int>{0}, tg, c->num_sms, c->stream);
         c->launches += 2;
         rc = cuda_check(c, cudaGetLastError(), "ground-state launch");
         if (rc) return rc;
@@ -1228,8 +1203,11 @@ int evolve_segments(tdmrg_ctx* c, int a, int b, const cplx* phi, int nseg, const
     launch_pdl(k_tridiag_exp, nseg, 32, 0, s, tri, flags, tt, n_v, coef);
     TargetPtrs tg{};
     for (int x = 0; x < n_v; ++x) tg.p[x] = targets[x];
-    launch_combine_seg(k->V, n, tb, G, flags, coef, n_v, tg, s);
-    c->launches += 1 + (n_v + 7) / 8;
+    std::vector<int> rows(n_v);
+    for (int x = 0; x < n_v; ++x) rows[x] = x;
+    const CombineList cl = combine_list(rows, tg);
+    launch_pdl(k_combine_seg, dim3(G, cl.n), CBT, 0, s, k->V, n, tb, flags, coef, cl);
+    c->launches += 2;
     return cuda_check(c, cudaGetLastError(), "evolve_segments launch");
 }
 
