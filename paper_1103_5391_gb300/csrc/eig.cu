@@ -421,12 +421,12 @@ constexpr float kSeedStop2 = 2.5e-7f;      // ... and sweeps end after one whose
 constexpr int kSeedSweeps = 15;
 
 // v 2^-e rounded to FP32, by integer instructions (conversions from double run on the narrow FP64 pipe);
-// values below 2^-126 give 0
+// zero and subnormal v give 0 whatever e (a zero sector has e = -1023), and so do results below 2^-126
 __device__ __forceinline__ float f32_of(double v, int e) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
-    const int ex = (int)((hi >> 20) & 0x7FFu) - 896 - e;
-    if (ex <= 0) return 0.f;
+    const int bx = (int)((hi >> 20) & 0x7FFu), ex = bx - 896 - e;
+    if (bx == 0 || ex <= 0) return 0.f;
     return __uint_as_float((hi & 0x80000000u) | ((((unsigned)ex << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u)));
 }
 // the double equal to v (subnormals give 0), by integer instructions
