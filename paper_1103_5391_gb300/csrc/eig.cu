@@ -19,7 +19,8 @@
 //      sixth is still above it (density matrices of DMRG blocks whose spectra span the whole FP64 range in
 //      large degenerate multiplets), two last steps only orthonormalise W (E = R / 2 for every pair, a
 //      Newton-Schulz step: orthogonality error eps -> ~eps^2 -> rounding), so that the kept states always
-//      form an orthonormal basis and the renormalised operators are projections.  At
+//      form an orthonormal basis and the renormalised operators are projections; the sixth itself turns no pair by more
+//      than 1e-5 (kLastTurn), as a large turn would leave more than those two steps can orthonormalise.  At
 //      iteration 1 a sector whose clustered pairs stay coupled is re-seeded instead (FP32 two-sided Jacobi
 //      on S with a relative criterion, k_jacobi32).  The iterate is kept as W = X^H, so every product
 //      is a plain or conjugate-transposed GEMM operand;
@@ -54,6 +55,12 @@ constexpr float kReseedFloor = 1e-14f; // ... and |S_pq| > kReseedFloor ||rho||_
 __host__ __device__ constexpr bool reseed_iter(int it) { return it == 1; }
 constexpr double kNearGap = 1e-11, kNearNum = 2e-15;   // in units of ||rho||_F, see k_oa_update
 constexpr double kSmallTurn = 3e-3;
+// Pairs that the last iteration would turn by more than this are clusters there: no iteration follows that could mend the
+// second order of the turn.  At 20 to 30 decades such a pair is rounding over a gap of a few 1e-14 ||rho||, and a turn by
+// 0.1 left eigenvectors with orthogonality errors up to 4e-7 behind the two orthonormalisation steps.  Simulated over
+// graded spectra and multiplets of 14 to 30 decades, n = 12 ... 110, the worst orthogonality and reconstruction:
+// 8e-7 and 3e-9 ||rho|| without the limit, 2e-14 and 2e-11 with 1e-3, 2e-14 and 2e-11 (others 1e-12) with 1e-5.
+constexpr double kLastTurn = 1e-5;
 constexpr double kTolE = 1e-7;   // |E| above this: the next error (~|E|^2) may exceed ~1e-14
 
 struct EigTables {
@@ -953,7 +960,8 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
             // Inside delta: in the first two iterations a pair whose correction is small (first-order perturbation theory
             // holds for it) is corrected all the same.  A close pair whose numerator is rounding (an exact multiplet in
             // an iterate that has converged while other sectors go on) would be turned by noise / noise: a cluster.
-            const bool near = (gap <= delta && (it >= 2 || nm > kSmallTurn * gap)) || (gap <= kNearGap * fro && nm <= kNearNum * fro);
+            const bool near = (gap <= delta && (it >= 2 || nm > kSmallTurn * gap)) || (gap <= kNearGap * fro && nm <= kNearNum * fro) ||
+                              (it == kOaIters - 1 && nm > kLastTurn * gap);
             if (!orth_only && i != j && !near) {
                 const double inv = 1.0 / (li - lj);
                 ev = make_double2(num.x * inv, num.y * inv);
