@@ -643,16 +643,31 @@ __global__ void __launch_bounds__(32) k_tridiag_exp_eq(double* __restrict__ tri,
     }
 }
 
+// The pair times one power of two, by integer instructions (the FP64 pipe is what bounds the chains below): the larger
+// between 1/2 and 1, a zero or what falls below 2^-1022 gives 0.
+__device__ __forceinline__ void rescale_pair(double& x, double& y) {
+    const int hx = __double2hiint(x), hy = __double2hiint(y);
+    const int ex = (hx >> 20) & 0x7FF, ey = (hy >> 20) & 0x7FF, s = 1022 - max(ex, ey);
+    x = ex == 0 || ex + s <= 0 ? 0.0 : __hiloint2double(hx + (s << 20), __double2loint(x));
+    y = ey == 0 || ey + s <= 0 ? 0.0 : __hiloint2double(hy + (s << 20), __double2loint(y));
+}
+
 // Lowest eigenpair of the Lanczos tridiagonal T (ground-state targeting, Sec. II.B), FP64, n <= 32.
 // The eigenvalue by multisection: x lies below it exactly when the leading minors d_k = det(T_k - x) are all
-// positive, d_k = (alpha_k - x) d_{k-1} - beta_{k-1}^2 d_{k-2} with T scaled by a power of two to norm <= 1 (|d_k| <= 3^k);
-// 128 threads try 128 points of the bracket at once, so it shrinks 129-fold in one chain of n steps.  Bisection on
-// the Sturm count with divisions took ~52 chains of n FP64 divisions (~700 cycles each) in one thread: 650 us at
-// n = 32, 30 us now (bound by the FP64 pipe: three instructions a step and warp).
+// positive, d_k = (alpha_k - x) d_{k-1} - beta_{k-1}^2 d_{k-2} with T scaled by a power of two to norm <= 1.
+// 128 threads try 128 points of the bracket at once, so it shrinks 129-fold in one chain of n steps.  Only the signs
+// count, so the pair (d_{k-1}, d_k) is scaled by a power of two every four steps: without it the minors of a T whose
+// spread is small against its norm (a constant or a penalty in H) underflow from ||T|| / 1e10 on, and the bracket walks
+// to an end of the Gershgorin interval.
+// Then the eigenvalue is known to 4e-16 of its size, which may be as much as the distance to the next.  The rest works on
+// T - lambda, whose differences are rounded relative to themselves: where the spread of T about lambda calls for it, the
+// bracket around 0 is narrowed to 4e-15 of that spread (no step for an ordinary spectrum).
 // The eigenvector by the twisted factorisation of T - lambda (Dhillon 1997): pivots p_k from the top and m_k from the
-// bottom (ratios of the leading and trailing minors), the twist r where |p_k + m_k - (alpha_k - lambda)| is smallest,
-// z_r = 1, z_k = -(beta_k / p_k) z_{k+1} above and z_k = -(beta_{k-1} / m_k) z_{k-1} below: one lane per component,
-// products by scans.  coef[0][k] = z_k / |z| (real), tri[T_EMIN] = lambda.
+// bottom (ratios of neighbouring leading and trailing minors), the twist r where |p_k + m_k - (alpha_k - lambda)| is
+// smallest, z_r = 1, z_k = -(beta_k / p_k) z_{k+1} above and z_k = -(beta_{k-1} / m_k) z_{k-1} below: one lane per
+// component, products by scans.  A pivot below eps |lambda| (a leading or trailing block with the same eigenvalue, or n = 1)
+// is replaced by that, in the minor itself, so that the pivots after it follow.  coef[0][k] = z_k / |z| (real),
+// tri[T_EMIN] = lambda.  ~30 us at n = 32, bound by the FP64 pipe: three instructions of 64 cycles a step and warp.
 constexpr int kMinThreads = 128;
 __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict__ tri, const int* __restrict__ flags,
                                                               cplx* __restrict__ coef) {
@@ -663,7 +678,7 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
         if (tid == 0) tri[T_EMIN] = 0.0;
         return;
     }
-    __shared__ double sa[32], sb2[32], sx[kMinThreads + 2], sd[2][32];
+    __shared__ double sa[32], sb2[32], sx[kMinThreads + 2], sd[2][32], sq[2][32];
     // every warp: alpha_l, beta_l (couples l and l + 1) and the Gershgorin interval
     double al = l < n ? tri[T_ALPHA + l] : 0.0, be = l < n - 1 ? tri[T_BETA + l] : 0.0;
     double bm = __shfl_up_sync(0xffffffffu, be, 1);
@@ -678,11 +693,12 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
     const double nrm = fmax(fabs(lo), fabs(hi));
     int e2 = 0;
     frexp(nrm, &e2);
+    e2 = max(e2, -1000);   // 2^-e2 stays finite
     const double sc = nrm > 0.0 ? ldexp(1.0, -e2) : 1.0, us = nrm > 0.0 ? ldexp(1.0, e2) : 1.0;
     al *= sc; be *= sc; bm *= sc; lo *= sc; hi *= sc;
     if (tid < 32) { sa[l] = al; sb2[l] = be * be; }
     __syncthreads();
-    for (int it = 0; it < 12 && hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) {
+    auto narrow = [&]() {   // the bracket [lo, hi] shrinks 129-fold
         const double x = fma(hi - lo, (tid + 1) * (1.0 / (kMinThreads + 1)), lo);
         double d0 = 1.0, d1 = sa[0] - x;
         bool below = d1 > 0.0;
@@ -691,6 +707,7 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
             d0 = d1;
             d1 = d2;
             below = below && d2 > 0.0;
+            if ((k & 3) == 0) rescale_pair(d0, d1);
         }
         sx[tid + 1] = x;
         if (tid == 0) { sx[0] = lo; sx[kMinThreads + 1] = hi; }
@@ -698,31 +715,45 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
         lo = sx[c];
         hi = sx[c + 1];
         __syncthreads();
-    }
+    };
+    for (int it = 0; it < 28 && hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) narrow();
+    // T - base from here on; the counts so far are exact for entries off by a few eps of the spread
+    const double base = 0.5 * (lo + hi);
+    al -= base;
+    double sp = l < n ? fabs(al) + fabs(be) + fabs(bm) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sp = fmax(sp, __shfl_xor_sync(0xffffffffu, sp, o));
+    if (tid < 32) sa[l] = al;
+    lo = lo - base - 1e-15 * sp;
+    hi = hi - base + 1e-15 * sp;
+    __syncthreads();
+    for (int it = 0; it < 12 && hi - lo > 4e-15 * sp; ++it) narrow();
     if (tid >= 32) return;
     const double lam = 0.5 * (lo + hi);
-    if (l < 2) {   // lane 0: leading minors, lane 1: trailing minors of T - lambda
-        double d0 = 1.0, d1 = sa[l == 0 ? 0 : n - 1] - lam;
-        sd[l][l == 0 ? 0 : n - 1] = d1;
-        for (int k = 1; k < n; ++k) {
+    al -= lam;
+    sa[l] = al;
+    __syncwarp();
+    const double pmin = fmax(2.2e-16 * fabs(base + lam), 0x1p-200);
+    if (l < 2) {   // lane 0: leading minors, lane 1: trailing minors of T - lambda, each with the one before it
+        double d0 = 0.0, d1 = 1.0, b2 = 0.0;
+        for (int k = 0; k < n; ++k) {
             const int i = l == 0 ? k : n - 1 - k;
-            const double d2 = fma(sa[i] - lam, d1, -sb2[l == 0 ? k - 1 : i] * d0);
+            double d2 = fma(sa[i], d1, -b2 * d0);
+            const double lim = pmin * d1;
+            if (!(fabs(d2) >= fabs(lim))) d2 = copysign(lim, d2);
+            sd[l][i] = d2;
+            sq[l][i] = d1;
             d0 = d1;
             d1 = d2;
-            sd[l][i] = d1;
+            b2 = l == 0 ? sb2[i] : (i > 0 ? sb2[i - 1] : 0.0);
+            if ((k & 3) == 3) rescale_pair(d0, d1);
         }
     }
     __syncwarp();
-    // a pivot that vanishes (lambda an eigenvalue of a leading or trailing block too, or n = 1) is replaced by eps ||T||
-    constexpr double pmin = 2.2e-16;
-    auto pivot = [&](double d, double prev) {
-        const double q = prev != 0.0 ? d / prev : d;
-        return fabs(q) < pmin ? (q < 0.0 ? -pmin : pmin) : q;
-    };
     const bool in = l < n;
-    const double p = in ? pivot(sd[0][l], l > 0 ? sd[0][l - 1] : 1.0) : 1.0;
-    const double m = in ? pivot(sd[1][l], l < n - 1 ? sd[1][l + 1] : 1.0) : 1.0;
-    double g = in ? fabs(p + m - (al - lam)) : 1e300;
+    const double p = in ? sd[0][l] / sq[0][l] : 1.0;
+    const double m = in ? sd[1][l] / sq[1][l] : 1.0;
+    double g = in ? fabs(p + m - al) : 1e300;
     int tw = l;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {   // the smallest, ties to the first
@@ -747,7 +778,7 @@ __global__ void __launch_bounds__(kMinThreads) k_tridiag_min(double* __restrict_
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
     if (in) coef[l] = make_double2(zs / sqrt(nn), 0.0);
-    if (l == 0) tri[T_EMIN] = lam * us;
+    if (l == 0) tri[T_EMIN] = (base + lam) * us;
 }
 
 struct TargetPtrs { cplx* p[16]; };
