@@ -10,9 +10,9 @@
 //         E_ij = (S_ij + lambda_j R_ij) / (lambda_j - lambda_i)   if |lambda_i - lambda_j| > delta,
 //         E_ij = R_ij / 2 otherwise (and on the diagonal),  delta = 2 (||S - diag(lambda)|| + ||rho|| ||R||),
 //         X <- X (I + E);
-//      inside delta the first two iterations still correct pairs with |E_ij|, |E_ji| <= 3e-3 (simulated with these
-//      seeds: 3.0 instead of 4.9 iterations at n = 152 with a spectrum over four decades, 2.1 instead of 3.1 at n = 60;
-//      multiplets and random graded spectra end no further off than with the global test alone);
+//      inside delta the first two iterations still correct pairs with |E_ij|, |E_ji| <= 3e-3 that are no closer than
+//      2e-7 ||rho||, in sectors up to 160 states (simulated with these seeds: 3.0 instead of 4.9 iterations at n = 152 with
+//      a spectrum over four decades, 2.1 instead of 3.1 at n = 60);
 //      convergence is quadratic: from the FP32 seed two iterations reach rounding level;
 //      up to four more run (decided on the device, launched regardless) while the last correction is
 //      above 1e-7, as for near-degenerate pairs that the first iteration treats as a cluster.  If the
@@ -55,6 +55,13 @@ constexpr float kReseedFloor = 1e-14f; // ... and |S_pq| > kReseedFloor ||rho||_
 __host__ __device__ constexpr bool reseed_iter(int it) { return it == 1; }
 constexpr double kNearGap = 1e-11, kNearNum = 2e-15;   // in units of ||rho||_F, see k_oa_update
 constexpr double kSmallTurn = 3e-3;
+// In units of ||rho||_F: pairs closer than this are not corrected inside delta, nor is any in a sector above 160 states: what
+// couples close states of different multiplets at first is of second order in the seed's errors, and correcting it early
+// costs an iteration that is then missing at the end (multiplets over 12 decades, n = 170 and 200: reconstruction up to
+// 3e-10 ||rho|| off; 6e-13 now).  Above 160 the seed takes ten times as long as an iteration.  Measured below that with
+// 0 / 2e-7 / 5e-7: multiplets at n = 12 ... 60 up to 2e-11 / 3e-12 / 3e-13 off, at n = 64 ... 152 9e-13 / 6e-13 / 3e-13 in the
+// geometric mean; the decomposition at L=48 m=1000 2953 / 2953 / 3578 us.
+constexpr double kMultipletGap = 2e-7;
 // Pairs that the last iteration would turn by more than this are clusters there: no iteration follows that could mend the
 // second order of the turn.  At 20 to 30 decades such a pair is rounding over a gap of a few 1e-14 ||rho||, and a turn by
 // 0.1 left eigenvectors with orthogonality errors up to 4e-7 behind the two orthonormalisation steps.  Simulated over
@@ -946,6 +953,8 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
     }
     bool big = false, clus = false;
     const bool orth_only = it >= kOaIters;   // E = R / 2: W <- (I + R / 2) W, a Newton-Schulz step
+    const bool last = it == kOaIters - 1;
+    const double turn = last ? kLastTurn : kSmallTurn, close = n > kSeedSmemN ? delta : kMultipletGap * fro;
 #pragma unroll
     for (int u = 0; u < kOaPer; ++u) {
         const int e = item.y + threadIdx.x + kOaThreads * u;
@@ -958,10 +967,12 @@ __global__ void __launch_bounds__(kOaThreads) k_oa_update(const cplx* __restrict
             // the larger numerator of E_ij and E_ji, so that both take the same branch
             const double nm = fmax(fmax(fabs(num.x), fabs(num.y)), fmax(fabs(sv[u].x + lj * r.x), fabs(sv[u].y + lj * r.y)));
             // Inside delta: in the first two iterations a pair whose correction is small (first-order perturbation theory
-            // holds for it) is corrected all the same.  A close pair whose numerator is rounding (an exact multiplet in
-            // an iterate that has converged while other sectors go on) would be turned by noise / noise: a cluster.
-            const bool near = (gap <= delta && (it >= 2 || nm > kSmallTurn * gap)) || (gap <= kNearGap * fro && nm <= kNearNum * fro) ||
-                              (it == kOaIters - 1 && nm > kLastTurn * gap);
+            // holds for it) is corrected all the same, unless it is as close as the members of a multiplet.  A close pair
+            // whose numerator is rounding (an exact multiplet in an iterate that has converged while other sectors go on)
+            // would be turned by noise / noise: a cluster, and so is a pair that the last iteration would turn far.
+            const bool far = nm > turn * gap;
+            const bool near = (gap <= delta && (it >= 2 || far || gap <= close)) || (gap <= kNearGap * fro && nm <= kNearNum * fro) ||
+                              (last && far);
             if (!orth_only && i != j && !near) {
                 const double inv = 1.0 / (li - lj);
                 ev = make_double2(num.x * inv, num.y * inv);
