@@ -84,8 +84,8 @@ void drop_krylov(tdmrg_ctx* c) {
         size_t n = (size_t)k.n;
         dev_free(c, k.V, (k.nk + 1) * n * sizeof(cplx));
         dev_free(c, k.w, n * sizeof(cplx));
-        dev_free(c, k.partA, 64 * kRedBlocks * sizeof(double2));
-        dev_free(c, k.partB, 64 * kRedBlocks * sizeof(double2));
+        dev_free(c, k.partA, kPartBytesA);
+        dev_free(c, k.partB, kPartBytesB);
         dev_free(c, k.tri, 128 * sizeof(double));
         dev_free(c, k.flags, 4 * sizeof(int));
         dev_free(c, k.coef, (16 + 32) * 32 * sizeof(cplx));

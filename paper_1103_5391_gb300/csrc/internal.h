@@ -285,8 +285,8 @@ struct KrylovWork {     // device workspace of tdmrg_evolve for one (Q, nk)
     int nk = 0;
     cplx* V = nullptr;          // (nk + 1) x n Lanczos vectors
     cplx* w = nullptr;          // n
-    double2* partA = nullptr;   // reduction partials
-    double2* partB = nullptr;
+    double2* partA = nullptr;   // reduction partials: first pass (two rows) and the start vector's norm
+    double2* partB = nullptr;   // two buffers of second-pass and two of third-pass partials, kPartRowsPass rows each
     double* tri = nullptr;      // alpha[32], beta[32], beta0, resid, err
     int* flags = nullptr;       // n_used
     cplx* coef = nullptr;       // [x][k] Krylov coefficients
@@ -471,6 +471,8 @@ int segments_info(tdmrg_ctx* c, int n_up, int n_dn, int nk, int nseg, int* nk_us
 cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* partials, int nblk,
                              cplx* out, int normalise, cudaStream_t s);
 constexpr int kRedBlocks = 304;   // 2 x 152 SMs: fixed, so reductions are deterministic
+constexpr int kPartRowsPass = 33; // partials of 32 Krylov vectors and the norm
+constexpr size_t kPartBytesA = 3 * kRedBlocks * sizeof(double2), kPartBytesB = 4 * (size_t)kPartRowsPass * kRedBlocks * sizeof(double2);
 
 // density.cu
 // With `grouped` (a side whose eigensolver runs two sector groups, eig_prepare done), the rho blocks of the

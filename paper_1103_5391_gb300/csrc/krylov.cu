@@ -89,14 +89,16 @@ __global__ void __launch_bounds__(NT) k_norm2(const cplx* __restrict__ x, int64_
 }
 
 // The partial-sum slots of the orthogonalisation steps, emptied before a Lanczos run (rows of grid blocks: the first
-// pass's two, then both buffers of the second pass's).
-struct OrthSlots { double2 *partA, *partB0, *partB1; int rows, grid; };
+// pass's two, then both buffers of the second and of the third pass's).
+struct OrthSlots { double2 *partA, *partB[2], *partC[2]; int rows, grid; };
 __device__ __forceinline__ void clear_slots(const OrthSlots& sl) {
     const double e = __longlong_as_double(0x7ff4dead7ff4deadll);
     const int n = sl.rows * sl.grid;
     for (int i = blockIdx.x * NT + threadIdx.x; i < n; i += gridDim.x * NT) {
-        sl.partB0[i] = make_double2(e, e);
-        sl.partB1[i] = make_double2(e, e);
+        sl.partB[0][i] = make_double2(e, e);
+        sl.partB[1][i] = make_double2(e, e);
+        sl.partC[0][i] = make_double2(e, e);
+        sl.partC[1][i] = make_double2(e, e);
         if (i < 2 * sl.grid) sl.partA[i] = make_double2(e, e);
     }
 }
@@ -130,9 +132,13 @@ __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, in
 // Two exchanges of partial sums between all blocks separate: (A) the first-pass dots h1_k = <v_k|w>; (B) w' = w -
 // sum h1_k v_k, the second-pass dots h2_k = <v_k|w'> and ||w'||^2; (C) beta = ||w' - sum h2_k v_k|| and
 // v_{j+1} = (w' - sum h2_k v_k) / beta.  Since h2 holds the projections of w' on orthonormal v_k,
-// ||w' - sum h2_k v_k||^2 = ||w'||^2 - sum |h2_k|^2 (h2 is at rounding level after the first pass, so
+// ||w' - sum h2_k v_k||^2 = ||w'||^2 - sum |h2_k|^2 (h2 is at the FP32 rounding level of the first pass, so
 // the difference loses nothing), which saves the exchange of a separate norm pass.  Every block
 // reduces the partials of all blocks in the same fixed order, so results do not depend on scheduling.
+// Where h2 is more than half of w' all the same (|alpha| above ~1e7 beta: a large constant in H), one pass in FP64 is
+// not enough, as the orthogonality lost would grow by |h2| / beta at every step: (B) and (C) are then done once more on
+// w' - sum h2_k v_k, with slots of their own.  Without that a spectrum of width 1e-8 around 1 gave Lanczos vectors without
+// any orthogonality after five steps.
 //
 // What bounds it is FP64 issue (a warp-wide FP64 instruction holds a sub-partition ~64 cycles) and, for short vectors,
 // the chain of latencies.  Hence:
@@ -154,7 +160,6 @@ constexpr int OB = 256;   // threads per block of the fused kernel
 constexpr long kPollLimit = 1L << 20;
 constexpr int kOrthAlign = 128;              // elements of a block: a multiple of this
 constexpr int kOrthSmem = 220 * 1024;        // dynamic shared memory of a block at most
-constexpr int kPartRowsB1 = 8;               // second buffer of the second-pass partials: rows of partA from here on
 constexpr unsigned long long kEmpty = 0x7ff4dead7ff4deadull;   // a signalling NaN: arithmetic gives quiet ones
 
 // Segmented mode: the vector holds independent problems side by side (a direct sum of superblocks);
@@ -177,7 +182,8 @@ struct OrthArgs {
     double tol;
     double2* partA;    // first-pass partials, rows k of gridDim.x blocks
     double2* partB;    // second-pass partials of this step (empty)
-    double2* partNext; // those of the next step (used by the step before): cleared here
+    double2* partC;    // third-pass partials of this step (empty)
+    double2 *nextB, *nextC;   // both of the next step (used by the step before): cleared here
     double* tri;
     int* flags;
     int* status;
@@ -273,8 +279,90 @@ __device__ __forceinline__ double2 warp_dot(const double2* v, const double2* x, 
     return make_double2(s.x + t.x, s.y - t.y);
 }
 
+// ||x||^2 over one warp's elements
+__device__ __forceinline__ double2 warp_norm2(const double2* x, int E) {
+    double s = 0.0, t = 0.0;
+    for (int i = threadIdx.x & 31; i < E; i += 32) {
+        const double2 v = x[i];
+        s = fma(v.x, v.x, s);
+        t = fma(v.y, v.y, t);
+    }
+    return make_double2(s + t, 0.0);
+}
+
+// The sum of d over the warp into a slot
+__device__ __forceinline__ void store_part(double2* slot, double2 d) {
+    const int lane = threadIdx.x & 31;
+    const bool up = lane & 16;
+    double v = (up ? d.y : d.x) + __shfl_xor_sync(0xffffffffu, up ? d.x : d.y, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 15) == 0) st_slot(reinterpret_cast<double*>(slot) + (lane >> 4), v);
+}
+
+// beta, alpha and the stop test of a step from the dots h and the norm h[nv], by one warp; sc = {beta, 1 / beta}, 0 instead
+// of 1 / beta to stop and -1 (first: only then) when the pass took more than half of ||w'||^2.
+__device__ __forceinline__ void orth_scalars(const OrthArgs& a, double* tri, int* flags, const double2* h, double* alpha1, double* sc,
+                                             bool write, bool first) {
+    const int lane = threadIdx.x & 31, nv = a.nv;
+    double q = lane < nv ? fma(h[lane].x, h[lane].x, h[lane].y * h[lane].y) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (lane != 0) return;
+    const double bt = sqrt(fmax(h[nv].x - q, 0.0));
+    const double alpha = *alpha1 + h[a.j].x;
+    const bool st = (a.j == a.nk - 1) || (bt <= a.tol * fmax(1.0, fabs(alpha)));
+    // q > ||w'||^2 / 2, by the words that hold the exponents and 20 bits (both are positive)
+    const bool again = first && !st && __double2hiint(q) > __double2hiint(h[nv].x) - (1 << 20);
+    sc[0] = bt;
+    sc[1] = st ? 0.0 : again ? -1.0 : 1.0 / bt;
+    if (again) {
+        *alpha1 = alpha;
+    } else if (write) {
+        tri[T_ALPHA + a.j] = alpha;
+        tri[T_BETA + a.j] = bt;
+        if (st) {
+            tri[T_RESID] = bt;
+            flags[0] = a.j + 1;   // read by later kernels only (every block is past its check)
+        }
+    }
+}
+
+// The third pass of a step, rare, so it reads V from global memory only: w' - sum h2_k v_k takes the place of w', then (B) and
+// (C) with the slots of partC.
+__device__ __noinline__ void third_pass(const OrthArgs& a, double* tri, int* flags, const cplx* gV, double2* w, cplx* vnext, double2* h,
+                                        double* alpha1, double* sc, int E, int b0, int b1) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nv = a.nv, G = (int)gridDim.x;
+    auto update = [&](int i) {
+        double2 x = w[i];
+        for (int k = 0; k < nv; ++k) {
+            const double2 v = gV[(int64_t)k * a.n + i];
+            x.x = fma(-h[k].x, v.x, fma(h[k].y, v.y, x.x));
+            x.y = fma(-h[k].x, v.y, fma(-h[k].y, v.x, x.y));
+        }
+        return x;
+    };
+    for (int i = tid; i < E; i += OB) w[i] = update(i);
+    __syncthreads();
+    for (int k = warp; k <= nv; k += OB / 32)
+        store_part(a.partC + (int64_t)k * G + blockIdx.x, k == nv ? warp_norm2(w, E) : warp_dot(gV + (int64_t)k * a.n, w, E));
+    for (int k = warp; k <= nv; k += OB / 32) {
+        const double v = poll_sum(a.partC + (int64_t)k * G, b0, b1, a.status);
+        if (lane == 0) h[k].x = v;
+        if (lane == 16) h[k].y = v;
+    }
+    __syncthreads();
+    if (warp == OB / 32 - 1) orth_scalars(a, tri, flags, h, alpha1, sc, (int)blockIdx.x == b0, false);
+    __syncthreads();
+    if (sc[1] == 0.0) return;
+    for (int i = tid; i < E; i += OB) {
+        const double2 x = update(i);
+        vnext[i] = make_double2(x.x * sc[1], x.y * sc[1]);
+    }
+}
+
 template <bool SEG, bool STAGED>
-__global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(OrthArgs a) {
+__global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(const __grid_constant__ OrthArgs a) {
     pdl_enter();
     // one problem: the whole grid stops together.  Segments: nobody waits for a stopped segment's blocks.
     int sg = 0, b0 = 0, b1 = (int)gridDim.x;
@@ -385,25 +473,8 @@ __global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(OrthArgs a) {
     __syncthreads();
     // second-pass dots with every v_k and ||w'||^2 (row nv), FP64: a warp per row
     for (int k = warp; k <= nv; k += OB / 32) {
-        double2 d = make_double2(0.0, 0.0);
-        if (k == nv) {
-            double s = 0.0, t = 0.0;
-            for (int i = lane; i < E; i += 32) {
-                const double2 x = w[i];
-                s = fma(x.x, x.x, s);
-                t = fma(x.y, x.y, t);
-            }
-            d.x = s + t;
-        } else if (STAGED && k >= s0) {
-            d = warp_dot(staged(k), osm, E);
-        } else {
-            d = warp_dot(gV + (int64_t)k * a.n, w, E);
-        }
-        const bool up = lane & 16;
-        double v = (up ? d.y : d.x) + __shfl_xor_sync(0xffffffffu, up ? d.x : d.y, 16);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((lane & 15) == 0) st_slot(reinterpret_cast<double*>(a.partB + (int64_t)k * G + blockIdx.x) + (lane >> 4), v);
+        const double2 d = k == nv ? warp_norm2(w, E) : STAGED && k >= s0 ? warp_dot(staged(k), osm, E) : warp_dot(gV + (int64_t)k * a.n, w, E);
+        store_part(a.partB + (int64_t)k * G + blockIdx.x, d);
     }
     for (int k = warp; k <= nv; k += OB / 32) {
         const double v = poll_sum(a.partB + (int64_t)k * G, b0, b1, a.status);
@@ -411,32 +482,19 @@ __global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(OrthArgs a) {
         if (lane == 16) h[k].y = v;
     }
     // every block of the problem has stored its second-pass partials, so it has read the first-pass ones, and the step
-    // before has ended: its own slots of both are cleared for the next step
+    // before has ended: its own slots of these are cleared for the next step
     __syncthreads();
-    if (tid < 2 * na) st_slot(reinterpret_cast<double*>(a.partA + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), __longlong_as_double((long long)kEmpty));
-    if (tid < 2 * (nv + 1)) st_slot(reinterpret_cast<double*>(a.partNext + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), __longlong_as_double((long long)kEmpty));
-    // (C) beta, stop test and 1 / beta by the last warp (h2 in parallel, one FP64 square root), beside the others'
-    // update x = w' - sum h2_k v_k
-    if (warp == OB / 32 - 1) {
-        double q = lane < nv ? fma(h[lane].x, h[lane].x, h[lane].y * h[lane].y) : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-        if (lane == 0) {
-            const double bt = sqrt(fmax(h[nv].x - q, 0.0));
-            const double alpha = alpha1 + h[a.j].x;
-            const bool st = (a.j == a.nk - 1) || (bt <= a.tol * fmax(1.0, fabs(alpha)));
-            sc[0] = bt;
-            sc[1] = st ? 0.0 : 1.0 / bt;
-            if ((int)blockIdx.x == b0) {
-                tri[T_ALPHA + a.j] = alpha;
-                tri[T_BETA + a.j] = bt;
-                if (st) {
-                    tri[T_RESID] = bt;
-                    flags[0] = a.j + 1;   // read by later kernels only (every block is past its check)
-                }
-            }
+    {
+        const double e = __longlong_as_double((long long)kEmpty);
+        if (tid < 2 * na) st_slot(reinterpret_cast<double*>(a.partA + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), e);
+        if (tid < 2 * (nv + 1)) {
+            st_slot(reinterpret_cast<double*>(a.nextB + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), e);
+            st_slot(reinterpret_cast<double*>(a.nextC + (int64_t)(tid >> 1) * G + blockIdx.x) + (tid & 1), e);
         }
     }
+    // (C) beta, stop test and 1 / beta by the last warp (h2 in parallel, one FP64 square root), beside the others'
+    // update x = w' - sum h2_k v_k
+    if (warp == OB / 32 - 1) orth_scalars(a, tri, flags, h, &alpha1, sc, (int)blockIdx.x == b0, true);
     const bool last_step = a.j == a.nk - 1;   // no next vector
     cplx* vnext = const_cast<cplx*>(a.V) + (int64_t)(a.j + 1) * a.n + lo;
     bool have_sc = false;
@@ -470,9 +528,12 @@ __global__ void __launch_bounds__(OB, 1) k_lanczos_orth_t(OrthArgs a) {
                 }
         }
         if (!have_sc) { __syncthreads(); have_sc = true; }   // sc
-        if (sc[1] == 0.0) return;
+        if (!(sc[1] > 0.0)) break;   // stopped, or another pass
         if (i < E) vnext[i] = make_double2(x.x * sc[1], x.y * sc[1]);
     }
+    if (last_step) return;
+    if (!have_sc) __syncthreads();   // a block without elements
+    if (sc[1] < 0.0) third_pass(a, tri, flags, gV, w, vnext, h, &alpha1, sc, E, b0, b1);
 }
 
 // Taylor terms for a substep with ||T h|| <= xs <= 2: the smallest K (per bucket of xs) whose remainder
@@ -932,8 +993,8 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
     k.nk = nk;
     int rc = dev_alloc(c, (void**)&k.V, (size_t)(nk + 1) * n * sizeof(cplx), "Krylov vectors");
     if (!rc) rc = dev_alloc(c, (void**)&k.w, (size_t)n * sizeof(cplx), "Krylov residual");
-    if (!rc) rc = dev_alloc(c, (void**)&k.partA, 64 * kRedBlocks * sizeof(double2), "Krylov partials");
-    if (!rc) rc = dev_alloc(c, (void**)&k.partB, 64 * kRedBlocks * sizeof(double2), "Krylov partials");
+    if (!rc) rc = dev_alloc(c, (void**)&k.partA, kPartBytesA, "Krylov partials");
+    if (!rc) rc = dev_alloc(c, (void**)&k.partB, kPartBytesB, "Krylov partials");
     if (!rc) rc = dev_alloc(c, (void**)&k.tri, 128 * sizeof(double), "Krylov tridiagonal");
     if (!rc) rc = dev_alloc(c, (void**)&k.flags, 4 * sizeof(int), "Krylov flags");
     // coefficients [x][k] of 16 targets, then the columns of the step exponential (32 x 32)
@@ -954,8 +1015,8 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
     if (rc) {
         dev_free(c, k.V, (size_t)(nk + 1) * n * sizeof(cplx));
         dev_free(c, k.w, (size_t)n * sizeof(cplx));
-        dev_free(c, k.partA, 64 * kRedBlocks * sizeof(double2));
-        dev_free(c, k.partB, 64 * kRedBlocks * sizeof(double2));
+        dev_free(c, k.partA, kPartBytesA);
+        dev_free(c, k.partB, kPartBytesB);
         dev_free(c, k.tri, 128 * sizeof(double));
         dev_free(c, k.flags, 4 * sizeof(int));
         dev_free(c, k.coef, kCoefWords * sizeof(cplx));
@@ -979,7 +1040,9 @@ cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* p
 
 // Partial-sum slots of a Lanczos run on `grid` blocks with nk steps; norm partials of the start vector are in row 2 of partA.
 static OrthSlots orth_slots(const KrylovWork* k, int grid, int nk) {
-    return OrthSlots{k->partA, k->partB, k->partA + kPartRowsB1 * (int64_t)kRedBlocks, nk + 1, grid};
+    double2* const b = k->partB;
+    const int64_t buf = kPartRowsPass * (int64_t)kRedBlocks;
+    return OrthSlots{k->partA, {b, b + buf}, {b + 2 * buf, b + 3 * buf}, nk + 1, grid};
 }
 static double2* norm_slots(const KrylovWork* k) { return k->partA + 2 * (int64_t)kRedBlocks; }
 
@@ -987,8 +1050,10 @@ static double2* norm_slots(const KrylovWork* k) { return k->partA + 2 * (int64_t
 static cudaError_t launch_orth(tdmrg_ctx* c, const KrylovWork* k, OrthArgs a, int grid, int emax) {
     const OrthSlots sl = orth_slots(k, grid, a.nk);
     a.partA = sl.partA;
-    a.partB = (a.j & 1) ? sl.partB1 : sl.partB0;
-    a.partNext = (a.j & 1) ? sl.partB0 : sl.partB1;
+    a.partB = sl.partB[a.j & 1];
+    a.partC = sl.partC[a.j & 1];
+    a.nextB = sl.partB[(a.j + 1) & 1];
+    a.nextC = sl.partC[(a.j + 1) & 1];
     a.emax = emax;
     // shared memory: w and as many of the newest vectors as fit; at least v_{j-1} and v_j, else nothing is staged
     const size_t row = (size_t)std::max(emax, 1) * sizeof(cplx), cap = (size_t)kOrthSmem / k->orth_per_sm;
