@@ -142,12 +142,15 @@ namespace tdmrg {
 
 int get_ham_plan(tdmrg_ctx* c, int a, int b, Plan** out) { return get_plan(c, 0, -1, -1, a, b, a, b, out); }
 
+int uploads_done(tdmrg_ctx* c, const char* what) { return cuda_check(c, cudaStreamSynchronize(cudaStreamLegacy), what); }
+
 int check_device_status(tdmrg_ctx* c) {
     int st = 0;
     int rc = cuda_check(c, cudaMemcpy(&st, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost), "device status");
     if (rc) return rc;
     if (st) {
         cudaMemset(c->dstatus, 0, sizeof(int));
+        uploads_done(c, "device status");
         return fail(c, TDMRG_ETIMEOUT, "a bounded device wait ran out (tensor-core or seed mbarrier, Lanczos "
                                        "exchange or the wait probe); results are invalid");
     }
@@ -191,6 +194,7 @@ int tdmrg_create(tdmrg_ctx** out, const tdmrg_opts* o) {
     if (!rc) rc = dev_alloc(c, (void**)&c->dscale, 64 * sizeof(double), "scale workspace");
     if (!rc) rc = dev_alloc(c, (void**)&c->dstatus, 32 * sizeof(int), "status word");
     if (!rc) rc = cuda_check(c, cudaMemset(c->dstatus, 0, 32 * sizeof(int)), "status word");
+    if (!rc) rc = uploads_done(c, "status word");
     if (rc) {
         g_err = c->err;
         tdmrg_destroy(c);

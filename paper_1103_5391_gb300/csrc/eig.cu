@@ -1155,6 +1155,7 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
         memcpy(ho.data(), items.data(), items.size() * sizeof(int4));
         memcpy(ho.data() + items.size() * sizeof(int4), first.data(), first.size() * sizeof(int));
         rc = cuda_check(c, cudaMemcpy(G.oa, ho.data(), bytes, cudaMemcpyHostToDevice), "eig work items");
+        if (!rc) rc = uploads_done(c, "eig work items");
         if (rc) return rc;
     }
     if (G.nbig) {   // replay: 8 rows of V and as many rounds of the record as fit in 48 KB of shared memory

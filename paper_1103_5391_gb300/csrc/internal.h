@@ -24,10 +24,10 @@ typedef double2 cplx;   // {re, im}, same layout as tdmrg_c64
 // every kernel of the library starts with pdl_enter(), which waits until the previous grid of the stream
 // has completed and its memory is visible: the launch of a kernel overlaps the end of the previous one,
 // while every global memory access still follows the previous kernel's completion, except the reads of a plan's tables in
-// the slicer and the grouped FP64 GEMM: no kernel writes those, and an upload is no kernel, so a launch behind one waits for
-// it as a whole.  Their two or three loads in a row then run beside the end of the previous kernel (H psi at L=8 8.7 -> 8.2
-// us, at L=32 m=400 with four slices 44.4 -> 44.0 us).  The same for the setup and first tile of the tensor kernel gave
-// nothing, for the segments of the slicer it spilled, for the correction GEMM it cost the launches that are skipped.  No kernel signals
+// the slicer and the grouped FP64 GEMM: no kernel writes those, and they are complete before the launch is made
+// (uploads_done; run_transient copies its tables on the launch's own stream, and a launch behind a copy waits for it as a
+// whole).  Their two or three loads in a row then run beside the end of the previous kernel (H psi at L=8 8.7 -> 8.2 us, at
+// L=32 m=400 with four slices 44.4 -> 44.0 us).  The setup and first tile of the tensor kernel gain nothing from it.  No kernel signals
 // its dependents early (measured: blocks parked in the wait beside a running kernel slow it down).
 // Without the launch attribute the wait returns at once.
 #ifdef __CUDACC__
@@ -427,6 +427,10 @@ int fail(tdmrg_ctx* c, int code, const std::string& msg);
 int cuda_check(tdmrg_ctx* c, cudaError_t e, const char* what);
 int dev_alloc(tdmrg_ctx* c, void** p, size_t bytes, const char* what);
 void dev_free(tdmrg_ctx* c, void* p, size_t bytes);
+// Ends a build of tables by cudaMemcpy and cudaMemset: waits until they are in device memory.  Both run on the legacy stream and
+// may return before that (a pageable copy once its source is staged), and nothing orders them before a kernel on a
+// non-blocking stream of the caller's.
+int uploads_done(tdmrg_ctx* c, const char* what);
 
 // plan.cu
 int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qin0, int qin1, int qout0, int qout1,

@@ -1246,6 +1246,8 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
         rc = cuda_check(c, e, "ozaki shared memory");
         if (rc) return rc;
     }
+    rc = uploads_done(c, "ozaki tables");
+    if (rc) return rc;
     // static operands: stage-1 B (operators, scales folded) and stage-2 A (operators, scales folded)
     GemmArgs g{};
     g.bufs[BUF_OPS] = c->pool;

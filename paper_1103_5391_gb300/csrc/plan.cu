@@ -41,7 +41,7 @@ int upload(tdmrg_ctx* c, TaskList& tl) {
     tl.bytes = tl.tasks.size() * sizeof(Task) + tl.segs.size() * sizeof(Seg) + tl.tiles.size() * sizeof(Tile) +
                tl.ctiles.size() * sizeof(CorrTile) +
                (size_t)tl.npartial * sizeof(cplx) + (size_t)tl.nsplit * sizeof(int);
-    return TDMRG_OK;
+    return uploads_done(c, "task list upload");
 }
 
 void release(tdmrg_ctx* c, TaskList& tl) {
