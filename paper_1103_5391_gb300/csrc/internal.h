@@ -128,6 +128,7 @@ struct TaskList {
     std::vector<Seg> segs;
     std::vector<Tile> tiles;
     std::vector<CorrTile> ctiles;   // instead of tiles: a list of the correction kernel
+    std::vector<int> group;         // sector products: the connected left sectors of each task (make_tiles)
     Task* d_tasks = nullptr;
     Seg* d_segs = nullptr;
     Tile* d_tiles = nullptr;

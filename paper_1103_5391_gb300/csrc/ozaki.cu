@@ -1017,6 +1017,7 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
         TaskList& thin = p->thin[stg];
         release(c, thin);
         thin.tasks.clear(); thin.segs.clear();
+        std::vector<int> gthin;   // groups of its tasks
         OzStage& st = oz.st[stg];
         std::map<int64_t, int> pair_row;   // stage 1: Psi block offset -> A panel row
         int rowsA = 0, rowsB = 0, kmax = 0;
@@ -1052,6 +1053,7 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
                 for (int s = tk.seg_begin; s < tk.seg_end; ++s) thin.segs.push_back(tl.segs[s]);
                 nt.seg_end = (int)thin.segs.size();
                 thin.tasks.push_back(nt);
+                gthin.push_back(tl.group[t]);
                 continue;
             }
             OzTask ot{};
@@ -1118,33 +1120,33 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
         }
         std::stable_sort(st.tiles.begin(), st.tiles.end(), [](const OzTile& a, const OzTile& b) { return a.cost > b.cost; });
         std::stable_sort(st.tiles128.begin(), st.tiles128.end(), [](const OzTile& a, const OzTile& b) { return a.cost > b.cost; });
-        // thin outputs in order of (segments, K, real operands), 32 per item; an item costs its longest chain and the latency
-        // of its tables and operands
+        // thin outputs in order of (segments, K, real operands), up to 32 per item; an item costs its longest chain and the
+        // latency of its tables and operands.  How many lanes share an output follows from its own task, and an item holds
+        // outputs of one such split, so that an output's order of summation does not depend on what is packed beside it.
         if (!st.ttasks.empty()) {
-            struct Key { int nseg, k, mode, task; };
+            struct Key { int nseg, k, mode, task, lps, lpk, cost; };
             std::vector<Key> keys;
             for (size_t t = 0; t < st.ttasks.size(); ++t) {
                 const Task& tk = st.ttasks[t];
-                Key kk{tk.seg_end - tk.seg_begin, 0, 0, (int)t};
+                Key kk{tk.seg_end - tk.seg_begin, 0, 0, (int)t, 0, 0, 0};
                 for (int s = tk.seg_begin; s < tk.seg_end; ++s) { kk.k += st.tsegs[s].K; kk.mode = kk.mode * 4 + (st.tsegs[s].rflags & 3); }
+                auto cost = [&] {   // k-steps in a row, segments in a row and the first loads
+                    return kk.k / (1 << (kk.lps + kk.lpk)) + 4 * ((kk.nseg + (1 << kk.lps) - 1) >> kk.lps) + 4;
+                };
+                while (kk.lps + kk.lpk < kThinLog2Parts && cost() > kThinChain)
+                    if ((1 << kk.lps) < kk.nseg) ++kk.lps;
+                    else ++kk.lpk;
+                kk.cost = cost();
                 keys.push_back(kk);
             }
             std::stable_sort(keys.begin(), keys.end(), [](const Key& x, const Key& y) {
-                return std::make_tuple(-x.nseg, -x.k, x.mode) < std::make_tuple(-y.nseg, -y.k, y.mode);
+                return std::make_tuple(-x.nseg, x.lps, x.lpk, -x.k, x.mode) < std::make_tuple(-y.nseg, y.lps, y.lpk, -y.k, y.mode);
             });
             for (const Key& kk : keys)
                 for (int o = 0; o < st.ttasks[kk.task].M * st.ttasks[kk.task].N; ++o) {
-                    if (st.titems.empty() || st.titems.back().cnt == 32 >> (st.titems.back().lps + st.titems.back().lpk)) {
-                        ThinItem it{(int)st.touts.size(), 0, 0, 0, 0};
-                        auto cost = [&] {   // k-steps in a row, segments in a row and the first loads
-                            return kk.k / (1 << (it.lps + it.lpk)) + 4 * ((kk.nseg + (1 << it.lps) - 1) >> it.lps) + 4;
-                        };
-                        while (it.lps + it.lpk < kThinLog2Parts && cost() > kThinChain)
-                            if ((1 << it.lps) < kk.nseg) ++it.lps;
-                            else ++it.lpk;
-                        it.cost = cost();
-                        st.titems.push_back(it);
-                    }
+                    const bool fits = !st.titems.empty() && st.titems.back().lps == kk.lps && st.titems.back().lpk == kk.lpk &&
+                                      st.titems.back().cnt < 32 >> (kk.lps + kk.lpk);
+                    if (!fits) st.titems.push_back(ThinItem{(int)st.touts.size(), 0, kk.cost, (int16_t)kk.lps, (int16_t)kk.lpk});
                     st.touts.push_back(make_int2(kk.task, o));
                     ++st.titems.back().cnt;
                 }
@@ -1234,7 +1236,7 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
             mk(st.sliceB, st.bjobs, st.d_bjobs, st.d_bvjob, st.d_bsegs, st.panelB, st.expB, st.rowsB);
         }
         if (!thin.tasks.empty()) {
-            make_tiles(thin);
+            make_tiles(thin, &gthin);
             rc = upload(c, thin);
             if (rc) return rc;
         }

@@ -411,6 +411,8 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         s2.tasks.push_back(tk);
         g2.push_back(find_root(pout[k].qi));
     }
+    s1.group = g1;
+    s2.group = g2;
     make_tiles(s1, &g1);
     make_tiles(s2, &g2);
     p->scratch = scr;
