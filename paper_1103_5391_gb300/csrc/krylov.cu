@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, in
 // 14200 / 20400 -> 6700 / 14500, its exchange 10300 / 10700 -> 3900 / 6000, pass C 8400 / 13700 -> 4500 / 11500; the launch
 // 23.4 / 26.8 -> 13.6 / 19.9 us on average over a run.  What remains at D = 46,868 is FP64 issue in B and C.
 constexpr int OB = 256;   // threads per block of the fused kernel
-constexpr long kPollLimit = 1L << 20;
+constexpr long kPollLimit = 1L << 24;        // polls of another block's value (a block may wait for an SM of its own)
+constexpr long kBulkLimit = 1L << 20;        // polls of the block's own copies
 constexpr int kOrthAlign = 128;              // elements of a block: a multiple of this
 constexpr int kOrthSmem = 220 * 1024;        // dynamic shared memory of a block at most
 constexpr unsigned long long kEmpty = 0x7ff4dead7ff4deadull;   // a signalling NaN: arithmetic gives quiet ones
@@ -253,7 +254,7 @@ __device__ __forceinline__ float f32_trunc(double x) {
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ bool wait_bulk(uint32_t bar) {
-    for (long i = 0; i < kPollLimit; ++i) {
+    for (long i = 0; i < kBulkLimit; ++i) {
         uint32_t done;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done) : "r"(bar) : "memory");
