@@ -92,14 +92,20 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
     int m = 0, n = 0;
     if (active) {
         const int o = tile.o0 + lo;
-        if (tile.N == 0) {   // row m of the lower triangle starts at m (m + 1) / 2
-            m = (int)((sqrtf(8.f * (float)o + 1.f) - 1.f) * 0.5f);
-            while ((m + 1) * (m + 2) / 2 <= o) ++m;
-            while (m * (m + 1) / 2 > o) --m;
-            n = o - m * (m + 1) / 2;
-        } else {
+        if (tile.N != 0) {
             m = o / tile.N;
             n = o - m * tile.N;
+            m += tile.m0;
+        } else if (tile.m0 < 4096) {   // row m of the lower triangle starts at m (m + 1) / 2
+            const int t = tile.m0 * (tile.m0 + 1) / 2 + o;
+            m = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+            while ((m + 1) * (m + 2) / 2 <= t) ++m;
+            while (m * (m + 1) / 2 > t) --m;
+            n = t - m * (m + 1) / 2;
+        } else {                       // at most one row further
+            m = tile.m0;
+            n = o;
+            while (n > m) n -= ++m;
         }
     }
     const int kspan = tile.k1 - tile.k0;
@@ -142,7 +148,7 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
     const bool out = active && part == 0;
     if (tile.split >= 0) {
         // split-K over CTAs: publish this part, the last part to arrive sums all parts in index order
-        cplx* base = args.partials + tile.split_base;
+        cplx* base = args.partials + 32 * (int64_t)tile.split_base;
         if (out) base[(int64_t)tile.part * pad + lo] = make_double2(re, im);
         __threadfence();
         __syncthreads();

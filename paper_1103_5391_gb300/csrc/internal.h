@@ -102,13 +102,13 @@ struct Task {
     int32_t pad2;
 };
 
-// One CTA's work: outputs [o0, o0 + cnt) of task `task` in flattened order (row-major, or the lower triangle row
-// by row when the task is Hermitian), over k in [k0, k1) counted from the start of segment seg_lo (segments
-// [seg_lo, seg_hi) cover it), the K range divided among `ks` groups of the CTA's warps.  A tile that is one
-// of several K parts has split >= 0: part `part` of `nparts`, partial sums at partials[split_base + part *
-// (cnt rounded up to 32)], completion ticket counters[split].
+// One CTA's work: `cnt` outputs of task `task` from row m0, column o0 on in flattened order (row-major, or the lower
+// triangle row by row when the task is Hermitian; a row and a column, as the flattened index of a block may need more than
+// 32 bits), over k in [k0, k1) counted from the start of segment seg_lo (segments [seg_lo, seg_hi) cover it), the K range
+// divided among `ks` groups of the CTA's warps.  A tile that is one of several K parts has split >= 0: part `part` of
+// `nparts`, partial sums at partials[32 split_base + part * (cnt rounded up to 32)], completion ticket counters[split].
 struct Tile {
-    int32_t task, o0, cnt, ks;
+    int32_t task, m0, o0, cnt, ks;
     int32_t seg_lo, seg_hi, k0, k1;
     int32_t split, part, nparts, split_base;
     int32_t cost;             // complex MACs, for ordering

@@ -180,6 +180,7 @@ void make_tiles(TaskList& tl, const std::vector<int>* group) {
         const int np = (int)parts.size();
         const int64_t nt = (outs[t] + area - 1) / area;
         const int64_t step = std::min<int64_t>(area, 32 * ((outs[t] + 32 * nt - 1) / (32 * nt)));
+        int64_t row = 0, col = 0;   // of output o0
         for (int64_t o0 = 0; o0 < outs[t]; o0 += step) {
             const int cnt = (int)std::min<int64_t>(step, outs[t] - o0), pad = (cnt + 31) & ~31;
             const int split = np > 1 ? tl.nsplit++ : -1;
@@ -187,13 +188,20 @@ void make_tiles(TaskList& tl, const std::vector<int>* group) {
             if (np > 1) tl.npartial += (int64_t)np * pad;
             for (int p = 0; p < np; ++p) {
                 Tile tile{};
-                tile.task = (int32_t)t; tile.o0 = (int32_t)o0; tile.cnt = cnt; tile.ks = cks;
+                tile.task = (int32_t)t; tile.m0 = (int32_t)row; tile.o0 = (int32_t)col; tile.cnt = cnt; tile.ks = cks;
                 tile.N = k.herm ? 0 : k.N;
                 tile.seg_lo = parts[p].seg_lo; tile.seg_hi = parts[p].seg_hi;
                 tile.k0 = (int32_t)parts[p].k0; tile.k1 = (int32_t)parts[p].k1;
-                tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = (int32_t)base;
+                tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = (int32_t)(base / 32);
                 tile.cost = (int32_t)std::min<int64_t>((int64_t)cnt * std::max<int64_t>(parts[p].k1 - parts[p].k0, 1), 0x7fffffff);
                 tl.tiles.push_back(tile);
+            }
+            col += step;
+            if (k.herm) {
+                while (col > row) col -= ++row;
+            } else {
+                row += col / k.N;
+                col %= k.N;
             }
         }
     }
