@@ -84,8 +84,7 @@ void drop_krylov(tdmrg_ctx* c) {
         size_t n = (size_t)k.n;
         dev_free(c, k.V, (k.nk + 1) * n * sizeof(cplx));
         dev_free(c, k.w, n * sizeof(cplx));
-        dev_free(c, k.partA, kPartBytesA);
-        dev_free(c, k.partB, kPartBytesB);
+        dev_free(c, k.part, part_bytes(k.nk));
         dev_free(c, k.tri, 128 * sizeof(double));
         dev_free(c, k.flags, 4 * sizeof(int));
         dev_free(c, k.coef, (16 + 32) * 32 * sizeof(cplx));
@@ -142,7 +141,13 @@ namespace tdmrg {
 
 int get_ham_plan(tdmrg_ctx* c, int a, int b, Plan** out) { return get_plan(c, 0, -1, -1, a, b, a, b, out); }
 
-int uploads_done(tdmrg_ctx* c, const char* what) { return cuda_check(c, cudaStreamSynchronize(cudaStreamLegacy), what); }
+int uploads_done(tdmrg_ctx* c, const char* what) {
+    unsigned flags = 0;
+    if (c->stream == nullptr || c->stream == cudaStreamLegacy) return TDMRG_OK;
+    int rc = cuda_check(c, cudaStreamGetFlags(c->stream, &flags), what);
+    if (!rc && (flags & cudaStreamNonBlocking)) rc = cuda_check(c, cudaStreamSynchronize(cudaStreamLegacy), what);
+    return rc;
+}
 
 int check_device_status(tdmrg_ctx* c) {
     int st = 0;
@@ -150,7 +155,7 @@ int check_device_status(tdmrg_ctx* c) {
     if (rc) return rc;
     if (st) {
         cudaMemset(c->dstatus, 0, sizeof(int));
-        uploads_done(c, "device status");
+        cudaStreamSynchronize(cudaStreamLegacy);
         return fail(c, TDMRG_ETIMEOUT, "a bounded device wait ran out (tensor-core or seed mbarrier, Lanczos "
                                        "exchange or the wait probe); results are invalid");
     }
@@ -194,7 +199,7 @@ int tdmrg_create(tdmrg_ctx** out, const tdmrg_opts* o) {
     if (!rc) rc = dev_alloc(c, (void**)&c->dscale, 64 * sizeof(double), "scale workspace");
     if (!rc) rc = dev_alloc(c, (void**)&c->dstatus, 32 * sizeof(int), "status word");
     if (!rc) rc = cuda_check(c, cudaMemset(c->dstatus, 0, 32 * sizeof(int)), "status word");
-    if (!rc) rc = uploads_done(c, "status word");
+    if (!rc) rc = cuda_check(c, cudaStreamSynchronize(cudaStreamLegacy), "status word");   // whatever stream comes to be used
     if (rc) {
         g_err = c->err;
         tdmrg_destroy(c);

@@ -183,8 +183,8 @@ int build_corr(tdmrg_ctx* c, int nL, const int32_t* opL, int nR, const int32_t* 
         rc = dev_alloc(c, (void**)&cp.copies, copies.size() * sizeof(CorrCopy), "correlation copies");
         if (!rc) rc = cuda_check(c, cudaMemcpy(cp.copies, copies.data(), copies.size() * sizeof(CorrCopy), cudaMemcpyHostToDevice),
                                  "correlation copies");
-        if (!rc) rc = uploads_done(c, "correlation copies");
     }
+    if (!rc) rc = uploads_done(c, "correlation upload");
     return rc;
 }
 

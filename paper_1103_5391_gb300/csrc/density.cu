@@ -218,6 +218,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
         make_tiles(*tl);
         first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
+        if (!rc) rc = uploads_done(c, "density plan upload");
         if (rc) { release(c, *tl); return rc; }
         it = c->rho_plans.emplace(key, std::move(tl)).first;
     }
@@ -251,6 +252,7 @@ int density_matrix(tdmrg_ctx* c, int side, int nt, const int32_t* Q, const cplx*
         make_tiles(*tl);
         first_tiles(*tl, nfirst);
         int rc = upload(c, *tl);
+        if (!rc) rc = uploads_done(c, "density plan upload");
         if (rc) { release(c, *tl); return rc; }
         it = c->rho_plans.emplace(key, std::move(tl)).first;
     }

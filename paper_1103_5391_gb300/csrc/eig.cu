@@ -1155,7 +1155,6 @@ int setup_group(tdmrg_ctx* c, const Side& L, const std::vector<int64_t>& goff, c
         memcpy(ho.data(), items.data(), items.size() * sizeof(int4));
         memcpy(ho.data() + items.size() * sizeof(int4), first.data(), first.size() * sizeof(int));
         rc = cuda_check(c, cudaMemcpy(G.oa, ho.data(), bytes, cudaMemcpyHostToDevice), "eig work items");
-        if (!rc) rc = uploads_done(c, "eig work items");
         if (rc) return rc;
     }
     if (G.nbig) {   // replay: 8 rows of V and as many rounds of the record as fit in 48 KB of shared memory
@@ -1320,6 +1319,7 @@ int eig_prepare(tdmrg_ctx* c, int side) {
             if (!rc) rc = cuda_check(c, cudaEventCreateWithFlags(&w.fork, cudaEventDisableTiming), "eig stream");
             if (!rc) rc = cuda_check(c, cudaEventCreateWithFlags(&w.join, cudaEventDisableTiming), "eig stream");
         }
+        if (!rc) rc = uploads_done(c, "eig tables");
         if (rc) return rc;
         w.ready = true;
     }

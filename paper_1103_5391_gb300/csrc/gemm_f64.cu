@@ -96,13 +96,12 @@ __global__ void __launch_bounds__(GT, 2) gemm_f64_kernel(GemmArgs args, const in
             m = o / tile.N;
             n = o - m * tile.N;
             m += tile.m0;
-        } else if (tile.m0 < 4096) {   // row m of the lower triangle starts at m (m + 1) / 2
-            const int t = tile.m0 * (tile.m0 + 1) / 2 + o;
-            m = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-            while ((m + 1) * (m + 2) / 2 <= t) ++m;
-            while (m * (m + 1) / 2 > t) --m;
-            n = t - m * (m + 1) / 2;
-        } else {                       // at most one row further
+        } else if (tile.m0 == 0) {   // row m of the lower triangle starts at m (m + 1) / 2
+            m = (int)((sqrtf(8.f * (float)o + 1.f) - 1.f) * 0.5f);
+            while ((m + 1) * (m + 2) / 2 <= o) ++m;
+            while (m * (m + 1) / 2 > o) --m;
+            n = o - m * (m + 1) / 2;
+        } else {
             m = tile.m0;
             n = o;
             while (n > m) n -= ++m;

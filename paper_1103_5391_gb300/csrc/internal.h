@@ -24,11 +24,11 @@ typedef double2 cplx;   // {re, im}, same layout as tdmrg_c64
 // every kernel of the library starts with pdl_enter(), which waits until the previous grid of the stream
 // has completed and its memory is visible: the launch of a kernel overlaps the end of the previous one,
 // while every global memory access still follows the previous kernel's completion, except the reads of a plan's tables in
-// the slicer and the grouped FP64 GEMM: no kernel writes those, and they are complete before the launch is made
-// (uploads_done; run_transient copies its tables on the launch's own stream, and a launch behind a copy waits for it as a
-// whole).  Their two or three loads in a row then run beside the end of the previous kernel (H psi at L=8 8.7 -> 8.2 us, at
-// L=32 m=400 with four slices 44.4 -> 44.0 us).  The setup and first tile of the tensor kernel gain nothing from it.  No kernel signals
-// its dependents early (measured: blocks parked in the wait beside a running kernel slow it down).
+// the slicer and the grouped FP64 GEMM: no kernel writes those, and an upload is either complete before the launch is made
+// or ahead of it in stream order (uploads_done, run_transient), where a launch behind a copy waits for it as a whole.
+// Their two or three loads in a row then run beside the end of the previous kernel (H psi at L=8 8.7 -> 8.2 us, at L=32
+// m=400 with four slices 44.4 -> 44.0 us).  The setup and first tile of the tensor kernel gain nothing from it.  No kernel
+// signals its dependents early (measured: blocks parked in the wait beside a running kernel slow it down).
 // Without the launch attribute the wait returns at once.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -102,15 +102,16 @@ struct Task {
     int32_t pad2;
 };
 
-// One CTA's work: `cnt` outputs of task `task` from row m0, column o0 on in flattened order (row-major, or the lower
-// triangle row by row when the task is Hermitian; a row and a column, as the flattened index of a block may need more than
-// 32 bits), over k in [k0, k1) counted from the start of segment seg_lo (segments [seg_lo, seg_hi) cover it), the K range
-// divided among `ks` groups of the CTA's warps.  A tile that is one of several K parts has split >= 0: part `part` of
-// `nparts`, partial sums at partials[32 split_base + part * (cnt rounded up to 32)], completion ticket counters[split].
+// One CTA's work: `cnt` outputs of task `task` from entry o0 of row m0 on in flattened order (row-major, or the lower
+// triangle row by row when the task is Hermitian; m0 = 0 unless the task has more than kFlatOuts outputs), over k in
+// [k0, k1) counted from the start of segment seg_lo (segments [seg_lo, seg_hi) cover it), the K range divided among `ks`
+// groups of the CTA's warps.  A tile that is one of several K parts has split >= 0: part `part` of `nparts`, partial sums
+// at partials[32 split_base + part * (cnt rounded up to 32)], completion ticket counters[split].
 struct Tile {
     int32_t task, m0, o0, cnt, ks;
     int32_t seg_lo, seg_hi, k0, k1;
-    int32_t split, part, nparts, split_base;
+    int32_t split, split_base;
+    uint16_t part, nparts;
     int32_t cost;             // complex MACs, for ordering
     int32_t N;                // columns of the task's output (0: lower triangle), so that its outputs need no second load
 };
@@ -128,7 +129,6 @@ struct TaskList {
     std::vector<Seg> segs;
     std::vector<Tile> tiles;
     std::vector<CorrTile> ctiles;   // instead of tiles: a list of the correction kernel
-    std::vector<int> group;         // sector products: the connected left sectors of each task (make_tiles)
     Task* d_tasks = nullptr;
     Seg* d_segs = nullptr;
     Tile* d_tiles = nullptr;
@@ -241,6 +241,7 @@ struct Plan {
     double flops = 0.0;
     OzPlan oz;
     TaskList thin[2];
+    std::vector<int> group[2];   // per stage: the connected left sectors of each task (make_tiles)
 };
 
 // The correlation grid <phi1| A_i B_j |phi2> (correlation.cu): the products Z_i and T_j on a common block list as one
@@ -286,8 +287,8 @@ struct KrylovWork {     // device workspace of tdmrg_evolve for one (Q, nk)
     int nk = 0;
     cplx* V = nullptr;          // (nk + 1) x n Lanczos vectors
     cplx* w = nullptr;          // n
-    double2* partA = nullptr;   // reduction partials: first pass (two rows) and the start vector's norm
-    double2* partB = nullptr;   // two buffers of second-pass and two of third-pass partials, kPartRowsPass rows each
+    double2* part = nullptr;    // reduction partials (part_bytes(nk)), rows of kRedBlocks: first pass (two rows), the start
+                                // vector's norm, two buffers of second-pass and two of third-pass partials of nk + 1 rows each
     double* tri = nullptr;      // alpha[32], beta[32], beta0, resid, err
     int* flags = nullptr;       // n_used
     cplx* coef = nullptr;       // [x][k] Krylov coefficients
@@ -428,9 +429,9 @@ int fail(tdmrg_ctx* c, int code, const std::string& msg);
 int cuda_check(tdmrg_ctx* c, cudaError_t e, const char* what);
 int dev_alloc(tdmrg_ctx* c, void** p, size_t bytes, const char* what);
 void dev_free(tdmrg_ctx* c, void* p, size_t bytes);
-// Ends a build of tables by cudaMemcpy and cudaMemset: waits until they are in device memory.  Both run on the legacy stream and
-// may return before that (a pageable copy once its source is staged), and nothing orders them before a kernel on a
-// non-blocking stream of the caller's.
+// Ends a build of tables by cudaMemcpy and cudaMemset.  Both run on the legacy stream and may return before the data are in
+// device memory (a pageable copy once its source is staged); a blocking stream follows the legacy stream by itself, before a
+// kernel on a non-blocking one the host waits, once per build.
 int uploads_done(tdmrg_ctx* c, const char* what);
 
 // plan.cu
@@ -447,6 +448,7 @@ int run_transient(tdmrg_ctx* c, TaskList* const* lists, int nlists, int64_t scra
 int run_plan(tdmrg_ctx* c, const Plan& p, const cplx* in, cplx* out, const int* skip_flag, int skip_step);
 
 // gemm_f64.cu: grouped complex FP64 GEMM (one output per lane), and the correction C = (I + A) B with A B in FP32
+constexpr int64_t kFlatOuts = 1 << 29;   // a task with no more outputs is indexed flat, in 32 bits
 constexpr int kTileOut = 256;    // outputs of a tile at most (threads of its CTA)
 constexpr int kTileSegs = 16;    // segments of a tile at most
 constexpr int kMaxParts = 8;     // CTAs that share one tile's K range at most (more only for its segments' sake)
@@ -476,8 +478,7 @@ int segments_info(tdmrg_ctx* c, int n_up, int n_dn, int nk, int nseg, int* nk_us
 cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* partials, int nblk,
                              cplx* out, int normalise, cudaStream_t s);
 constexpr int kRedBlocks = 304;   // 2 x 152 SMs: fixed, so reductions are deterministic
-constexpr int kPartRowsPass = 33; // partials of 32 Krylov vectors and the norm
-constexpr size_t kPartBytesA = 3 * kRedBlocks * sizeof(double2), kPartBytesB = 4 * (size_t)kPartRowsPass * kRedBlocks * sizeof(double2);
+constexpr size_t part_bytes(int nk) { return (3 + 4 * ((size_t)nk + 1)) * kRedBlocks * sizeof(double2); }   // KrylovWork::part
 
 // density.cu
 // With `grouped` (a side whose eigensolver runs two sector groups, eig_prepare done), the rho blocks of the

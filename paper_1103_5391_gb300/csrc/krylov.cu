@@ -994,16 +994,14 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
     k.nk = nk;
     int rc = dev_alloc(c, (void**)&k.V, (size_t)(nk + 1) * n * sizeof(cplx), "Krylov vectors");
     if (!rc) rc = dev_alloc(c, (void**)&k.w, (size_t)n * sizeof(cplx), "Krylov residual");
-    if (!rc) rc = dev_alloc(c, (void**)&k.partA, kPartBytesA, "Krylov partials");
-    if (!rc) rc = dev_alloc(c, (void**)&k.partB, kPartBytesB, "Krylov partials");
+    if (!rc) rc = dev_alloc(c, (void**)&k.part, part_bytes(nk), "Krylov partials");
     if (!rc) rc = dev_alloc(c, (void**)&k.tri, 128 * sizeof(double), "Krylov tridiagonal");
     if (!rc) rc = dev_alloc(c, (void**)&k.flags, 4 * sizeof(int), "Krylov flags");
     // coefficients [x][k] of 16 targets, then the columns of the step exponential (32 x 32)
     if (!rc) rc = dev_alloc(c, (void**)&k.coef, kCoefWords * sizeof(cplx), "Krylov coefficients");
     // the ticket of k_tridiag_exp_eq (word 2)
     if (!rc) rc = dev_alloc(c, (void**)&k.bar, kBarWords * sizeof(unsigned), "Krylov ticket");
-    if (!rc) rc = cuda_check(c, cudaMemset(k.bar, 0, kBarWords * sizeof(unsigned)), "Krylov ticket");
-    if (!rc) rc = uploads_done(c, "Krylov ticket");
+    if (!rc) rc = cuda_check(c, cudaMemsetAsync(k.bar, 0, kBarWords * sizeof(unsigned), c->stream), "Krylov ticket");
     if (!rc) {   // co-resident grid of the fused orthogonalisation: at most one block per SM, at most NB
         int per_sm = 0;
         rc = cuda_check(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lanczos_orth_t<true, false>, OB, 0), "occupancy");
@@ -1017,8 +1015,7 @@ int ensure_work(tdmrg_ctx* c, int a, int b, int nk, int64_t n, KrylovWork** out)
     if (rc) {
         dev_free(c, k.V, (size_t)(nk + 1) * n * sizeof(cplx));
         dev_free(c, k.w, (size_t)n * sizeof(cplx));
-        dev_free(c, k.partA, kPartBytesA);
-        dev_free(c, k.partB, kPartBytesB);
+        dev_free(c, k.part, part_bytes(nk));
         dev_free(c, k.tri, 128 * sizeof(double));
         dev_free(c, k.flags, 4 * sizeof(int));
         dev_free(c, k.coef, kCoefWords * sizeof(cplx));
@@ -1040,13 +1037,13 @@ cudaError_t launch_dot_final(const cplx* x, const cplx* y, int64_t n, double2* p
     return cudaGetLastError();
 }
 
-// Partial-sum slots of a Lanczos run on `grid` blocks with nk steps; norm partials of the start vector are in row 2 of partA.
+// Partial-sum slots of a Lanczos run on `grid` blocks with nk steps; norm partials of the start vector are in row 2.
 static OrthSlots orth_slots(const KrylovWork* k, int grid, int nk) {
-    double2* const b = k->partB;
-    const int64_t buf = kPartRowsPass * (int64_t)kRedBlocks;
-    return OrthSlots{k->partA, {b, b + buf}, {b + 2 * buf, b + 3 * buf}, nk + 1, grid};
+    const int64_t buf = (nk + 1) * (int64_t)kRedBlocks;
+    double2* const b = k->part + 3 * (int64_t)kRedBlocks;
+    return OrthSlots{k->part, {b, b + buf}, {b + 2 * buf, b + 3 * buf}, nk + 1, grid};
 }
-static double2* norm_slots(const KrylovWork* k) { return k->partA + 2 * (int64_t)kRedBlocks; }
+static double2* norm_slots(const KrylovWork* k) { return k->part + 2 * (int64_t)kRedBlocks; }
 
 // One orthogonalisation step on `grid` co-resident blocks of at most emax elements.
 static cudaError_t launch_orth(tdmrg_ctx* c, const KrylovWork* k, OrthArgs a, int grid, int emax) {

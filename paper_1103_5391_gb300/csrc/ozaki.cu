@@ -1053,7 +1053,7 @@ int build_oz(tdmrg_ctx* c, Plan* p, int S) {
                 for (int s = tk.seg_begin; s < tk.seg_end; ++s) thin.segs.push_back(tl.segs[s]);
                 nt.seg_end = (int)thin.segs.size();
                 thin.tasks.push_back(nt);
-                gthin.push_back(tl.group[t]);
+                gthin.push_back(p->group[stg][t]);
                 continue;
             }
             OzTask ot{};

@@ -10,13 +10,14 @@
 // Each stage-2 output block owns one task whose segments are all its left products, so every
 // output tile accumulates all of its terms in registers before a single store (no atomics).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "internal.h"
 
 namespace tdmrg {
 
-int upload(tdmrg_ctx* c, TaskList& tl) {
+int upload(tdmrg_ctx* c, TaskList& tl) {   // uploads_done follows, once for all lists of a build
     release(c, tl);
     struct { void** dst; const void* src; size_t bytes; } parts[4] = {
         {(void**)&tl.d_tasks, tl.tasks.data(), tl.tasks.size() * sizeof(Task)},
@@ -41,7 +42,7 @@ int upload(tdmrg_ctx* c, TaskList& tl) {
     tl.bytes = tl.tasks.size() * sizeof(Task) + tl.segs.size() * sizeof(Seg) + tl.tiles.size() * sizeof(Tile) +
                tl.ctiles.size() * sizeof(CorrTile) +
                (size_t)tl.npartial * sizeof(cplx) + (size_t)tl.nsplit * sizeof(int);
-    return uploads_done(c, "task list upload");
+    return TDMRG_OK;
 }
 
 void release(tdmrg_ctx* c, TaskList& tl) {
@@ -180,11 +181,16 @@ void make_tiles(TaskList& tl, const std::vector<int>* group) {
         const int np = (int)parts.size();
         const int64_t nt = (outs[t] + area - 1) / area;
         const int64_t step = std::min<int64_t>(area, 32 * ((outs[t] + 32 * nt - 1) / (32 * nt)));
-        int64_t row = 0, col = 0;   // of output o0
         for (int64_t o0 = 0; o0 < outs[t]; o0 += step) {
             const int cnt = (int)std::min<int64_t>(step, outs[t] - o0), pad = (cnt + 31) & ~31;
             const int split = np > 1 ? tl.nsplit++ : -1;
             const int64_t base = tl.npartial;
+            int64_t row = 0, col = o0;   // of output o0, where a flattened index does not do
+            if (outs[t] > kFlatOuts) {
+                row = k.herm ? (int64_t)((std::sqrt(8.0 * (double)o0 + 1.0) - 1.0) * 0.5) : o0 / k.N;
+                if (k.herm) row += (row + 1) * (row + 2) / 2 <= o0 ? 1 : row * (row + 1) / 2 > o0 ? -1 : 0;
+                col = k.herm ? o0 - row * (row + 1) / 2 : o0 - row * k.N;
+            }
             if (np > 1) tl.npartial += (int64_t)np * pad;
             for (int p = 0; p < np; ++p) {
                 Tile tile{};
@@ -192,16 +198,9 @@ void make_tiles(TaskList& tl, const std::vector<int>* group) {
                 tile.N = k.herm ? 0 : k.N;
                 tile.seg_lo = parts[p].seg_lo; tile.seg_hi = parts[p].seg_hi;
                 tile.k0 = (int32_t)parts[p].k0; tile.k1 = (int32_t)parts[p].k1;
-                tile.split = split; tile.part = p; tile.nparts = np; tile.split_base = (int32_t)(base / 32);
+                tile.split = split; tile.part = (uint16_t)p; tile.nparts = (uint16_t)np; tile.split_base = (int32_t)(base / 32);
                 tile.cost = (int32_t)std::min<int64_t>((int64_t)cnt * std::max<int64_t>(parts[p].k1 - parts[p].k0, 1), 0x7fffffff);
                 tl.tiles.push_back(tile);
-            }
-            col += step;
-            if (k.herm) {
-                while (col > row) col -= ++row;
-            } else {
-                row += col / k.N;
-                col %= k.N;
             }
         }
     }
@@ -419,14 +418,15 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
         s2.tasks.push_back(tk);
         g2.push_back(find_root(pout[k].qi));
     }
-    s1.group = g1;
-    s2.group = g2;
+    p->group[0] = g1;
+    p->group[1] = g2;
     make_tiles(s1, &g1);
     make_tiles(s2, &g2);
     p->scratch = scr;
     p->flops = s1.flops + s2.flops;
     int urc = upload(c, s1);
     if (!urc) urc = upload(c, s2);
+    if (!urc) urc = uploads_done(c, "plan upload");
     if (urc) return urc;
     if (scr > c->scratch_cap) {
         if (c->scratch) dev_free(c, c->scratch, c->scratch_cap * sizeof(cplx));

@@ -21,7 +21,7 @@ int main(int argc, char** argv) {
     int64_t next = 0, partial = 0;
     for (const Tile& x : tl.tiles) {   // one cost but for the last tile's, so they stay in order
         const int64_t o = t.herm ? (int64_t)x.m0 * (x.m0 + 1) / 2 + x.o0 : (int64_t)x.m0 * t.N + x.o0;
-        if (x.m0 < 0 || x.m0 >= t.M || x.o0 < 0 || x.o0 >= (t.herm ? x.m0 + 1 : t.N) || x.cnt < 1 || x.cnt > 256) {
+        if (x.m0 < 0 || x.m0 >= t.M || x.o0 < 0 || x.cnt < 1 || x.cnt > 256 || (outs > kFlatOuts && x.o0 >= (t.herm ? x.m0 + 1 : t.N))) {
             printf("tile out of range: row %d column %d count %d\n", x.m0, x.o0, x.cnt);
             return 1;
         }
