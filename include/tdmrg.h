@@ -159,7 +159,7 @@ int tdmrg_evolve(tdmrg_ctx* ctx, int n_up, int n_dn, const tdmrg_c64* phi_d, int
 
 /* Ground state in sector Q (the ground-state targeting of Sec. II.B, needed at every DMRG step):
  * `restarts` times, nk Lanczos steps started at psi_d (full re-orthogonalisation, FP64), the lowest
- * eigenvector of the tridiagonal (multisection on its Sturm count, a twisted factorisation, FP64) combined
+ * eigenvector of the tridiagonal (multisection on the signs of its leading minors, a twisted factorisation, FP64) combined
  * in place into psi_d, normalised.  psi_d (device, sector Q) is the start vector on entry and the ground
  * state on return; *energy (host, nullable) receives the lowest Ritz value of the last restart.  The
  * call synchronises the stream once at the end.  Errors: EINVAL (nk outside 2..nk_max, restarts < 1),
@@ -173,7 +173,8 @@ int tdmrg_ground_state(tdmrg_ctx* ctx, int n_up, int n_dn, tdmrg_c64* psi_d, int
  * product of the sum pairs blocks of different sources, and source k's operator id becomes 2^20 k + id.
  * The vector of ctx in Qsum is the concatenation of the sources' vectors in their sectors Q_k, in source
  * order: seg_off (host, nsrc + 1, nullable) receives their offsets, Qsum (host, 2, nullable) the common
- * sector.  One H psi of ctx is then one grouped product over all sources (Sec. IV).  Sources keep their
+ * sector.  One H psi of ctx is then one grouped product over all sources (Sec. IV), in either precision with
+ * the bits of every source's own product.  Sources keep their
  * own data (ctx holds copies); their quantum numbers must lie in 0..2047 and their coefficients be
  * static.  Synchronises the streams.  Errors: EINVAL, ESTATE (a source without Hamiltonian), ESECTOR,
  * ENOMEM, ECUDA. */
@@ -255,8 +256,8 @@ int tdmrg_density_eig(tdmrg_ctx* ctx, int side, int ntargets, const int32_t* Q, 
  * 1e-12 lambda_max of the m-th largest are ties, broken by (sector index, eigen index) ascending, so
  * every sector keeps its leading eigenvectors.  kept_d (device, one int per left sector) receives the
  * states kept per sector (all of them when the block has at most m); discarded_d (device, one double,
- * nullable) the sum of the dropped eigenvalues (the truncation error).  Synchronises the stream once to
- * upload the sector tables.  Errors: EINVAL (m < 1, more than 1024 sectors), ESTATE, ECUDA. */
+ * nullable) the sum of the dropped eigenvalues (the truncation error).  The first call on a block uploads its
+ * sector tables and synchronises the stream.  Errors: EINVAL (m < 1, more than 1024 sectors), ESTATE, ECUDA. */
 int tdmrg_truncate(tdmrg_ctx* ctx, const double* evals_d, int m, int32_t* kept_d, double* discarded_d);
 
 /* tdmrg_truncate for either block (evals_d and kept_d over that side's sectors). */

@@ -2,8 +2,9 @@
 //
 // GB300 runs FP64 at about 1 TFLOP/s chip-wide (~7 GFLOP/s per SM), so an FP64 Jacobi on one SM per
 // sector would take milliseconds for the largest sectors.  Instead:
-//   1. seed: a one-sided Jacobi in FP32 on the Cholesky factor of each sector (one CTA per sector, parallel
-//      round-robin ordering of disjoint rotations), giving eigenvectors X0 accurate to about 1e-6;
+//   1. seed: a one-sided Jacobi in FP32 on the Cholesky factor of each sector (parallel round-robin ordering of disjoint
+//      rotations; up to 64 states on one CTA, up to 160 on a cluster of four, above that one CTA with the factor in global
+//      memory), giving eigenvectors X0 accurate to about 1e-6;
 //   2. refine: iterative refinement for Hermitian eigenproblems (Ogita & Aishima, 2018), whose work is
 //      grouped GEMMs spread over every SM (FP64, except the small correction E^H W in FP32):
 //         G = X^H X,  S = X^H (rho X),  lambda_i = Re S_ii / Re G_ii,  R = I - G,
@@ -26,7 +27,7 @@
 //      is a plain or conjugate-transposed GEMM operand;
 //   3. sort each sector's eigenpairs by descending eigenvalue.
 // The sectors run in one group, or in two on two streams: the few with the longest Jacobi seeds (the
-// seed of a sector runs on one SM, so its cost grows with n, not with the total work) seed and refine on
+// seed of a sector runs on one or four SMs, so its cost grows with n, not with the total work) seed and refine on
 // a second stream while the others' seeds and refinement fill the rest of the GPU; a cost model picks the
 // split (long_sectors).
 #include <algorithm>
@@ -357,7 +358,8 @@ __global__ void __launch_bounds__(JT) k_jacobi32(const cplx* __restrict__ src, c
 // V of the sectors beyond kSmemMaxN from their rotation record: V starts as the identity and every
 // recorded rotation J_r acts on columns (p, q) of every row, so rows are independent: CTA (b, y) holds
 // rows 8y .. 8y + 7 of V of big sector b in shared memory and replays all rounds on them, the record
-// staged through shared memory a batch of rounds at a time.  Writes V^H - I like jacobi_store.  Runs after each k_jacobi32 launch; nrec < 0 marks a skipped sector.
+// staged through shared memory a batch of rounds at a time.  Writes V^H - I like jacobi_store.  Runs after each
+// k_jacobi32 launch; nrec < 0 marks a skipped sector.
 __global__ void __launch_bounds__(kReplayThreads) k_jacobi_replay(const float4* __restrict__ grec, const int* __restrict__ nrec,
                                                                   cplx* __restrict__ dst, EigTables tb, int batch) {
     pdl_enter();
@@ -419,12 +421,13 @@ __global__ void __launch_bounds__(kReplayThreads) k_jacobi_replay(const float4* 
 // four pairs of a warp (a warp per pair issued 250 instructions a pair at n = 152, 4 x the columns' own work).  A sector
 // above kSeedClusterN columns is spread over a cluster of four CTAs by rows (a round moves 16 n^2 bytes through shared
 // memory, 2900 cycles on one SM at n = 152).
-// Measured, cycles per round: n = 60 1480 (warp per pair) -> 1130, n = 124 3830 -> 3230 (eight lanes) -> 1940 (cluster),
-// n = 152 5330 -> 4610 -> 2510; the decomposition at L=32 m=400 1041 us (two-sided seed with V by rotation replay) -> 568
-// -> 521, at L=48 m=1000 8.93 ms -> 4.95 -> 4.67 -> 3.99.  Bound by the latency of a pair's chain (load, 3 shuffle levels,
-// rotation, store, barrier: ~640 cycles; the cluster's exchange adds ~700) and, from n ~ 100, by instruction issue.
+// Measured, cycles per round: 1130 at n = 60, 1940 at 124 and 2510 at 152 (on one SM 3230 and 4610).  Bound by the latency of
+// a pair's chain (load, 3 shuffle levels, rotation, store, barrier: ~640 cycles; the cluster's exchange adds ~700) and,
+// from n ~ 100, by instruction issue.
 // Columns are rows of T (T[c][r] = L[r][c], contiguous in r), lanes run over r.  T in shared memory up to n = kSeedSmemN,
-// else in `gwork` (one CTA, a warp per pair).
+// else in `gwork` (one CTA, a warp per pair).  The whole decomposition of one sector, four decades / rank n/3 / 14 decades:
+// 15 / 14 / 42 ms at n = 200 and 250 / 225 / 600 ms at n = 512, with the two-sided Jacobi it replaces 39 / 22 / 67 and
+// 549 / 293 / 881 ms.
 constexpr int ST = 640;                    // threads of the seed CTA: 80 pairs of eight lanes
 constexpr int kSeedSmemN = 160;            // largest sector with T in shared memory (2 * ST / 8 columns, 205 KB)
 __host__ __device__ constexpr int seed_ld(int n) { return (n + 15) / 16 * 16; }
@@ -1054,7 +1057,8 @@ enum { EB_RHO = BUF_EXTRA0, EB_W, EB_AX, EB_S, EB_G, EB_E, EB_WN };
 // Cost model of the split into two groups, in SM cycles: the seed of one sector (about 7.5 sweeps of n - 1 rounds; a
 // round costs ~500 + 12 n cycles, in a cluster ~600 + 14 n) and the refinement of a sector spread over the GPU,
 // 0.4 n^3 (the products alone are ~0.1 n^3; measured over 0.03 ... 1.5: the decomposition at L=48 m=1000 took 5.7 ms up
-// to 0.12 and 4.95 ms from 0.2 on, L=32 m=400 and m=800 changed by 4 %).  It only decides the scheduling.
+// to 0.12 and 4.95 ms from 0.2 on, L=32 m=400 and m=800 changed by 4 %).  It only decides the scheduling; a seed above 160
+// states takes about five times what it gives.
 double jacobi_cost(int n) { return 7.5 * std::max(n - 1, 0) * (n <= kSeedClusterN ? 500.0 + 12.0 * n : 600.0 + 14.0 * n); }
 double refine_cost(int n) { return 0.4 * (double)n * n * n; }
 

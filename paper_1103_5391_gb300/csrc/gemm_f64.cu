@@ -14,9 +14,8 @@
 //   - operands go from global memory (L1 / L2) straight to registers, four k ahead of their use: at 256
 //     cycles per complex multiply-add of a warp the loads are hidden without shared memory or barriers;
 //   - conjugations and the segment factor are applied once per segment on the accumulated sums.
-// Measured (before: 16 x 16 tiles of m8n8k4 MMAs staged through shared memory, each warp one 8 x 8 block over the
-// whole K): rho_L at L=48 m=1000 872 -> 581 us (0.60 GFLOP of lower triangles, 1.04 TFLOP/s), H psi at L=8 m=16
-// 17.7 -> 8.7 us, a Krylov advance at L=16 m=120 (12 steps) 985 -> 526 us.
+// Measured: rho_L at L=48 m=1000 564 us (0.60 GFLOP of lower triangles, 1.07 TFLOP/s), H psi at L=8 m=16 8.3 us; as 16 x 16
+// tiles of m8n8k4 MMAs, each warp one 8 x 8 block over the whole K, 872 and 17.7 us.
 // CTAs that share a K split store partial sums; the last part to arrive (atomic ticket) sums all parts in index
 // order, so results do not depend on scheduling.
 //

@@ -400,9 +400,9 @@ struct tdmrg_ctx {
     int orth_per_sm = 0;           // blocks per SM of the cooperative orthogonalisation (0: the default)
     struct TruncTables { void* d = nullptr; size_t bytes = 0; bool valid = false; int64_t nev = 0; };
     TruncTables trunc[2];          // per side: sector tables of tdmrg_truncate
-    int thin_dim = 12;
+    int thin_dim = 12;             // tensor path: sector products with min(M, N) below this run on FP64 warps
     int real_basis = 0;            // tdmrg_density_matrix forms Re rho_L (targets' real and imaginary parts apart)
-    const tdmrg::cplx* dcoef = nullptr;   // caller's device array of connection coefficients (null: static)             // tensor path: sector products with min(M, N) below this run on FP64 warps
+    const tdmrg::cplx* dcoef = nullptr;   // caller's device array of connection coefficients (null: static)
     int* dstatus = nullptr;        // device word: nonzero when a bounded device wait ran out; 16 tickets follow at +16
     tdmrg::EigWork eig[2];         // per side (rho_L, rho_R)
     void* transient = nullptr;     // task lists and scratch of calls that do not keep a plan (run_transient)

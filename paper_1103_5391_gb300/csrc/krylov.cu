@@ -2,11 +2,11 @@
 // Eq. lanczosevolution2; time targets of Sec. II.B).
 //
 // Lanczos is started from phi itself: v_0 = phi / ||phi||.  Step j: w = H v_j (grouped superblock
-// product), alpha_j = Re <v_j|w>, then two classical Gram-Schmidt passes against v_0..v_j
-// (the first pass also removes the alpha_j v_j and beta_j v_{j-1} components; its dots in FP32, the second
-// pass in FP64 removes what they leave, and alpha_j is the sum of both passes' coefficients),
-// beta_{j+1} = ||w||, v_{j+1} = w / beta_{j+1}, all in one cooperative launch per step with two grid
-// barriers; the recursion stops at n_K vectors or when beta_{j+1} <= tol * max(1, |alpha_j|).  Then the
+// product), then two classical Gram-Schmidt passes: the first removes the alpha_j v_j and beta_j v_{j-1} components (H v_j
+// has none above rounding along the others), its dots in FP32; the second, in FP64 against v_0..v_j, removes what it
+// leaves, a third the rest where that is most of the vector; alpha_j is the sum of the passes' coefficients,
+// beta_{j+1} = ||w||, v_{j+1} = w / beta_{j+1}.  All in one cooperative launch per step, whose blocks exchange partial
+// sums twice; the recursion stops at n_K vectors or when beta_{j+1} <= tol * max(1, |alpha_j|).  Then the
 // coefficients c_x = ||phi|| e^{-i T t_x} e_0 (= ||phi|| [S^dag e^{-i D t_x} S]_{.,0} with T = S^dag D S)
 // are computed on the tridiagonal itself (Taylor series on short substeps, FP64; for equally spaced
 // times by powers of the step exponential) and the targets phi(t_x) = sum_k v_k c_x[k] are formed in
@@ -152,10 +152,9 @@ __global__ void __launch_bounds__(NT) k_init_v0(const cplx* __restrict__ phi, in
 //     value, and readers poll the values themselves.  Against a counter barrier this saves the arrival's round trip
 //     twice.  Slots are cleared a phase later, when every block is known to have read them.
 // Polls are bounded: when one runs out the kernel sets a status bit and finishes.
-// Measured, cycles at j = 8 (D = 5000 / 46,868), before (dots by element, a counter barrier and then the partials, loads
-// where used) -> now: pass A with its loads 3000 / 3800 -> 3500 / 4000, its exchange 6700 / 6000 -> 3700 / 8000, pass B
-// 14200 / 20400 -> 6700 / 14500, its exchange 10300 / 10700 -> 3900 / 6000, pass C 8400 / 13700 -> 4500 / 11500; the launch
-// 23.4 / 26.8 -> 13.6 / 19.9 us on average over a run.  What remains at D = 46,868 is FP64 issue in B and C.
+// Measured, cycles at j = 8 (D = 5000 / 46,868): pass A with its loads 3500 / 4000, its exchange 3700 / 8000, pass B 6700 /
+// 14500, its exchange 3900 / 6000, pass C 4500 / 11500; the launch 13.6 / 19.9 us on average over a run (23.4 / 26.8 with dots
+// split by element, counter barriers and loads where used).  What remains at D = 46,868 is FP64 issue in B and C.
 constexpr int OB = 256;   // threads per block of the fused kernel
 constexpr long kPollLimit = 1L << 24;        // polls of another block's value (a block may wait for an SM of its own)
 constexpr long kBulkLimit = 1L << 20;        // polls of the block's own copies

@@ -495,10 +495,9 @@ __device__ __forceinline__ bool mbar_wait_ws(uint32_t bar, uint32_t parity, vola
 // of one task or of several, so that blocks of a few entries fill their warps; items go to CTAs at plan build, longest
 // first onto the least loaded.  What bounds them is latency (tables and operands, one segment after the other, and 4 FP64
 // instructions of 64 cycles per complex k), so an output whose chain is above kThinChain k-steps (a segment as 4) is
-// shared by up to 2^kThinLog2Parts lanes, over segments first.  Measured, stage 1 of six batched jobs (where the thin
-// products are the longest chain) and L = 32, m = 400 H psi: 8 x 8 blocks of m8n8k4 MMAs (3 x padding) 57 us, 46 us;
-// a warp per task and 32 outputs 60 us, 46 us; outputs packed over tasks 51 us; the epilogue warps joining in 29 us,
-// 47.4 us; the split over lanes 29 us, 46.3 us; the CTA's range passed on in shared memory 29 us, 45.8 us.
+// shared by up to 2^kThinLog2Parts lanes, over segments first.  Measured, stage 1 of six batched jobs, where the thin
+// products are the longest chain: 29 us; as 8 x 8 blocks of m8n8k4 MMAs (3 x padding) 57 us, without packing over tasks
+// 60 us, without the epilogue warps 51 us.
 __device__ __forceinline__ void thin_item(const ThinItem& it, int lane, const OzGemmArgs& oa, const GemmArgs& g) {
     const int W = 32 >> (it.lps + it.lpk);   // outputs of the item; lanes of part p of every output: p W .. p W + W - 1
     const int oi = lane & (W - 1), part = lane / W;
@@ -725,9 +724,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_ozaki_gemm_ws(const __grid_co
             long long acc[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) acc[j] = 0;
-            // the exponents while the products are formed (after them: H psi at L=32 m=400 45.0 instead of 44.4 us): a row's in a register, the columns' in a per-warp row of shared
-            // memory; accumulator columns 2j, 2j + 1 hold Re and Im of output column j: this warp's 16 columns are output
-            // columns 8 part .. 8 part + 7
+            // the exponents while the products are formed (after them: H psi at L=32 m=400 45.0 instead of 44.4 us): a
+            // row's in a register, the columns' in a per-warp row of shared memory; accumulator columns 2j, 2j + 1 hold Re
+            // and Im of output column j: this warp's 16 columns are output columns 8 part .. 8 part + 7
             const int Ei = row_lane && tile.m0 + row < task.M ? oa.expA[task.aexp0 + tile.m0 + row] - 7 * (S + 1) : 0;
             if (lane < 16) {
                 const int j = 8 * part + (lane >> 1);

@@ -120,10 +120,9 @@ int64_t sector_size(const tdmrg_ctx* c, int n_up, int n_dn) {
 // Tiles of the grouped FP64 GEMM.  The K range one warp runs through aims at half the launch's work per FP64 pipe
 // (152 SMs x 4), between 8 and 192: small launches are cut finely so that every pipe has work and no chain is long,
 // but not more finely than that needs, as a CTA's fixed latency (its tables, the first operands, the sums of its
-// shares: ~6000 cycles) is that of ~25 complex k of a warp.  Measured with half / a sixth of the work: ground state
-// L=16 m=200 4.86 / 6.09 ms, eigendecomposition L=32 m=400 458 / 500 us; a floor of 4 or 16 instead of 8 makes a
-// Krylov advance at L=16 m=120 614 or 542 us instead of 527, a cap of 64 instead of 192 rho_L at L=48 m=1000 607 us
-// instead of 581.
+// shares: ~6000 cycles) is that of ~25 complex k of a warp.  Measured: a sixth of the work instead of half makes a ground
+// state at L=16 m=200 25 % slower, a floor of 4 or 16 instead of 8 a Krylov advance at L=16 m=120 17 % or 3 %, a cap of 64
+// instead of 192 rho_L at L=48 m=1000 4 %.
 // With groups (group[t] of task t) the work is that of the task's group alone, so that the sums of a group's outputs do
 // not depend on what else is launched with it.
 // A task's K is divided first among the warps of a CTA (ks = 1, 2, 4, 8 shares, 256 / ks outputs), then over CTAs.
@@ -155,8 +154,8 @@ void make_tiles(TaskList& tl, const std::vector<int>* group) {
         const int area = kTileOut / cks;
         int want = (int)std::min<int64_t>({(shares + cks - 1) / cks, (int64_t)kMaxParts, std::max<int64_t>(ks[t], 1)});
         // sector products: parts of 96 k and a segment at least (a tile's segments may ask for more), so that the partial
-        // sums stay within what the allocation-free product's static array is made for: one part per 96 k.  It costs
-        // nothing: a Krylov advance at L=16 m=120 423 -> 419 us, a drawn one 1160 -> 1129 us, others unchanged.
+        // sums stay within what the allocation-free product's static array is made for: one part per 96 k (a Krylov
+        // advance at L=16 m=120 is 1 % faster for it).
         if (group) want = (int)std::min<int64_t>({(int64_t)want, (ks[t] + 95) / 96, std::max<int64_t>(k.seg_end - k.seg_begin, 1)});
         want = std::max(want, 1);
         // K parts [lo, hi) of the concatenated range, each within kTileSegs segments
@@ -297,9 +296,8 @@ int build_plan(tdmrg_ctx* c, const std::vector<Term>& terms, int qa, int qb, int
     for (size_t k = 0; k < pout.size(); ++k) out_of_q[pout[k].qi] = (int)k;
 
     // left sectors that the terms connect: the superblocks of a direct sum stay apart, and every one gets the K parts (so
-    // the bits) that it has alone; without the groups H psi of the jobs of a batch differed from theirs alone in
-    // the last bit, and with parts by a task's own size instead H psi at L=16 m=200 takes 40 to 49 us instead of 41, the
-    // ground state 4.84 to 5.99 ms instead of 4.87, a Krylov advance at L=16 m=120 427 to 466 us instead of 429
+    // the bits) that it has alone.  Parts by a task's own size would do that too, but are up to 20 % slower (H psi and the
+    // ground state at L=16 m=200) where they are not the same.
     std::vector<int> root(L.dim.size());
     for (size_t k = 0; k < root.size(); ++k) root[k] = (int)k;
     auto find_root = [&](int q) {
